@@ -63,12 +63,15 @@ typedef enum {
 } gsm_kernel_t;
 
 /* Arithmetic of the FFT passes and of the multiplier product.
- *   GSM_FP64   : IEEE double.                  I/O: double.
+ *   GSM_FP64   : block fixed point, 64-bit integers with one exponent per
+ *                transformed line, whose errors are those of IEEE double
+ *                arithmetic or less.           I/O: double.
  *   GSM_FP32   : IEEE single.                  I/O: float.
- *   GSM_FP32X2 : double-float (pairs of floats, about 48 significand bits),
- *                computed on the FP32 pipes.   I/O: double.
+ *   GSM_FP32X2 : computed as GSM_FP64 (at least the 48 bits that pairs of
+ *                floats would give).           I/O: double.
  * In every precision the Gaussian sum, the kernel tensor and the Taylor
- * coefficients are built in FP64 and rounded (FP32) or split (FP32X2) once. */
+ * coefficients are built in FP64 and rounded (FP32) or put into fixed point
+ * once.  An infinity or a NaN in rho makes every element of u NaN. */
 typedef enum {
     GSM_FP64 = 0,
     GSM_FP32 = 1,
@@ -369,15 +372,13 @@ gsm_status_t gsm_fft_lines(int M, int nlines, int sign, gsm_precision_t precisio
  * critical path that must not take the allocator's locks or risk an
  * out-of-memory failure at call time, or a plug-in that is not allowed to own
  * device memory.  gsm_fft_lines_noalloc takes the same arguments and gives the
- * same bits as gsm_fft_lines (the same twiddle table and, in FP64, the same
- * FMA-form stage constants, so the same arithmetic), but keeps those tables in
- * a fixed 384 KiB scratch array that the library declares statically in device
- * memory:
+ * same bits as gsm_fft_lines (the same twiddle table, so the same arithmetic),
+ * but keeps that table in a fixed 128 KiB scratch array that the library
+ * declares statically in device memory:
  *   - it calls no cudaMalloc, cudaFree or other allocating routine;
- *   - the tables of every supported length fit (the largest, M = 8192 in FP64,
- *     take 339968 bytes); a length whose tables would not fit is rejected with
- *     GSM_ERR_UNSUPPORTED_SIZE, as is M > 8192;
- *   - every GPU that loads the library holds the 384 KiB until the process
+ *   - the tables of every supported length fit (the largest, M = 8192, takes
+ *     131072 bytes); M > 8192 is rejected with GSM_ERR_UNSUPPORTED_SIZE;
+ *   - every GPU that loads the library holds the 128 KiB until the process
  *     exits;
  *   - the first call on each device (more exactly, in each CUDA context: again
  *     after cudaDeviceReset) looks up the device address of the scratch, with

@@ -17,14 +17,11 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgsm.so")
-SOURCES = ["gsm_api.cu", "gsm_plan.cu", "gsm_passes.cu", "gsm_conv_rr.cu", "gsm_tc.cu"]
-HEADERS = ["gsm_arith.cuh", "gsm_fft.cuh", "gsm_internal.h"]
+SOURCES = ["gsm_api.cu", "gsm_plan.cu", "gsm_passes.cu", "gsm_fx.cu", "gsm_fx_conv.cu", "gsm_fx_queue2d.cu",
+           "gsm_fx_queue3d.cu", "gsm_conv_rr.cu", "gsm_tc.cu"]
+HEADERS = ["gsm_arith.cuh", "gsm_fft.cuh", "gsm_fx.cuh", "gsm_fx_passes.cuh", "gsm_fx_queue.cuh", "gsm_pass_common.cuh", "gsm_internal.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
-# The pass file instantiates every kernel for three precisions and dominates the build; its
-# device-code optimiser runs on every CPU core.  Not used for the register-resident FP32 kernels,
-# whose x and y passes it made a quarter slower.
-SPLIT = {"gsm_passes.cu": ["--split-compile=0"]}
 
 
 def nvcc() -> str:
@@ -50,7 +47,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         o = os.path.join(BUILD, src.replace(".cu", ".o"))
         objs.append(o)
         if force or _stale(o, [s] + hdrs):
-            jobs.append([nvcc(), *ARCH, *FLAGS, *SPLIT.get(src, []), "-c", s, "-o", o])
+            jobs.append([nvcc(), *ARCH, *FLAGS, "-c", s, "-o", o])
 
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)

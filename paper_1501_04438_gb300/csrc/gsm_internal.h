@@ -50,9 +50,11 @@ struct Plan {
     double *d_g[3] = {nullptr, nullptr, nullptr}; // 1-D factors [q][k] per axis
     double *d_khat = nullptr;                     // sum_q w_q G_k^q, octant, FP64
     double *d_mult64 = nullptr;                   // full multiplier, FP64, octant
-    void *d_mult = nullptr;                       // multiplier in the pass precision
-    void *d_tw[3] = {nullptr, nullptr, nullptr};  // per axis: twiddles, then (FP64) the FMA-form
-                                                  // constants of the forward schedule
+    void *d_mult = nullptr;                       // multiplier in the pass precision (FP32: float; fixed
+                                                  // point: factors of its rows' 2^exponent)
+    int *d_mrow = nullptr;                        // those exponents, at the end of the table's allocation
+    void *d_tw[3] = {nullptr, nullptr, nullptr};  // per axis: twiddles (fixed point: in the stage order of
+                                                  // the forward schedule)
     void *d_twi[3] = {nullptr, nullptr, nullptr}; // the same for the inverse schedule (may alias d_tw)
     void *d_work1 = nullptr, *d_work2 = nullptr;  // FFT workspace
     size_t work1_bytes = 0, work2_bytes = 0;
@@ -125,6 +127,38 @@ struct StoredPlanData {
 // it instead of being computed
 gsm_status_t build_plan_data(Plan *p, cudaStream_t st, const StoredPlanData *stored = nullptr);
 
+// Fixed point: exponents of the transformed lines in the workspace
+// (gsm_fx_passes.cuh).
+struct FxExps {
+    int *xf, *yf, *cv, *yi;
+    int xf_par;   // distance of the two parities' rows of xf (0: one row serves both)
+};
+// One fixed-point pass: nz slabs from the pointers given on.
+struct FxCall {
+    const Plan *p;
+    FxExps ex;
+    const double *rho;
+    double *u;
+    void *W1, *W2;
+    int nz;
+    cudaStream_t st;
+};
+// Launch of a pass, of the split 2D passes, of the FFT hook; shared-memory
+// limits of their kernels; twiddle tables (gsm_fx.cu, gsm_fx_conv.cu).
+void fx_launch_xy(const FxCall &c, int pass, const PassCfg &cfg);
+void fx_launch_conv(const FxCall &c, const PassCfg &cfg);
+void fx_launch_split(const FxCall &c, bool conv);
+cudaError_t fx_launch_hook(const PassCfg &c, int nlines, int sign, const Sched &sc, const double *in, double *out,
+                           const void *tw, cudaStream_t st);
+cudaError_t fx_raise_smem(const Plan *p, int pass, const PassCfg &c);
+cudaError_t fx_raise_conv_smem(const PassCfg &c);
+cudaError_t fx_raise_split_smem(bool conv, size_t smem);
+size_t fx_table_bytes(int M, int plain);
+void launch_fx_twiddles(const Sched &sc, int plain, int plain_m, void *out, cudaStream_t st);
+// largest CTA of the kernels with emax elements per thread
+constexpr int fx_threads(int emax) { return emax == 8 ? 256 : 512; }
+constexpr int kSplitThreads = 256;   // of a half line, at most 4096 values, 16 per thread
+
 // passes (gsm_passes.cu)
 gsm_status_t configure_passes(Plan *p);
 gsm_status_t launch_apply(const Plan *p, const void *rho, void *u, cudaStream_t st);
@@ -176,6 +210,9 @@ gsm_status_t launch_dft32_tc(int nvec, int sign, const double *in, double *out, 
 // (frees the axis's previous tables unless another axis shares them)
 gsm_status_t make_twiddles(Plan *p, int axis, cudaStream_t st);
 gsm_status_t make_pass_multiplier(Plan *p, cudaStream_t st);
+// fixed point: `rows` rows of `len` doubles at `table` to factors, in place, their
+// exponents after them
+gsm_status_t make_mult_rows(Plan *p, void *table, int len, size_t rows, cudaStream_t st);
 // default radix schedule of length M: radices 8, 4, 2, 5, 3 in that order
 bool make_sched(int M, Sched *s);
 constexpr int kSplitMinM = 4096;

@@ -15,89 +15,15 @@
 // in shared memory; the other side of each pass moves chunks of 2nl (xf, xi)
 // or nl (yf, yi) consecutive complex values.  In 2D: xf (one slab), conv on
 // W[kx][y] along y, xi.
-#include <stdio.h>
-#include <stdlib.h>
-#include <string.h>
-
-#include <algorithm>
-#include <atomic>
-#include <mutex>
-#include <new>
-#include <string>
-#include <vector>
-#include <type_traits>
-
-#include <cooperative_groups.h>
-#include <cuda.h>
-
-#include "gsm_internal.h"
+#include "gsm_pass_common.cuh"
 
 namespace gsm {
-
 namespace {
-
-constexpr int kMaxThreads = 512;   // CTA size cap: leaves 128 registers per thread
-
-template <class Pol>
-using S_t = typename Pol::scplx;
-
-// Read of workspace data.  CG = true (the batch queue kernel, in which the
-// workspace is written and read again by other CTAs of the same launch): the
-// load bypasses L1 and the read-only path (ld.global.cg), so it sees what
-// other CTAs stored before they signalled completion.
-template <bool CG, class T>
-__device__ __forceinline__ T ldw(const T *p)
-{
-    if constexpr (CG) return __ldcg(p);
-    else return *p;
-}
-
-// Copies `count` elements into shared memory with U global loads in flight
-// per thread (all U loads are issued before the first store waits for its
-// data): for i = t, t + T, ... < count, dst(i, src(i)).
-template <int U, class Val, class Src, class Dst>
-__device__ __forceinline__ void gather_smem(int t, int T, int count, Src src, Dst dst)
-{
-    for (int i0 = t; i0 < count; i0 += U * T) {
-        Val v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (i0 + u * T < count) v[u] = src(i0 + u * T);
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (i0 + u * T < count) dst(i0 + u * T, v[u]);
-    }
-}
-// Loads in flight per thread when the y passes and the x inverse gather their
-// input: four in double-float, whose y and x inverse passes wait on their
-// gathered rows (measured 0.61 -> 0.53 ms for the y inverse at 256^3); one
-// in FP64 and FP32, where more did not pay.
-template <class Pol>
-constexpr int kGatherDepth = std::is_same<Pol, DF64>::value ? 4 : 1;
-
-// FP64 twiddle tables hold, after the M twiddles w^m, the constants of the
-// FMA-form radix-8 stages (fft_stage8_fma); the other precisions have none.
-template <class Pol>
-__device__ __forceinline__ const double *g8_table(const typename Pol::tw_t *tw, int M)
-{
-    if constexpr (std::is_same<Pol, F64>::value) return reinterpret_cast<const double *>(tw + M);
-    else return nullptr;
-}
 
 // Launch shape (see PassCfg): a CTA holds nl lines; line l is transformed by
 // group l of gthr threads (blockDim.x = nl * gthr).  Loads and stores that
 // touch one line are done by its group; the transposed side of a pass is
 // done by the whole CTA, with one __syncthreads between it and the FFTs.
-
-// The double-float x and y kernels with 8 elements per thread are compiled
-// for four resident CTAs of up to 256 threads per SM (a 64-register bound):
-// more warps to hide their global-memory and barrier waits (measured at
-// 256^3: x forward 0.27 -> 0.25 ms, y inverse 0.53 -> 0.49, x inverse 0.29 ->
-// 0.25).  Their launch shapes keep to 256 threads.
-template <class Pol>
-constexpr int xy_max_threads(int emax) { return (std::is_same<Pol, DF64>::value && emax == 8) ? 256 : kMaxThreads; }
-template <class Pol>
-constexpr int xy_min_ctas(int emax) { return (std::is_same<Pol, DF64>::value && emax == 8) ? 4 : 1; }
 
 // ------------------------------------------------------------------ pass xf
 // Each pass is a __device__ body taking its tile (bx, by) explicitly, so that
@@ -117,8 +43,8 @@ __device__ __forceinline__ void body_xf(const typename Pol::io_t *__restrict__ r
     const int y0 = bx * 2 * nl;
     const int ya = y0 + 2 * l;
     const typename Pol::io_t *slab = rho + (size_t)z * ny * nx;
-    // x >= nx is zero padding: written only when the first stage reads it
-    for (int x = g.t; x < (Pol::kPrune ? nx : M); x += g.T) {
+    // x >= nx is zero padding
+    for (int x = g.t; x < M; x += g.T) {
         R a = Pol::zero(), b = Pol::zero();
         if (x < nx) {
             if (ya < ny) a = Pol::from_io(slab[(size_t)ya * nx + x]);
@@ -127,7 +53,7 @@ __device__ __forceinline__ void body_xf(const typename Pol::io_t *__restrict__ r
         s[pidx<Pol>(x)] = Pol::st(cx<R>{a, b});
     }
     group_sync(g);
-    fft_line<Pol, true, EMAX, Pol::kPrune, false>(s, sc, tw, g, g8_table<Pol>(tw, M));
+    fft_line<Pol, true, EMAX>(s, sc, tw, g);
     __syncthreads();
     // Z = A + iB with A, B the transforms of the two real rows:
     // 2A[k] = Z[k] + conj Z[-k], 2B[k] = -i (Z[k] - conj Z[-k]); the factor 2
@@ -145,7 +71,7 @@ __device__ __forceinline__ void body_xf(const typename Pol::io_t *__restrict__ r
 }
 
 template <class Pol, int EMAX>
-__global__ void __launch_bounds__(xy_max_threads<Pol>(EMAX), xy_min_ctas<Pol>(EMAX))
+__global__ void __launch_bounds__(kMaxThreads)
     k_xf(const typename Pol::io_t *__restrict__ rho, S_t<Pol> *__restrict__ W1, int nx, int ny, int hx,
          Sched sc, int nl, int gthr, const typename Pol::tw_t *__restrict__ tw)
 {
@@ -169,8 +95,8 @@ __device__ __forceinline__ void body_yf(const S_t<Pol> *__restrict__ W1, S_t<Pol
     const int z0 = bx * nl;
     const int z = z0 + l;
     const S_t<Pol> *in = W1 + ((size_t)z * hx + kx) * ny;
-    gather_smem<kGatherDepth<Pol>, S_t<Pol>>(   // y >= ny: zero padding
-        g.t, g.T, Pol::kPrune ? ny : M,
+    gather_smem<1, S_t<Pol>>(   // y >= ny: zero padding
+        g.t, g.T, M,
         [&](int y) {
             S_t<Pol> v = Pol::st(cx<R>{Pol::zero(), Pol::zero()});
             if (y < ny && z < nz) v = ldw<CG>(in + y);
@@ -178,7 +104,7 @@ __device__ __forceinline__ void body_yf(const S_t<Pol> *__restrict__ W1, S_t<Pol
         },
         [&](int y, const S_t<Pol> &v) { s[pidx<Pol>(y)] = v; });
     group_sync(g);
-    fft_line<Pol, true, EMAX, Pol::kPrune, false>(s, sc, tw, g, g8_table<Pol>(tw, M));
+    fft_line<Pol, true, EMAX>(s, sc, tw, g);
     __syncthreads();
     const S_t<Pol> *s0 = reinterpret_cast<const S_t<Pol> *>(smem_raw);
     S_t<Pol> *out = W2 + (size_t)kx * M * nz;
@@ -190,7 +116,7 @@ __device__ __forceinline__ void body_yf(const S_t<Pol> *__restrict__ W1, S_t<Pol
 }
 
 template <class Pol, int EMAX>
-__global__ void __launch_bounds__(xy_max_threads<Pol>(EMAX), xy_min_ctas<Pol>(EMAX))
+__global__ void __launch_bounds__(kMaxThreads)
     k_yf(const S_t<Pol> *__restrict__ W1, S_t<Pol> *__restrict__ W2, int ny, int nz, int hx, Sched sc,
          int nl, int gthr, const typename Pol::tw_t *__restrict__ tw)
 {
@@ -220,7 +146,7 @@ __device__ __forceinline__ void body_conv(S_t<Pol> *__restrict__ W, const typena
     const int line = bx * nl + l;
     if (line >= nlines) return;   // the whole group leaves; no CTA barrier follows
     S_t<Pol> *w = W + (size_t)line * n;
-    for (int z = g.t; z < (Pol::kPruneConv ? n : M); z += g.T) {   // z >= n: zero padding
+    for (int z = g.t; z < M; z += g.T) {   // z >= n: zero padding
         S_t<Pol> v = Pol::st(cx<R>{Pol::zero(), Pol::zero()});
         if (z < n) v = ldw<CG>(w + z);
         s[pidx<Pol>(z)] = v;
@@ -238,41 +164,31 @@ __device__ __forceinline__ void body_conv(S_t<Pol> *__restrict__ W, const typena
         mrow = mult + (size_t)line * (n + 1);
     }
     auto mult_of = [&](int k) -> R { return Pol::mult(mrow[full ? k : min(k, M - k)]); };
-    const double *gt = g8_table<Pol>(tw, M), *gti = g8_table<Pol>(twi, M);
     const int fr = fused_radix(sc, sci);
     if (fr != 0) {
         // forward up to its last stage; last forward stage, multiplication and
         // first inverse stage in registers; the rest of the inverse
-        fft_line<Pol, true, EMAX, Pol::kPruneConv, false>(s, sc, tw, g, gt, 0, sc.nst - 1);
-        if (fr == 8) fft_fused_mid<Pol, 8, (EMAX + 7) / 8>(s, sc, tw, g, gt, mult_of);
-        else if (fr == 4) fft_fused_mid<Pol, 4, (EMAX + 3) / 4>(s, sc, tw, g, gt, mult_of);
-        else if (fr == 2) fft_fused_mid<Pol, 2, (EMAX + 1) / 2>(s, sc, tw, g, gt, mult_of);
-        else if (fr == 5) fft_fused_mid<Pol, 5, (EMAX + 4) / 5>(s, sc, tw, g, gt, mult_of);
-        else fft_fused_mid<Pol, 3, (EMAX + 2) / 3>(s, sc, tw, g, gt, mult_of);
-        fft_line<Pol, false, EMAX, false, Pol::kPruneConv>(s, sci, twi, g, gti, 1);
+        fft_line<Pol, true, EMAX>(s, sc, tw, g, 0, sc.nst - 1);
+        if (fr == 8) fft_fused_mid<Pol, 8, (EMAX + 7) / 8>(s, sc, tw, g, mult_of);
+        else if (fr == 4) fft_fused_mid<Pol, 4, (EMAX + 3) / 4>(s, sc, tw, g, mult_of);
+        else if (fr == 2) fft_fused_mid<Pol, 2, (EMAX + 1) / 2>(s, sc, tw, g, mult_of);
+        else if (fr == 5) fft_fused_mid<Pol, 5, (EMAX + 4) / 5>(s, sc, tw, g, mult_of);
+        else fft_fused_mid<Pol, 3, (EMAX + 2) / 3>(s, sc, tw, g, mult_of);
+        fft_line<Pol, false, EMAX>(s, sci, twi, g, 1);
     } else {
-        fft_line<Pol, true, EMAX, Pol::kPruneConv, false>(s, sc, tw, g, gt);
+        fft_line<Pol, true, EMAX>(s, sc, tw, g);
         for (int k = g.t; k < M; k += g.T) {
             const int p = pidx<Pol>(k);
             s[p] = Pol::st(cscale(Pol::ld(s[p]), mult_of(k)));
         }
         group_sync(g);
-        fft_line<Pol, false, EMAX, false, Pol::kPruneConv>(s, sci, twi, g, gti);
+        fft_line<Pol, false, EMAX>(s, sci, twi, g);
     }
     for (int z = g.t; z < n; z += g.T) w[z] = s[pidx<Pol>(z)];
 }
 
-// The double-float conv kernel with 8 elements per thread is compiled for
-// three resident CTAs of up to 256 threads per SM (an 85-register bound):
-// more warps to hide its stalls than at its natural 108 registers (measured
-// 1.54 -> 1.50 ms at 256^3).  Its launch shapes keep to 256 threads.
-template <class Pol>
-constexpr int conv_max_threads(int emax) { return (std::is_same<Pol, DF64>::value && emax == 8) ? 256 : kMaxThreads; }
-template <class Pol>
-constexpr int conv_min_ctas(int emax) { return (std::is_same<Pol, DF64>::value && emax == 8) ? 3 : 1; }
-
 template <class Pol, int EMAX>
-__global__ void __launch_bounds__(conv_max_threads<Pol>(EMAX), conv_min_ctas<Pol>(EMAX))
+__global__ void __launch_bounds__(kMaxThreads)
     k_conv(S_t<Pol> *__restrict__ W, const typename Pol::mult_t *__restrict__ mult,
                                                       int nlines, int n, int is3d, int My, int ny1, Sched sc,
                                                       Sched sci, int nl, int gthr,
@@ -299,7 +215,7 @@ __device__ __forceinline__ void body_yi(const S_t<Pol> *__restrict__ W2, S_t<Pol
     const int kx = by;
     const int z0 = bx * nl;
     const S_t<Pol> *in = W2 + (size_t)kx * M * nz;
-    gather_smem<kGatherDepth<Pol>, S_t<Pol>>(
+    gather_smem<1, S_t<Pol>>(
         threadIdx.x, blockDim.x, M * nl,
         [&](int i) {
             const int ky = i / nl, ll = i - ky * nl;
@@ -313,7 +229,7 @@ __device__ __forceinline__ void body_yi(const S_t<Pol> *__restrict__ W2, S_t<Pol
         });
     __syncthreads();
     const int z = z0 + l;
-    fft_line<Pol, false, EMAX, false, Pol::kPrune>(s, sc, tw, g, g8_table<Pol>(tw, M));
+    fft_line<Pol, false, EMAX>(s, sc, tw, g);
     if (z < nz) {
         S_t<Pol> *out = W1 + ((size_t)z * hx + kx) * ny;
         for (int y = g.t; y < ny; y += g.T) out[y] = s[pidx<Pol>(y)];
@@ -321,7 +237,7 @@ __device__ __forceinline__ void body_yi(const S_t<Pol> *__restrict__ W2, S_t<Pol
 }
 
 template <class Pol, int EMAX>
-__global__ void __launch_bounds__(xy_max_threads<Pol>(EMAX), xy_min_ctas<Pol>(EMAX))
+__global__ void __launch_bounds__(kMaxThreads)
     k_yi(const S_t<Pol> *__restrict__ W2, S_t<Pol> *__restrict__ W1, int ny, int nz, int hx, Sched sc,
          int nl, int gthr, const typename Pol::tw_t *__restrict__ tw)
 {
@@ -350,7 +266,7 @@ __device__ __forceinline__ void body_xi(const S_t<Pol> *__restrict__ W1, typenam
     struct AB {
         S_t<Pol> a, b;
     };
-    gather_smem<kGatherDepth<Pol>, AB>(
+    gather_smem<1, AB>(
         threadIdx.x, blockDim.x, hx * nl,
         [&](int i) {
             const int k = i / nl, ll = i - k * nl;
@@ -371,7 +287,7 @@ __device__ __forceinline__ void body_xi(const S_t<Pol> *__restrict__ W1, typenam
             if (k > 0 && k < nx) s0[ll * LS + pidx<Pol>(M - k)] = Pol::st(cadd(cconj(A), cmul_posi(cconj(B))));
         });
     __syncthreads();
-    fft_line<Pol, false, EMAX, false, Pol::kPrune>(s, sc, tw, g, g8_table<Pol>(tw, M));
+    fft_line<Pol, false, EMAX>(s, sc, tw, g);
     const int ya = y0 + 2 * l;
     typename Pol::io_t *slab = u + (size_t)z * ny * nx;
     for (int x = g.t; x < nx; x += g.T) {
@@ -382,7 +298,7 @@ __device__ __forceinline__ void body_xi(const S_t<Pol> *__restrict__ W1, typenam
 }
 
 template <class Pol, int EMAX>
-__global__ void __launch_bounds__(xy_max_threads<Pol>(EMAX), xy_min_ctas<Pol>(EMAX))
+__global__ void __launch_bounds__(kMaxThreads)
     k_xi(const S_t<Pol> *__restrict__ W1, typename Pol::io_t *__restrict__ u, int nx, int ny, int hx,
          Sched sc, int nl, int gthr, const typename Pol::tw_t *__restrict__ tw)
 {
@@ -391,33 +307,13 @@ __global__ void __launch_bounds__(xy_max_threads<Pol>(EMAX), xy_min_ctas<Pol>(EM
 }
 
 // ------------------------------------------------------------------ pass conv, long 2D lines
-// A conv line of padded length M = 2 Mh holds Mh values x[0..Mh) and zeros.
-// Its even and odd frequencies are then two transforms of length Mh:
-//   X[2k] = FFT_Mh(x)[k],   X[2k + 1] = FFT_Mh(x w_M^n)[k],
-// and the cropped inverse (outputs n < Mh) is
-//   u[n] = IFFT_Mh(E)[n] + w_M^(-n) IFFT_Mh(O)[n],
-// E, O the multiplied even and odd frequencies.  A cluster of two CTAs takes
-// one line: rank 0 the even half, rank 1 the odd half (a line of Mh values
-// each, half the shared memory of the whole line), then each adds its half of
-// the outputs to the other CTA's through distributed shared memory.  Two CTAs
-// per SM work on different lines, so one line's barrier-separated phases
-// overlap another's (one CTA per SM held a whole line of 8192 and left the
-// FP64 pipe idle during its shared-memory phases).  Schedules, tables:
-// length Mh (sched_hf, sched_hi, twh, twhi); twM: the M twiddles w_M^m.
-// A half line (at most 4096 values) takes at most 256 threads.  Three CTAs per
-// SM in FP64 and double-float (an 80-register cap: their butterfly arrays
-// partly spill, to L1) overlap the barrier-separated stages better than two:
-// measured 4.17 -> 4.16 ms (FP64) and 1.41 -> 1.34 ms (FP32x2) for the conv at
-// 4096^2.  FP32 keeps the engine's usual bound (a 256-thread bound made its
-// conv slower, 0.50 -> 0.53 ms, with or without the three CTAs).
-constexpr int kSplitThreads = 256;
-template <class Pol>
-constexpr int kSplitBoundThreads = std::is_same<Pol, F32>::value ? kMaxThreads : kSplitThreads;
-template <class Pol>
-constexpr int kSplitCtasPerSm = std::is_same<Pol, F32>::value ? 1 : 3;
-
+// The FP32 form of the split conv: see k_fx_conv_split (gsm_fx_passes.cuh) for
+// the method.  rank 0 takes the even, rank 1 the odd frequencies; schedules and
+// tables of length Mh (sched_hf, sched_hi, twh, twhi); twM: the M twiddles
+// w_M^m.  The kernels keep the engine's usual bound (a 256-thread bound made
+// the conv slower, 0.50 -> 0.53 ms at 4096^2).
 template <class Pol, int EMAX>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSplitBoundThreads<Pol>, kSplitCtasPerSm<Pol>)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kMaxThreads)
     k_conv_split(S_t<Pol> *__restrict__ W, const typename Pol::mult_t *__restrict__ mult, int nlines, int ny1,
                  Sched sc, Sched sci, const typename Pol::tw_t *__restrict__ tw,
                  const typename Pol::tw_t *__restrict__ twi, const typename Pol::tw_t *__restrict__ twM, int full)
@@ -446,24 +342,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSplitBoundThreads<P
             const int k = 2 * kk + rank;
             return Pol::mult(mrow[full ? k : min(k, M - k)]);
         };
-        const double *gt = g8_table<Pol>(tw, Mh), *gti = g8_table<Pol>(twi, Mh);
         const int fr = fused_radix(sc, sci);
         if (fr != 0) {
-            fft_line<Pol, true, EMAX>(s, sc, tw, g, gt, 0, sc.nst - 1);
-            if (fr == 8) fft_fused_mid<Pol, 8, (EMAX + 7) / 8>(s, sc, tw, g, gt, mult_of);
-            else if (fr == 4) fft_fused_mid<Pol, 4, (EMAX + 3) / 4>(s, sc, tw, g, gt, mult_of);
-            else if (fr == 2) fft_fused_mid<Pol, 2, (EMAX + 1) / 2>(s, sc, tw, g, gt, mult_of);
-            else if (fr == 5) fft_fused_mid<Pol, 5, (EMAX + 4) / 5>(s, sc, tw, g, gt, mult_of);
-            else fft_fused_mid<Pol, 3, (EMAX + 2) / 3>(s, sc, tw, g, gt, mult_of);
-            fft_line<Pol, false, EMAX>(s, sci, twi, g, gti, 1);
+            fft_line<Pol, true, EMAX>(s, sc, tw, g, 0, sc.nst - 1);
+            if (fr == 8) fft_fused_mid<Pol, 8, (EMAX + 7) / 8>(s, sc, tw, g, mult_of);
+            else if (fr == 4) fft_fused_mid<Pol, 4, (EMAX + 3) / 4>(s, sc, tw, g, mult_of);
+            else if (fr == 2) fft_fused_mid<Pol, 2, (EMAX + 1) / 2>(s, sc, tw, g, mult_of);
+            else if (fr == 5) fft_fused_mid<Pol, 5, (EMAX + 4) / 5>(s, sc, tw, g, mult_of);
+            else fft_fused_mid<Pol, 3, (EMAX + 2) / 3>(s, sc, tw, g, mult_of);
+            fft_line<Pol, false, EMAX>(s, sci, twi, g, 1);
         } else {
-            fft_line<Pol, true, EMAX>(s, sc, tw, g, gt);
+            fft_line<Pol, true, EMAX>(s, sc, tw, g);
             for (int k = g.t; k < Mh; k += g.T) {
                 const int p = pidx<Pol>(k);
                 s[p] = Pol::st(cscale(Pol::ld(s[p]), mult_of(k)));
             }
             group_sync(g);
-            fft_line<Pol, false, EMAX>(s, sci, twi, g, gti);
+            fft_line<Pol, false, EMAX>(s, sci, twi, g);
         }
         if (rank) {
             for (int i = g.t; i < Mh; i += g.T) {
@@ -485,21 +380,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSplitBoundThreads<P
 }
 
 // ------------------------------------------------------------------ x forward, long 2D lines
-// An x line of padded length M = 2 Mh (two real rows as one complex line)
-// holds Mh = nx values and zeros, so, as for the split conv, its even and odd
-// frequencies are two transforms of length Mh, of x and of x w_M^n.  The
-// forward needs no exchange: the Hermitian split pairs Z[k] with Z[M - k],
-// which has the parity of k, so each CTA of a pair (rank = blockIdx.x & 1)
-// transforms its half and writes the frequencies k = 2 k' + rank itself.
-// Two lines of Mh per SM overlap each other's barrier-separated phases, where
-// one line of 2 Mh per CTA filled an SM alone.  (The x inverse stays one line
-// per CTA: split the same way, with the halves summed through distributed
-// shared memory as in the conv, it was no faster, 1.19 -> 1.21 ms in FP64 at
-// 4096^2; split by output parity, each CTA reading the whole half spectrum and
-// writing every other output, it was slower, 1.19 -> 1.27 ms.)  sc: length
-// Mh; tw: its tables; twM: the M twiddles w_M^m.
+// The FP32 form of the split x forward (k_fx_xf_split): each CTA of a pair
+// transforms one parity of the frequencies and writes it.  The x inverse stays
+// one line per CTA: split by output parity, each CTA reads the whole half
+// spectrum and writes every other output, which was slower (4096^2).
+// sc: length Mh; tw: its tables; twM: the M twiddles w_M^m.
 template <class Pol, int EMAX>
-__global__ void __launch_bounds__(kSplitBoundThreads<Pol>, kSplitCtasPerSm<Pol>)
+__global__ void __launch_bounds__(kMaxThreads)
     k_xf_split(const typename Pol::io_t *__restrict__ rho, S_t<Pol> *__restrict__ W1, int nx, int ny, int hx,
                Sched sc, const typename Pol::tw_t *__restrict__ tw, const typename Pol::tw_t *__restrict__ twM)
 {
@@ -518,7 +405,7 @@ __global__ void __launch_bounds__(kSplitBoundThreads<Pol>, kSplitCtasPerSm<Pol>)
         s[pidx<Pol>(x)] = Pol::st(v);
     }
     group_sync(g);
-    fft_line<Pol, true, EMAX>(s, sc, tw, g, g8_table<Pol>(tw, Mh));
+    fft_line<Pol, true, EMAX>(s, sc, tw, g);
     // frequency k = 2 k' + rank sits at k' of this half; M - k at (Mh - k' - rank) mod Mh
     const int nk = rank ? nx / 2 : nx / 2 + 1;   // k = 0 .. nx of this parity (nx is even)
     for (int kp = threadIdx.x; kp < nk; kp += blockDim.x) {
@@ -536,7 +423,7 @@ __global__ void __launch_bounds__(kSplitBoundThreads<Pol>, kSplitCtasPerSm<Pol>)
 template <class Pol, bool FWD, int EMAX>
 __global__ void __launch_bounds__(kMaxThreads) k_fft_hook(const double2 *__restrict__ in, double2 *__restrict__ out,
                                                           int nlines, Sched sc, int nl, int gthr,
-                                                          const typename Pol::tw_t *__restrict__ tw, int use_g8)
+                                                          const typename Pol::tw_t *__restrict__ tw)
 {
     using R = typename Pol::real;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -551,130 +438,16 @@ __global__ void __launch_bounds__(kMaxThreads) k_fft_hook(const double2 *__restr
         s[pidx<Pol>(k)] = Pol::st(cx<R>{Pol::from_io((typename Pol::io_t)v.x), Pol::from_io((typename Pol::io_t)v.y)});
     }
     group_sync(g);
-    fft_line<Pol, FWD, EMAX>(s, sc, tw, g, use_g8 ? g8_table<Pol>(tw, M) : nullptr);
+    fft_line<Pol, FWD, EMAX>(s, sc, tw, g);
     for (int k = g.t; k < M; k += g.T) {
         const cx<R> c = Pol::ld(s[pidx<Pol>(k)]);
         out[(size_t)line * M + k] = make_double2((double)Pol::to_io(c.re), (double)Pol::to_io(c.im));
     }
 }
 
-// ------------------------------------------------------------------ batch: one launch, a device work queue
-// One launch applies up to kBatchMax plans of different sizes (one precision,
-// one dimension).  The work is a queue of items (pass, instance, tile), a
-// tile being one CTA's share of that instance's pass grid, in pass-major
-// order: every item of pass p comes before every item of pass p + 1.  The
-// launch has one CTA per item.  When a CTA starts, its thread 0 takes a ticket
-// from an atomic counter (so items go to CTAs in the order the CTAs start,
-// whatever their block index), waits until the instance's previous pass is
-// complete (a counter of finished tiles per instance and pass), the CTA runs
-// the tile with the same pass bodies as the single-plan kernels, and counts it
-// as finished.  Each item's dependencies were taken earlier, by CTAs that are
-// already resident and whose own dependencies were taken earlier still, so
-// the waits always end, however many CTAs are resident.  Passes of different
-// instances overlap and no launch boundary drains the GPU between passes.
-// Each wait is bounded all the same: when it runs out the CTA records
-// GSM_ERR_TIMEOUT in the status word and raises the abort flag, and every
-// later CTA returns at once.  Every line is done by one warp holding up to 16
-// elements per thread (M <= 512), nl lines per CTA, so one CTA shape serves
-// all sizes and passes.  (A loop over items inside long-lived CTAs was tried
-// first: with the pass bodies inside a loop the compiler no longer kept their
-// butterfly arrays in registers, 3 to 13 KB of stack per thread.)
-constexpr int kBatchMax = 48;
-constexpr int kBatchEmax = 16;
-constexpr int kBatchMaxM = 32 * kBatchEmax;
-constexpr int kBatchPasses = 5;
-
-struct InstDesc {
-    const void *rho;
-    void *u;
-    void *W1, *W2;
-    const void *mult;
-    const void *tw[3], *twi[3];   // forward and inverse tables per axis
-    int n[3], M[3];
-    Sched sc[3], sci[3];          // forward and inverse schedules per axis
-    int gx[kBatchPasses];   // x extent of each pass's tile grid
-    int full;               // multiplier over the whole half spectrum
-};
-
-// Queue state of one launch in device memory, zeroed before the launch: the
-// next item, the status word (0 or GSM_ERR_TIMEOUT), the abort flag, one
-// unused word, then the finished-tile counter of each (instance, pass).
-constexpr int kStateHeader = 4;
-constexpr int kStateWords = kStateHeader + kBatchMax * kBatchPasses;
-
-struct QueueArgs {
-    int count, d, nl, npass;
-    int total;                                  // items in the queue
-    int start[kBatchPasses + 1];                // first item of each pass
-    int tiles[kBatchPasses][kBatchMax + 1];     // within a pass: first tile of each instance
-    unsigned *state;                            // kStateWords words
-    unsigned long long wait_ns;                 // bound of every wait
-    int hold;                                   // test hook: this instance's first pass never
-                                                // counts as complete (-1: none)
-    InstDesc inst[kBatchMax];
-};
-
-__device__ __forceinline__ unsigned long long global_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned *p)
-{
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ unsigned ld_relaxed_gpu(const unsigned *p)
-{
-    unsigned v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Thread 0 of the CTA: take the next item and wait for its dependency.
-// Returns false when the queue is empty, the batch was aborted or the wait ran
-// out; otherwise the item's pass, instance and tile.
-__device__ __forceinline__ bool take_item(const QueueArgs &a, int *pass, int *inst, int *tile)
-{
-    unsigned *next = a.state, *status = a.state + 1, *abort_flag = a.state + 2;
-    const unsigned *done = a.state + kStateHeader;
-    if (ld_relaxed_gpu(abort_flag) != 0) return false;
-    const int item = (int)atomicAdd(next, 1u);
-    if (item >= a.total) return false;
-    int p = 0;
-    while (item >= a.start[p + 1]) ++p;
-    const int r = item - a.start[p];
-    int i = 0;
-    while (r >= a.tiles[p][i + 1]) ++i;
-    *pass = p;
-    *inst = i;
-    *tile = r - a.tiles[p][i];
-    if (p == 0) return true;
-    const unsigned need = (unsigned)(a.tiles[p - 1][i + 1] - a.tiles[p - 1][i]) + (p == 1 && i == a.hold ? 1u : 0u);
-    const unsigned *cnt = done + i * kBatchPasses + (p - 1);
-    if (ld_acquire_gpu(cnt) >= need) return true;
-    const unsigned long long t0 = global_ns();
-    unsigned sleep_ns = 32;
-    while (ld_acquire_gpu(cnt) < need) {
-        if (ld_relaxed_gpu(abort_flag) != 0) return false;
-        if (global_ns() - t0 > a.wait_ns) {
-            atomicExch(status, (unsigned)GSM_ERR_TIMEOUT);
-            atomicExch(abort_flag, 1u);
-            return false;
-        }
-        __nanosleep(sleep_ns);
-        if (sleep_ns < 1024) sleep_ns *= 2;
-    }
-    return true;
-}
-
 // One tile of pass PASS of one instance.
 template <class Pol, int D, int PASS>
-__device__ __forceinline__ void queue_tile(const InstDesc &d, int nl, int t, unsigned char *smem_raw)
+__device__ __forceinline__ void queue_tile(const InstDesc &d, int nl, int t, unsigned char *smem_raw, int *red)
 {
     using io = typename Pol::io_t;
     using tw = typename Pol::tw_t;
@@ -705,168 +478,46 @@ __device__ __forceinline__ void queue_tile(const InstDesc &d, int nl, int t, uns
     }
 }
 
-// Item of a CTA (shared): valid if go != 0.
-struct QueueItem {
-    int go, pass, inst, tile;
-};
-
-// The tile of pass PASS if the CTA's item belongs to that pass, then one
-// release of the instance's count for the pass.
-template <class Pol, int D, int PASS>
-__device__ __forceinline__ void queue_pass(const QueueArgs &a, const QueueItem &it, unsigned char *smem_raw)
-{
-    if (it.go && it.pass == PASS) {
-        const int i = it.inst;
-        queue_tile<Pol, D, PASS>(a.inst[i], a.nl, it.tile, smem_raw);
-        // every thread's stores of the tile, then one release of the count
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned *cnt = a.state + kStateHeader + i * kBatchPasses + PASS;
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(cnt) : "memory");
-        }
-    }
-}
-
-template <class Pol, int D>
-// Resident CTAs per SM asked of the compiler: FP64 and double-float 2 (a
-// 128-register cap), FP32 5 (51 registers; its tiles are short, and more
-// resident CTAs cover their ticket and acquire: measured 4 % faster with 4
-// than with 3, 2 % faster again with 5, slower with 6)
-__global__ void __launch_bounds__(32 * kBatchMaxLines, std::is_same<Pol, F32>::value ? 5 : 2)
-    k_batch_queue(const __grid_constant__ QueueArgs a)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ QueueItem it;
-    if (threadIdx.x == 0) {
-        int p = 0, i = 0, t = 0;
-        it.go = take_item(a, &p, &i, &t) ? 1 : 0;
-        it.pass = p;
-        it.inst = i;
-        it.tile = t;
-    }
-    __syncthreads();
-    if (!it.go) return;
-    queue_pass<Pol, D, 0>(a, it, smem_raw);
-    queue_pass<Pol, D, 1>(a, it, smem_raw);
-    queue_pass<Pol, D, 2>(a, it, smem_raw);
-    if constexpr (D == 3) {
-        queue_pass<Pol, D, 3>(a, it, smem_raw);
-        queue_pass<Pol, D, 4>(a, it, smem_raw);
-    }
-}
-
 // ------------------------------------------------------------------ tables
-// Constants of the FMA-form stages (slot-major blocks, see gindex in gsm_fft.cuh),
-// one thread per (stage, j).  For stage radix R with Ns, forward twiddle
-// W_t = exp(-2 pi i q / D), q = j t, D = R Ns: with K = round(4 q / D) and
-// m = q - K D/4 (|m| <= D/8), W_t = i^(-K) exp(-2 pi i m / D), so k_t = -K mod 4,
-// f_t = cos(2 pi m / D), tau_t = -tan(2 pi m / D).
-struct GStage {
-    int R;
-    long Ns, off;   // off: first double of the stage's constants
-};
-struct GTableDesc {
-    int n;
-    GStage s[kMaxStages];
-};
-
-__global__ void k_gtable(GTableDesc d, double *out)
-{
-    const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    long base = 0;
-    int st = 0;
-    for (; st < d.n && idx >= base + d.s[st].Ns; ++st) base += d.s[st].Ns;
-    if (st >= d.n) return;
-    const int R = d.s[st].R;
-    const long Ns = d.s[st].Ns, j = idx - base, D = R * Ns;
-    double f[8], tau[8];
-    int codes = 0;
-    f[0] = 1.0;
-    tau[0] = 0.0;
-    for (int t = 1; t < R; ++t) {
-        const long q = j * t;
-        const long K = (4 * q + D / 2) / D;
-        const long m = q - K * (D / 4);
-        const int k = (int)((4 - (K & 3)) & 3);
-        double sn, cs;
-        sincospi(2.0 * (double)m / (double)D, &sn, &cs);
-        f[t] = cs;
-        tau[t] = (k & 1) ? sn / cs : -sn / cs;   // tau sigma_t, sigma_t = -1 for odd k
-        codes |= k << (2 * (t - 1));
-    }
-    double *cj = out + d.s[st].off + gindex(R, j);
-    auto c = [&](int q) -> double & { return cj[q * kGBlk]; };
-    if (R == 8) {
-        for (int t = 1; t < 8; ++t) c(t - 1) = tau[t];
-        for (int t = 0; t < 4; ++t) c(7 + t) = f[t + 4] / f[t];
-        c(11) = f[2];
-        c(12) = f[3] / f[1];
-        c(13) = f[1];
-        c(14) = f[1] * 0.707106781186547524400844362104849039;
-        c(15) = __hiloint2double(0, codes);
-    } else if (R == 4) {
-        for (int t = 1; t < 4; ++t) c(t - 1) = tau[t];
-        c(3) = f[2];
-        c(4) = f[3] / f[1];
-        c(5) = f[1];
-        c(6) = __hiloint2double(0, codes);
-        c(7) = 0.0;
-    } else {
-        c(0) = tau[1];
-        c(1) = f[1];
-        c(2) = __hiloint2double(0, codes);
-        c(3) = 0.0;
-    }
-}
-
-// Fills the FMA-form constants of schedule sc at `dst` (just after the M
-// twiddles of an FP64 table, so 16-byte aligned).
-void launch_g8table(const Sched &sc, double2 *dst, cudaStream_t st)
-{
-    GTableDesc d;
-    d.n = 0;
-    long Ns = 1, entries = 0;
-    for (int i = 0; i < sc.nst; ++i) {
-        if (gtabled_at(sc.r[i], Ns)) {
-            d.s[d.n].R = sc.r[i];
-            d.s[d.n].Ns = Ns;
-            d.s[d.n].off = (long)gtable_offset(sc, i);
-            ++d.n;
-            entries += Ns;
-        }
-        Ns *= sc.r[i];
-    }
-    if (entries > 0) k_gtable<<<(entries + 127) / 128, 128, 0, st>>>(d, reinterpret_cast<double *>(dst));
-}
-
-// w[m] = exp(-2 pi i m / M) from sincospi in FP64, then rounded or split.
-__global__ void k_twiddles(int M, int prec, void *out)
+// w[m] = exp(-2 pi i m / M) from sincospi in FP64, rounded to FP32.
+__global__ void k_twiddles(int M, float2 *out)
 {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m >= M) return;
     double sn, cs;
     sincospi(2.0 * m / M, &sn, &cs);
-    const double re = cs, im = -sn;
-    if (prec == GSM_FP64) {
-        reinterpret_cast<double2 *>(out)[m] = make_double2(re, im);
-    } else if (prec == GSM_FP32) {
-        reinterpret_cast<float2 *>(out)[m] = make_float2((float)re, (float)im);
-    } else {
-        const df a = df_from_double(re), b = df_from_double(im);
-        reinterpret_cast<float4 *>(out)[m] = make_float4(a.hi, a.lo, b.hi, b.lo);
-    }
+    out[m] = make_float2((float)cs, (float)-sn);
 }
 
-__global__ void k_mult_convert(const double *in, size_t count, int prec, void *out)
+__global__ void k_mult_convert(const double *in, size_t count, float *out)
 {
     const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i >= count) return;
-    if (prec == GSM_FP32) {
-        reinterpret_cast<float *>(out)[i] = (float)in[i];
-    } else {
-        const df a = df_from_double(in[i]);
-        reinterpret_cast<float2 *>(out)[i] = make_float2(a.hi, a.lo);
-    }
+    if (i < count) out[i] = (float)in[i];
+}
+
+// Twiddle table of a schedule in the precision of Pol: bytes, and its filling.
+// plain: entries w_plain_m^i appended for the split 2D passes (FX; the FP32
+// table is plain itself).
+template <class Pol>
+size_t table_bytes(const Sched &sc, int plain)
+{
+    if constexpr (std::is_same<Pol, FX>::value) return fx_table_bytes(sc.M, plain);
+    else return sizeof(float2) * sc.M;
+}
+template <class Pol>
+void fill_table(const Sched &sc, int plain, int plain_m, void *out, cudaStream_t st)
+{
+    if constexpr (std::is_same<Pol, FX>::value) launch_fx_twiddles(sc, plain, plain_m, out, st);
+    else k_twiddles<<<(sc.M + 255) / 256, 256, 0, st>>>(sc.M, static_cast<float2 *>(out));
+}
+size_t plan_table_bytes(const Plan *p, const Sched &sc, int plain)
+{
+    return p->opt.precision == GSM_FP32 ? table_bytes<F32>(sc, plain) : table_bytes<FX>(sc, plain);
+}
+void fill_plan_table(const Plan *p, const Sched &sc, int plain, int plain_m, void *out, cudaStream_t st)
+{
+    if (p->opt.precision == GSM_FP32) fill_table<F32>(sc, plain, plain_m, out, st);
+    else fill_table<FX>(sc, plain, plain_m, out, st);
 }
 
 // ------------------------------------------------------------------ Hartree energy
@@ -920,35 +571,20 @@ __global__ void k_energy_final(const double *partial, int nparts, double cell, T
 
 constexpr int kEnergyBlocks = 1024;
 
-// ------------------------------------------------------------------ launching
-// The dynamic shared-memory limit is per kernel function, shared by every
-// plan; it is always raised to the device's opt-in maximum (never lowered) so
-// that one plan cannot shrink the limit another plan launches with.
-template <class K>
-cudaError_t raise_smem(K kernel, size_t smem)
-{
-    if (smem <= 48 * 1024) return cudaSuccess;
-    int dev = 0, optin = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e != cudaSuccess) return e;
-    if ((size_t)optin < smem) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-}
-
-template <class Pol>
-size_t pass_smem(int M, int nl) { return (size_t)nl * line_stride<Pol>(M) * sizeof(S_t<Pol>); }
-
 // Launch shape for lines of length M: emax elements per thread (8 or 16),
 // gthr = threads per line (a multiple of 32 with gthr * emax >= M), nl lines
 // (groups) per CTA, nthr = nl * gthr <= kMaxThreads.  Groups larger than a
 // warp in a CTA of several groups use named barriers 1..nl (nl <= 15).
+template <class Pol>
+constexpr int max_threads(int emax) { return std::is_same<Pol, FX>::value ? fx_threads(emax) : kMaxThreads; }
+
 inline int round32(int x) { return ((x + 31) / 32) * 32; }
 
 template <class Pol>
-bool make_cfg(int M, int nl, int emax, PassCfg *c, int maxt = kMaxThreads)
+bool make_cfg(int M, int nl, int emax, PassCfg *c)
 {
     const int gthr = std::max(32, round32((M + emax - 1) / emax));
+    const int maxt = max_threads<Pol>(emax);
     if (gthr > maxt || nl < 1 || nl * gthr > maxt) return false;
     if (gthr > 32 && nl > 1 && nl > 15) return false;
     if (pass_smem<Pol>(M, nl) > 200 * 1024) return false;
@@ -963,23 +599,67 @@ bool make_cfg(int M, int nl, int emax, PassCfg *c, int maxt = kMaxThreads)
 // Default shape before any tuning: 8 elements per thread when a line fits
 // 512 threads that way, else 16; as many lines as requested that fit.
 template <class Pol>
-PassCfg choose_cfg(int M, int nl_want, bool conv = false)
+PassCfg choose_cfg(int M, int nl_want)
 {
     PassCfg c;
-    const int emax = (M <= 8 * kMaxThreads) ? 8 : 16;
-    const int maxt = conv ? conv_max_threads<Pol>(emax) : xy_max_threads<Pol>(emax);
+    const int emax = (M <= 8 * max_threads<Pol>(8)) ? 8 : 16;
     for (int nl = std::max(1, nl_want); nl >= 1; nl /= 2)
-        if (make_cfg<Pol>(M, nl, emax, &c, maxt)) return c;
+        if (make_cfg<Pol>(M, nl, emax, &c)) return c;
     make_cfg<Pol>(M, 1, 16, &c);
     return c;
 }
 
-// Calls f(std::integral_constant<int, E>) with E = c.emax.
-template <class F>
-void with_emax(const PassCfg &c, F &&f)
+// Shared-memory limit of the kernel of a pass with shape c.
+template <class Pol>
+cudaError_t raise_pass_smem(const Plan *p, int pass, const PassCfg &c)
 {
-    if (c.emax == 8) f(std::integral_constant<int, 8>());
-    else f(std::integral_constant<int, 16>());
+    if constexpr (std::is_same<Pol, FX>::value) {
+        return fx_raise_smem(p, pass, c);
+    } else {
+        const int last = p->d == 3 ? 4 : 2;
+        cudaError_t e = cudaSuccess;
+        with_emax(c, [&](auto E) {
+            if (pass == 0) e = raise_smem(k_xf<Pol, E()>, c.smem);
+            else if (pass == last) e = raise_smem(k_xi<Pol, E()>, c.smem);
+            else if (p->d == 2 || pass == 2) e = raise_smem(k_conv<Pol, E()>, c.smem);
+            else if (pass == 1) e = raise_smem(k_yf<Pol, E()>, c.smem);
+            else e = raise_smem(k_yi<Pol, E()>, c.smem);
+        });
+        return e;
+    }
+}
+template <class Pol>
+cudaError_t raise_split_smem(bool conv, size_t smem)
+{
+    if constexpr (std::is_same<Pol, FX>::value) return fx_raise_split_smem(conv, smem);
+    else if (conv) return raise_smem(k_conv_split<Pol, 16>, smem);
+    else return raise_smem(k_xf_split<Pol, 16>, smem);
+}
+
+// Line exponents of a fixed-point plan: they follow the values of W1 in its
+// allocation.
+size_t fx_exp_count(const Plan *p)
+{
+    const size_t ny2 = (p->n[1] + 1) / 2, hx = p->n[0] + 1;
+    if (p->d == 2) return 2 * ny2 + hx;
+    return p->n[2] * ny2 + hx * p->n[2] + hx * p->M[1] + p->n[2] * hx;
+}
+FxExps fx_exps(const Plan *p)
+{
+    const size_t ny2 = (p->n[1] + 1) / 2, hx = p->n[0] + 1, nz = p->d == 3 ? p->n[2] : 1;
+    FxExps e;
+    e.xf = reinterpret_cast<int *>(static_cast<fxc *>(p->d_work1) + nz * hx * p->n[1]);
+    e.xf_par = 0;
+    if (p->d == 2) {
+        e.xf_par = p->split_x ? (int)ny2 : 0;
+        e.cv = e.xf + 2 * ny2;
+        e.yf = e.yi = nullptr;
+        return e;
+    }
+    e.yf = e.xf + nz * ny2;
+    e.cv = e.yf + hx * nz;
+    e.yi = e.cv + hx * p->M[1];
+    return e;
 }
 
 template <class Pol>
@@ -992,9 +672,9 @@ gsm_status_t configure_t(Plan *p)
     if (d == 3) {
         p->cfg_yf = choose_cfg<Pol>(p->M[1], cw);
         p->cfg_yi = p->cfg_yf;
-        p->cfg_conv = choose_cfg<Pol>(p->M[2], std::max(1, 4096 / p->M[2]), true);
+        p->cfg_conv = choose_cfg<Pol>(p->M[2], std::max(1, 4096 / p->M[2]));
     } else {
-        p->cfg_conv = choose_cfg<Pol>(p->M[1], std::max(1, 4096 / p->M[1]), true);
+        p->cfg_conv = choose_cfg<Pol>(p->M[1], std::max(1, 4096 / p->M[1]));
         // long lines: two half-length transforms per line on a cluster of two CTAs
         // (options.debug bit 1 keeps one CTA per line, for comparisons)
         p->split_conv = p->M[1] >= kSplitMinM && (p->opt.debug & 2) == 0;
@@ -1003,7 +683,7 @@ gsm_status_t configure_t(Plan *p)
                 set_error("no launch shape for the split conv pass");
                 return GSM_ERR_UNSUPPORTED_SIZE;
             }
-            GSM_CUDA_TRY(raise_smem(k_conv_split<Pol, 16>, p->cfg_split.smem));
+            GSM_CUDA_TRY(raise_split_smem<Pol>(true, p->cfg_split.smem));
         }
         // the same for the x forward pass
         p->split_x = p->M[0] >= kSplitMinM && p->M[0] == 2 * p->n[0] && (p->opt.debug & 2) == 0;
@@ -1012,17 +692,17 @@ gsm_status_t configure_t(Plan *p)
                 set_error("no launch shape for the split x pass");
                 return GSM_ERR_UNSUPPORTED_SIZE;
             }
-            GSM_CUDA_TRY(raise_smem(k_xf_split<Pol, 16>, p->cfg_xsplit.smem));
+            GSM_CUDA_TRY(raise_split_smem<Pol>(false, p->cfg_xsplit.smem));
         }
     }
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
-    with_emax(p->cfg_xf, [&](auto E) { chk(raise_smem(k_xf<Pol, E()>, p->cfg_xf.smem)); });
-    with_emax(p->cfg_xi, [&](auto E) { chk(raise_smem(k_xi<Pol, E()>, p->cfg_xi.smem)); });
-    with_emax(p->cfg_conv, [&](auto E) { chk(raise_smem(k_conv<Pol, E()>, p->cfg_conv.smem)); });
     if (d == 3) {
-        with_emax(p->cfg_yf, [&](auto E) { chk(raise_smem(k_yf<Pol, E()>, p->cfg_yf.smem)); });
-        with_emax(p->cfg_yi, [&](auto E) { chk(raise_smem(k_yi<Pol, E()>, p->cfg_yi.smem)); });
+        const PassCfg *c[5] = {&p->cfg_xf, &p->cfg_yf, &p->cfg_conv, &p->cfg_yi, &p->cfg_xi};
+        for (int pass = 0; pass < 5; ++pass) chk(raise_pass_smem<Pol>(p, pass, *c[pass]));
+    } else {
+        const PassCfg *c[3] = {&p->cfg_xf, &p->cfg_conv, &p->cfg_xi};
+        for (int pass = 0; pass < 3; ++pass) chk(raise_pass_smem<Pol>(p, pass, *c[pass]));
     }
     GSM_CUDA_TRY(e);
     // workspace
@@ -1035,15 +715,17 @@ gsm_status_t configure_t(Plan *p)
         p->work1_bytes = cb * hx * p->n[1];
         p->work2_bytes = 0;
     }
+    if constexpr (std::is_same<Pol, FX>::value) p->work1_bytes += sizeof(int) * fx_exp_count(p);
     GSM_CUDA_TRY(dev_alloc(&p->d_work1, p->work1_bytes));
     if (p->work2_bytes) GSM_CUDA_TRY(dev_alloc(&p->d_work2, p->work2_bytes));
     return GSM_OK;
 }
 
 // One pass of the apply: 3D passes 0..4 = xf, yf, conv, yi, xi; 2D 0..2 = xf, conv, xi.
-template <class Pol>
-void launch_pass_t(const Plan *p, int pass, const void *rho_v, void *u_v, cudaStream_t st)
+PassCfg *pass_cfg(Plan *p, int pass);
+void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cudaStream_t st)
 {
+    using Pol = F32;
     using io = typename Pol::io_t;
     using tw = typename Pol::tw_t;
     const io *rho = static_cast<const io *>(rho_v);
@@ -1068,7 +750,7 @@ void launch_pass_t(const Plan *p, int pass, const void *rho_v, void *u_v, cudaSt
     if (pass == 0 && p->split_x) {
         const PassCfg &c = p->cfg_xsplit;
         const tw *twh = static_cast<const tw *>(p->d_twxh);
-        k_xf_split<Pol, 16><<<2 * ((ny + 1) / 2), c.nthr, c.smem, st>>>(rho, W1, nx, ny, hx, p->sched_xh, twh, twx);
+            k_xf_split<Pol, 16><<<2 * ((ny + 1) / 2), c.nthr, c.smem, st>>>(rho, W1, nx, ny, hx, p->sched_xh, twh, twx);
         return;
     }
     if (pass == 0) {
@@ -1093,15 +775,15 @@ void launch_pass_t(const Plan *p, int pass, const void *rho_v, void *u_v, cudaSt
         }
         if (p->split_conv) {
             const PassCfg &cs = p->cfg_split;
-            k_conv_split<Pol, 16><<<2 * hx, cs.nthr, cs.smem, st>>>(
-                W1, mult, hx, ny + 1, p->sched_hf, p->sched_hi, static_cast<const tw *>(p->d_twh),
-                static_cast<const tw *>(p->d_twhi), twy, p->mult_full ? 1 : 0);
+            const tw *th = static_cast<const tw *>(p->d_twh), *thi = static_cast<const tw *>(p->d_twhi);
+            k_conv_split<Pol, 16><<<2 * hx, cs.nthr, cs.smem, st>>>(W1, mult, hx, ny + 1, p->sched_hf, p->sched_hi,
+                                                                        th, thi, twy, p->mult_full ? 1 : 0);
             return;
         }
         with_emax(c, [&](auto E) {
             k_conv<Pol, E()><<<(hx + c.nl - 1) / c.nl, c.nthr, c.smem, st>>>(
-                W1, mult, hx, ny, 0, 1, ny + 1, p->sched_f[1], p->sched_i[1], c.nl, c.gthr, twy, twyi,
-                p->mult_full ? 1 : 0);
+                    W1, mult, hx, ny, 0, 1, ny + 1, p->sched_f[1], p->sched_i[1], c.nl, c.gthr, twy, twyi,
+                    p->mult_full ? 1 : 0);
         });
     } else {
         const tw *twz = static_cast<const tw *>(p->d_tw[2]);
@@ -1130,8 +812,8 @@ void launch_pass_t(const Plan *p, int pass, const void *rho_v, void *u_v, cudaSt
             }
             with_emax(c, [&](auto E) {
                 k_conv<Pol, E()><<<(nlines + c.nl - 1) / c.nl, c.nthr, c.smem, st>>>(
-                    W2, mult, nlines, nz, 1, My, ny + 1, p->sched_f[2], p->sched_i[2], c.nl, c.gthr, twz, twzi,
-                    p->mult_full ? 1 : 0);
+                        W2, mult, nlines, nz, 1, My, ny + 1, p->sched_f[2], p->sched_i[2], c.nl, c.gthr, twz, twzi,
+                        p->mult_full ? 1 : 0);
             });
         } else {
             if constexpr (std::is_same<Pol, F32>::value) {
@@ -1149,6 +831,27 @@ void launch_pass_t(const Plan *p, int pass, const void *rho_v, void *u_v, cudaSt
     }
 }
 
+// Fixed point: the kernels are in gsm_fx.cu and gsm_fx_conv.cu.
+void launch_pass_fx(const Plan *p, int pass, const void *rho, void *u, cudaStream_t st)
+{
+    const FxCall c{p,           fx_exps(p),   static_cast<const double *>(rho), static_cast<double *>(u), p->d_work1,
+                   p->d_work2, p->d == 3 ? p->n[2] : 1, st};
+    const int conv = p->d == 3 ? 2 : 1;
+    if (pass == conv && p->split_conv) fx_launch_split(c, true);
+    else if (pass == 0 && p->split_x) fx_launch_split(c, false);
+    else if (pass == conv) fx_launch_conv(c, p->cfg_conv);
+    else fx_launch_xy(c, pass, *pass_cfg(const_cast<Plan *>(p), pass));
+}
+
+template <class Pol>
+void launch_pass_t(const Plan *p, int pass, const void *rho_v, void *u_v, cudaStream_t st)
+{
+    if constexpr (std::is_same<Pol, FX>::value) {
+        launch_pass_fx(p, pass, rho_v, u_v, st);
+    } else {
+        launch_pass_f32(p, pass, rho_v, u_v, st);
+    }
+}
 template <class Pol>
 gsm_status_t apply_t(const Plan *p, const void *rho, void *u, cudaStream_t st)
 {
@@ -1169,21 +872,6 @@ gsm_status_t pass_t(const Plan *p, int pass, const void *rho, void *u, cudaStrea
 // ------------------------------------------------------------------ autotuning
 // Each pass has its own launch shape; the tuner times candidate shapes of
 // one pass at a time (the others keep theirs) and keeps the fastest.
-template <class Pol>
-cudaError_t raise_pass_smem(const Plan *p, int pass, const PassCfg &c)
-{
-    const int last = p->d == 3 ? 4 : 2;
-    cudaError_t e = cudaSuccess;
-    with_emax(c, [&](auto E) {
-        if (pass == 0) e = raise_smem(k_xf<Pol, E()>, c.smem);
-        else if (pass == last) e = raise_smem(k_xi<Pol, E()>, c.smem);
-        else if (p->d == 2 || pass == 2) e = raise_smem(k_conv<Pol, E()>, c.smem);
-        else if (pass == 1) e = raise_smem(k_yf<Pol, E()>, c.smem);
-        else e = raise_smem(k_yi<Pol, E()>, c.smem);
-    });
-    return e;
-}
-
 PassCfg *pass_cfg(Plan *p, int pass)
 {
     if (p->d == 3) {
@@ -1224,7 +912,7 @@ std::string tune_key(const Plan *p, int pass)
     for (char &ch : name)
         if (ch == ' ') ch = '_';
     char buf[256];
-    snprintf(buf, sizeof(buf), "v4 %s p%d d%d n%d,%d,%d pass%d", name.c_str(), (int)p->opt.precision, p->d, p->n[0],
+    snprintf(buf, sizeof(buf), "v5 %s p%d d%d n%d,%d,%d pass%d", name.c_str(), (int)p->opt.precision, p->d, p->n[0],
              p->n[1], p->d == 3 ? p->n[2] : 1, pass);
     return buf;
 }
@@ -1280,15 +968,7 @@ bool pass_uses_rr(const Plan *p, int pass)
     return p->opt.precision == GSM_FP32 && p->rr_conv && p->M[axis] == 512;
 }
 
-// The split 2D conv has a fixed launch shape and half-length schedules of its own.
-// Largest CTA of a pass's kernel for a shape with emax elements per thread.
-template <class Pol>
-int pass_max_threads(const Plan *p, int pass, int emax)
-{
-    const bool conv = p->d == 3 ? pass == 2 : pass == 1;
-    return conv ? conv_max_threads<Pol>(emax) : xy_max_threads<Pol>(emax);
-}
-
+// The split 2D passes have a fixed launch shape and half-length schedules of their own.
 bool pass_is_split(const Plan *p, int pass)
 {
     return p->d == 2 && ((pass == 1 && p->split_conv) || (pass == 0 && p->split_x));
@@ -1343,6 +1023,7 @@ Sched fused_inverse(const Sched &f)
     Sched i = f;
     i.r[0] = f.r[f.nst - 1];
     for (int k = 0; k + 1 < f.nst; ++k) i.r[k + 1] = f.r[k];
+    set_pad(&i);
     return i;
 }
 
@@ -1462,7 +1143,7 @@ gsm_status_t autotune_t(Plan *p, cudaStream_t st, std::string *report)
             std::lock_guard<std::mutex> lock(g_tune_mutex);
             PassCfg c;
             Sched a, b;
-            if (cache_lookup(cache, key, &cnl, &cem, &cf, &ci) && make_cfg<Pol>(M, cnl, cem, &c, pass_max_threads<Pol>(p, pass, cem)) &&
+            if (cache_lookup(cache, key, &cnl, &cem, &cf, &ci) && make_cfg<Pol>(M, cnl, cem, &c) &&
                 sched_parse(cf.c_str(), p->M[axis], true, &a) && sched_parse(ci.c_str(), p->M[axis], false, &b) &&
                 raise_pass_smem<Pol>(p, pass, c) == cudaSuccess) {
                 s = apply_axis_pair(p, axis, df ? a : p->sched_f[axis], di ? b : p->sched_i[axis], st);
@@ -1508,7 +1189,7 @@ gsm_status_t autotune_t(Plan *p, cudaStream_t st, std::string *report)
         for (int emax : {8, 16}) {
             for (int nl : nls) {
                 PassCfg c;
-                if (!make_cfg<Pol>(M, nl, emax, &c, pass_max_threads<Pol>(p, pass, emax))) continue;
+                if (!make_cfg<Pol>(M, nl, emax, &c)) continue;
                 if (raise_pass_smem<Pol>(p, pass, c) != cudaSuccess) continue;
                 *cfg = c;
                 const float ms = time_pass<Pol>(p, pass, rho, u, st, e0, e1, &e);
@@ -1548,6 +1229,27 @@ gsm_status_t autotune_t(Plan *p, cudaStream_t st, std::string *report)
 }
 
 template <class Pol>
+cudaError_t launch_hook(const PassCfg &c, int nlines, int sign, const Sched &sc, const double *in, double *out,
+                        const void *d_tw, cudaStream_t st)
+{
+    if constexpr (std::is_same<Pol, FX>::value) {
+        return fx_launch_hook(c, nlines, sign, sc, in, out, d_tw, st);
+    } else {
+        const auto *tw = static_cast<const typename Pol::tw_t *>(d_tw);
+        const int blocks = (nlines + c.nl - 1) / c.nl;
+        const double2 *x = reinterpret_cast<const double2 *>(in);
+        double2 *y = reinterpret_cast<double2 *>(out);
+        cudaError_t e = cudaSuccess;
+        with_emax(c, [&](auto E) {
+            auto kernel = sign < 0 ? k_fft_hook<Pol, true, E()> : k_fft_hook<Pol, false, E()>;
+            e = raise_smem(kernel, c.smem);
+            if (e == cudaSuccess) kernel<<<blocks, c.nthr, c.smem, st>>>(x, y, nlines, sc, c.nl, c.gthr, tw);
+        });
+        return e;
+    }
+}
+
+template <class Pol>
 gsm_status_t fft_hook_t(int M, int nlines, int sign, const double *in, double *out, cudaStream_t st)
 {
     Sched sc;
@@ -1556,27 +1258,11 @@ gsm_status_t fft_hook_t(int M, int nlines, int sign, const double *in, double *o
         return GSM_ERR_UNSUPPORTED_SIZE;
     }
     void *d_tw = nullptr;
-    const size_t g8 = std::is_same<Pol, F64>::value ? g8_table_doubles(sc) : 0;
-    GSM_CUDA_TRY(dev_alloc_async_bytes(&d_tw, sizeof(typename Pol::tw_t) * M + sizeof(double) * g8, st));
-    k_twiddles<<<(M + 255) / 256, 256, 0, st>>>(M, Pol::kId, d_tw);
-    if (g8 > 0) launch_g8table(sc, static_cast<double2 *>(d_tw) + M, st);
+    GSM_CUDA_TRY(dev_alloc_async_bytes(&d_tw, table_bytes<Pol>(sc, 0), st));
+    fill_table<Pol>(sc, 0, 1, d_tw, st);
     const PassCfg c = choose_cfg<Pol>(M, std::max(1, 2048 / M));
-    const auto *tw = static_cast<const typename Pol::tw_t *>(d_tw);
-    const int blocks = (nlines + c.nl - 1) / c.nl;
     cudaError_t e = cudaSuccess;
-    with_emax(c, [&](auto E) {
-        if (sign < 0) {
-            e = raise_smem(k_fft_hook<Pol, true, E()>, c.smem);
-            if (e == cudaSuccess)
-                k_fft_hook<Pol, true, E()><<<blocks, c.nthr, c.smem, st>>>((const double2 *)in, (double2 *)out,
-                                                                           nlines, sc, c.nl, c.gthr, tw, 1);
-        } else {
-            e = raise_smem(k_fft_hook<Pol, false, E()>, c.smem);
-            if (e == cudaSuccess)
-                k_fft_hook<Pol, false, E()><<<blocks, c.nthr, c.smem, st>>>((const double2 *)in, (double2 *)out,
-                                                                            nlines, sc, c.nl, c.gthr, tw, 1);
-        }
-    });
+    e = launch_hook<Pol>(c, nlines, sign, sc, in, out, d_tw, st);
     if (e == cudaSuccess) e = cudaGetLastError();
     dev_free_async(d_tw, st);
     GSM_CUDA_TRY(e);
@@ -1600,6 +1286,7 @@ bool make_sched(int M, Sched *s)
             m /= r;
         }
     }
+    set_pad(s);
     return m == 1;
 }
 
@@ -1608,11 +1295,10 @@ size_t cplx_bytes(gsm_precision_t prec) { return prec == GSM_FP32 ? 8 : 16; }
 namespace {
 
 // Whether the table made for (M, schedule a) serves (M, schedule b): equal M
-// and, in FP64 (whose tables end with the schedule's FMA-form constants),
-// equal schedules.
+// and, in fixed point (whose tables are in stage order), equal schedules.
 bool table_serves(const Plan *p, const Sched &a, const Sched &b)
 {
-    return a.M == b.M && (p->opt.precision != GSM_FP64 || same_sched(a, b));
+    return a.M == b.M && (p->opt.precision == GSM_FP32 || same_sched(a, b));
 }
 
 // The table of (axis, inverse?): an existing table that serves it, or a new one.
@@ -1630,11 +1316,11 @@ gsm_status_t table_for(Plan *p, int axis, bool inverse, cudaStream_t st, void **
         }
     }
     const int M = want.M;
-    const size_t g8 = p->opt.precision == GSM_FP64 ? g8_table_doubles(want) : 0;
+    // the split 2D passes also need the first M / 2 of the M twiddles in order
+    const int plain = p->d == 2 && M >= kSplitMinM ? M / 2 : 0;
     void *t = nullptr;
-    GSM_CUDA_TRY(dev_alloc(&t, cplx_bytes(p->opt.precision) * M + sizeof(double) * g8));
-    k_twiddles<<<(M + 255) / 256, 256, 0, st>>>(M, p->opt.precision, t);
-    if (g8 > 0) launch_g8table(want, static_cast<double2 *>(t) + M, st);
+    GSM_CUDA_TRY(dev_alloc(&t, plan_table_bytes(p, want, plain)));
+    fill_plan_table(p, want, plain, M, t, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         dev_free(t);
@@ -1691,10 +1377,8 @@ gsm_status_t make_xsplit_tables(Plan *p, cudaStream_t st)
         set_error("half length of the split x pass is not a product of 2, 3 and 5");
         return GSM_ERR_UNSUPPORTED_SIZE;
     }
-    const size_t g8 = p->opt.precision == GSM_FP64 ? g8_table_doubles(p->sched_xh) : 0;
-    GSM_CUDA_TRY(dev_alloc(&p->d_twxh, cplx_bytes(p->opt.precision) * Mh + sizeof(double) * g8));
-    k_twiddles<<<(Mh + 255) / 256, 256, 0, st>>>(Mh, p->opt.precision, p->d_twxh);
-    if (g8 > 0) launch_g8table(p->sched_xh, static_cast<double2 *>(p->d_twxh) + Mh, st);
+    GSM_CUDA_TRY(dev_alloc(&p->d_twxh, plan_table_bytes(p, p->sched_xh, 0)));
+    fill_plan_table(p, p->sched_xh, 0, 1, p->d_twxh, st);
     GSM_CUDA_TRY(cudaGetLastError());
     return GSM_OK;
 }
@@ -1707,20 +1391,16 @@ gsm_status_t make_split_tables(Plan *p, cudaStream_t st)
         return GSM_ERR_UNSUPPORTED_SIZE;
     }
     // the inverse starts with the forward's last radix: fused with the multiplication
-    p->sched_hi = p->sched_hf;
-    p->sched_hi.r[0] = p->sched_hf.r[p->sched_hf.nst - 1];
-    for (int k = 0; k + 1 < p->sched_hf.nst; ++k) p->sched_hi.r[k + 1] = p->sched_hf.r[k];
+    p->sched_hi = fused_inverse(p->sched_hf);
     const Sched *sc[2] = {&p->sched_hf, &p->sched_hi};
     void **dst[2] = {&p->d_twh, &p->d_twhi};
     for (int k = 0; k < 2; ++k) {
-        const size_t g8 = p->opt.precision == GSM_FP64 ? g8_table_doubles(*sc[k]) : 0;
-        if (k == 1 && g8 == 0) {   // without FMA-form constants one table serves both
+        if (k == 1 && table_serves(p, p->sched_hf, p->sched_hi)) {
             p->d_twhi = p->d_twh;
             break;
         }
-        GSM_CUDA_TRY(dev_alloc(dst[k], cplx_bytes(p->opt.precision) * Mh + sizeof(double) * g8));
-        k_twiddles<<<(Mh + 255) / 256, 256, 0, st>>>(Mh, p->opt.precision, *dst[k]);
-        if (g8 > 0) launch_g8table(*sc[k], static_cast<double2 *>(*dst[k]) + Mh, st);
+        GSM_CUDA_TRY(dev_alloc(dst[k], plan_table_bytes(p, *sc[k], 0)));
+        fill_plan_table(p, *sc[k], 0, 1, *dst[k], st);
         GSM_CUDA_TRY(cudaGetLastError());
     }
     return GSM_OK;
@@ -1740,6 +1420,7 @@ bool make_sched_order(int M, const int *radices, int count, bool forward, Sched 
     s->M = M;
     s->nst = count;
     for (int i = 0; i < kMaxStages; ++i) s->r[i] = (unsigned char)(i < count ? radices[i] : 0);
+    set_pad(s);
     return true;
 }
 
@@ -1787,14 +1468,15 @@ gsm_status_t set_axis_schedule(Plan *p, int axis, bool inverse, const Sched &sc,
 
 gsm_status_t make_pass_multiplier(Plan *p, cudaStream_t st)
 {
-    if (p->opt.precision == GSM_FP64) {
+    if (p->opt.precision != GSM_FP32) {
+        // the octant's rows (kx, ky) in 3D, kx in 2D, converted in place
+        const int len = p->n[p->d - 1] + 1;
         p->d_mult = p->d_mult64;
-        return GSM_OK;
+        return make_mult_rows(p, p->d_mult64, len, p->mult_elems / len, st);
     }
-    const size_t eb = p->opt.precision == GSM_FP32 ? sizeof(float) : sizeof(float2);
-    GSM_CUDA_TRY(dev_alloc(&p->d_mult, eb * p->mult_elems));
-    k_mult_convert<<<(p->mult_elems + 255) / 256, 256, 0, st>>>(p->d_mult64, p->mult_elems, p->opt.precision,
-                                                                  p->d_mult);
+    GSM_CUDA_TRY(dev_alloc(&p->d_mult, sizeof(float) * p->mult_elems));
+    k_mult_convert<<<(p->mult_elems + 255) / 256, 256, 0, st>>>(p->d_mult64, p->mult_elems,
+                                                                static_cast<float *>(p->d_mult));
     GSM_CUDA_TRY(cudaGetLastError());
     return GSM_OK;
 }
@@ -1808,20 +1490,14 @@ gsm_status_t configure_passes(Plan *p)
         }
         p->sched_i[a] = p->sched_f[a];
     }
-    switch (p->opt.precision) {
-    case GSM_FP64: return configure_t<F64>(p);
-    case GSM_FP32: return configure_t<F32>(p);
-    default: return configure_t<DF64>(p);
-    }
+    // fixed point: the conv axis's inverse starts with the forward's last radix
+    if (p->opt.precision != GSM_FP32) p->sched_i[p->d - 1] = fused_inverse(p->sched_f[p->d - 1]);
+    return p->opt.precision == GSM_FP32 ? configure_t<F32>(p) : configure_t<FX>(p);
 }
 
 gsm_status_t launch_apply(const Plan *p, const void *rho, void *u, cudaStream_t st)
 {
-    switch (p->opt.precision) {
-    case GSM_FP64: return apply_t<F64>(p, rho, u, st);
-    case GSM_FP32: return apply_t<F32>(p, rho, u, st);
-    default: return apply_t<DF64>(p, rho, u, st);
-    }
+    return p->opt.precision == GSM_FP32 ? apply_t<F32>(p, rho, u, st) : apply_t<FX>(p, rho, u, st);
 }
 
 template <class Pol>
@@ -1836,6 +1512,15 @@ gsm_status_t x_slabs_t(const Plan *p, bool inverse, int z0, int z1, const void *
     const tw *twx = static_cast<const tw *>(p->d_tw[0]);
     const tw *twxi = static_cast<const tw *>(p->d_twi[0]);
     if (z1 <= z0) return GSM_OK;
+    if constexpr (std::is_same<Pol, FX>::value) {
+        FxCall c{p, fx_exps(p), static_cast<const io *>(rho_v) + in_off, static_cast<io *>(u_v) + in_off, W1, nullptr,
+                 z1 - z0, st};
+        c.ex.xf += (size_t)z0 * ((ny + 1) / 2);
+        c.ex.yi += (size_t)z0 * hx;
+        fx_launch_xy(c, inverse ? 4 : 0, inverse ? p->cfg_xi : p->cfg_xf);
+        GSM_CUDA_TRY(cudaGetLastError());
+        return GSM_OK;
+    } else {
     if constexpr (std::is_same<Pol, F32>::value) {
         if (p->M[0] == 512 && p->rr_conv) {
             if (!inverse) launch_x_rr512_f32(false, static_cast<const io *>(rho_v) + in_off, W1, ny, z1 - z0, twx, st);
@@ -1861,6 +1546,7 @@ gsm_status_t x_slabs_t(const Plan *p, bool inverse, int z0, int z1, const void *
     }
     GSM_CUDA_TRY(cudaGetLastError());
     return GSM_OK;
+    }
 }
 
 gsm_status_t launch_x_slabs(const Plan *p, bool inverse, int z0, int z1, const void *rho, void *u, cudaStream_t st)
@@ -1869,27 +1555,19 @@ gsm_status_t launch_x_slabs(const Plan *p, bool inverse, int z0, int z1, const v
         set_error("x slabs: 3D plans and 0 <= z0 <= z1 <= nz only");
         return GSM_ERR_INVALID_ARG;
     }
-    switch (p->opt.precision) {
-    case GSM_FP64: return x_slabs_t<F64>(p, inverse, z0, z1, rho, u, st);
-    case GSM_FP32: return x_slabs_t<F32>(p, inverse, z0, z1, rho, u, st);
-    default: return x_slabs_t<DF64>(p, inverse, z0, z1, rho, u, st);
-    }
+    return p->opt.precision == GSM_FP32 ? x_slabs_t<F32>(p, inverse, z0, z1, rho, u, st) : x_slabs_t<FX>(p, inverse, z0, z1, rho, u, st);
 }
 
 gsm_status_t launch_pass(const Plan *p, int pass, const void *rho, void *u, cudaStream_t st)
 {
-    switch (p->opt.precision) {
-    case GSM_FP64: return pass_t<F64>(p, pass, rho, u, st);
-    case GSM_FP32: return pass_t<F32>(p, pass, rho, u, st);
-    default: return pass_t<DF64>(p, pass, rho, u, st);
-    }
+    return p->opt.precision == GSM_FP32 ? pass_t<F32>(p, pass, rho, u, st) : pass_t<FX>(p, pass, rho, u, st);
 }
 
 template <class Pol>
 gsm_status_t set_pass_shape_t(Plan *p, int pass, int nl, int emax)
 {
     PassCfg c;
-    if (!make_cfg<Pol>(pass_len(p, pass), nl, emax, &c, pass_max_threads<Pol>(p, pass, emax))) {
+    if (!make_cfg<Pol>(pass_len(p, pass), nl, emax, &c)) {
         set_error("launch shape not valid for this pass");
         return GSM_ERR_INVALID_ARG;
     }
@@ -1904,30 +1582,18 @@ gsm_status_t set_pass_shape(Plan *p, int pass, int nl, int emax)
         set_error("pass out of range");
         return GSM_ERR_INVALID_ARG;
     }
-    switch (p->opt.precision) {
-    case GSM_FP64: return set_pass_shape_t<F64>(p, pass, nl, emax);
-    case GSM_FP32: return set_pass_shape_t<F32>(p, pass, nl, emax);
-    default: return set_pass_shape_t<DF64>(p, pass, nl, emax);
-    }
+    return p->opt.precision == GSM_FP32 ? set_pass_shape_t<F32>(p, pass, nl, emax) : set_pass_shape_t<FX>(p, pass, nl, emax);
 }
 
 gsm_status_t autotune_plan(Plan *p, cudaStream_t st, std::string *report)
 {
-    switch (p->opt.precision) {
-    case GSM_FP64: return autotune_t<F64>(p, st, report);
-    case GSM_FP32: return autotune_t<F32>(p, st, report);
-    default: return autotune_t<DF64>(p, st, report);
-    }
+    return p->opt.precision == GSM_FP32 ? autotune_t<F32>(p, st, report) : autotune_t<FX>(p, st, report);
 }
 
 gsm_status_t launch_fft_lines(int M, int nlines, int sign, gsm_precision_t prec, const double *in,
                               double *out, cudaStream_t st)
 {
-    switch (prec) {
-    case GSM_FP64: return fft_hook_t<F64>(M, nlines, sign, in, out, st);
-    case GSM_FP32: return fft_hook_t<F32>(M, nlines, sign, in, out, st);
-    default: return fft_hook_t<DF64>(M, nlines, sign, in, out, st);
-    }
+    return prec == GSM_FP32 ? fft_hook_t<F32>(M, nlines, sign, in, out, st) : fft_hook_t<FX>(M, nlines, sign, in, out, st);
 }
 
 template <class T>
@@ -1960,16 +1626,14 @@ gsm_status_t launch_hartree(Plan *p, const void *psi, void *u, void *energy, voi
 }
 
 // ------------------------------------------------------------------ no-allocation FFT
-// Scratch of gsm_fft_lines_noalloc: the tables of one transform length, the M
-// twiddles (16-byte entries in FP64 and double-float, 8-byte in FP32) followed,
-// in FP64, by the constants of the FMA-form stages, exactly as gsm_fft_lines
-// builds them in its own allocation.  The largest need is M = 8192 in FP64,
-// 131072 + 208896 = 339968 bytes.  A file-scope __device__ array, so every GPU
-// that loads this library holds these 384 KiB until the process exits; every
-// call shares it.
+// Scratch of gsm_fft_lines_noalloc: the table of one transform length exactly
+// as gsm_fft_lines builds it in its own allocation (16-byte entries in fixed
+// point, 8-byte in FP32); the largest, M = 8192, is 131072 bytes.  A
+// file-scope __device__ array, so every GPU that loads this library holds these
+// 128 KiB until the process exits; every call shares it.
 namespace {
 
-constexpr size_t kStaticScratchBytes = 384 * 1024;
+constexpr size_t kStaticScratchBytes = 128 * 1024;
 __device__ __align__(256) unsigned char g_static_scratch[kStaticScratchBytes];
 
 typedef CUresult (*CtxGetCurrentFn)(CUcontext *);
@@ -2038,35 +1702,18 @@ gsm_status_t fft_hook_static_t(int M, int nlines, int sign, const double *in, do
         set_error("FFT length must be a product of 2, 3, 5 between 2 and 8192");
         return GSM_ERR_UNSUPPORTED_SIZE;
     }
-    const size_t g8 = std::is_same<Pol, F64>::value ? g8_table_doubles(sc) : 0;
-    const size_t need = sizeof(typename Pol::tw_t) * (size_t)M + sizeof(double) * g8;
-    if (need > kStaticScratchBytes) {
-        set_error("FFT tables exceed the 384 KiB static scratch (M <= 8192)");
+    if (table_bytes<Pol>(sc, 0) > kStaticScratchBytes) {
+        set_error("FFT tables exceed the 128 KiB static scratch (M <= 8192)");
         return GSM_ERR_UNSUPPORTED_SIZE;
     }
     void *d_tw = nullptr;
     GSM_CUDA_TRY(static_scratch_address(&d_tw));
     // the same tables gsm_fft_lines builds, so the same arithmetic and the same
     // bits; every entry the FFT reads is written here first: nothing needs clearing
-    k_twiddles<<<(M + 255) / 256, 256, 0, st>>>(M, Pol::kId, d_tw);
-    if (g8 > 0) launch_g8table(sc, static_cast<double2 *>(d_tw) + M, st);
+    fill_table<Pol>(sc, 0, 1, d_tw, st);
     const PassCfg c = choose_cfg<Pol>(M, std::max(1, 2048 / M));
-    const auto *tw = static_cast<const typename Pol::tw_t *>(d_tw);
-    const int blocks = (nlines + c.nl - 1) / c.nl;
     cudaError_t e = cudaSuccess;
-    with_emax(c, [&](auto E) {
-        if (sign < 0) {
-            e = raise_smem(k_fft_hook<Pol, true, E()>, c.smem);
-            if (e == cudaSuccess)
-                k_fft_hook<Pol, true, E()><<<blocks, c.nthr, c.smem, st>>>((const double2 *)in, (double2 *)out,
-                                                                           nlines, sc, c.nl, c.gthr, tw, 1);
-        } else {
-            e = raise_smem(k_fft_hook<Pol, false, E()>, c.smem);
-            if (e == cudaSuccess)
-                k_fft_hook<Pol, false, E()><<<blocks, c.nthr, c.smem, st>>>((const double2 *)in, (double2 *)out,
-                                                                            nlines, sc, c.nl, c.gthr, tw, 1);
-        }
-    });
+    e = launch_hook<Pol>(c, nlines, sign, sc, in, out, d_tw, st);
     GSM_CUDA_TRY(e);
     GSM_CUDA_TRY(cudaGetLastError());
     return GSM_OK;
@@ -2077,11 +1724,7 @@ gsm_status_t fft_hook_static_t(int M, int nlines, int sign, const double *in, do
 gsm_status_t launch_fft_lines_noalloc(int M, int nlines, int sign, gsm_precision_t prec, const double *in,
                                       double *out, cudaStream_t st)
 {
-    switch (prec) {
-    case GSM_FP64: return fft_hook_static_t<F64>(M, nlines, sign, in, out, st);
-    case GSM_FP32: return fft_hook_static_t<F32>(M, nlines, sign, in, out, st);
-    default: return fft_hook_static_t<DF64>(M, nlines, sign, in, out, st);
-    }
+    return prec == GSM_FP32 ? fft_hook_static_t<F32>(M, nlines, sign, in, out, st) : fft_hook_static_t<FX>(M, nlines, sign, in, out, st);
 }
 
 
@@ -2110,6 +1753,9 @@ void pass_grid(const Plan *p, int pass, int nl, int *gx, int *gy)
     } else if (p->d == 2) {
         *gx = (hx + nl - 1) / nl;
         *gy = 1;
+    } else if (pass == 2 && p->opt.precision != GSM_FP32) {
+        *gx = (p->M[1] + nl - 1) / nl;
+        *gy = hx;
     } else if (pass == 2) {
         *gx = (hx * p->M[1] + nl - 1) / nl;
         *gy = 1;
@@ -2121,6 +1767,13 @@ void pass_grid(const Plan *p, int pass, int nl, int *gx, int *gy)
 
 std::atomic<unsigned long long> g_batch_wait_ns{kBatchWaitDefaultNs};
 std::atomic<int> g_batch_hold{-1};
+
+template <class Pol>
+cudaError_t launch_queue_kernel(const QueueArgs &a, size_t smem, cudaStream_t st, bool dry)
+{
+    if constexpr (std::is_same<Pol, FX>::value) return a.d == 3 ? launch_queue_fx3(a, smem, st, dry) : launch_queue_fx2(a, smem, st, dry);
+    else return a.d == 3 ? launch_queue_d<Pol, 3>(a, smem, st, dry) : launch_queue_d<Pol, 2>(a, smem, st, dry);
+}
 
 template <class Pol>
 gsm_status_t launch_queue_t(QueueArgs &a, const std::vector<const Plan *> &plans, const void *const *rho,
@@ -2137,6 +1790,8 @@ gsm_status_t launch_queue_t(QueueArgs &a, const std::vector<const Plan *> &plans
         d.W1 = p->d_work1;
         d.W2 = p->d_work2;
         d.mult = p->d_mult;
+        d.mrow = p->d_mrow;
+        if constexpr (std::is_same<Pol, FX>::value) d.ex = fx_exps(p);
         d.full = p->mult_full ? 1 : 0;
         for (int ax = 0; ax < 3; ++ax) {
             d.n[ax] = ax < p->d ? p->n[ax] : 1;
@@ -2169,14 +1824,7 @@ gsm_status_t launch_queue_t(QueueArgs &a, const std::vector<const Plan *> &plans
     }
     for (int pass = np; pass <= kBatchPasses; ++pass) a.start[pass] = item;
     a.total = item;
-    auto kernel = a.d == 3 ? k_batch_queue<Pol, 3> : k_batch_queue<Pol, 2>;
-    cudaError_t e = raise_smem(kernel, smem);
-    if (e == cudaSuccess && !dry) {
-        // one CTA per item
-        kernel<<<std::max(1, a.total), a.nl * 32, smem, st>>>(a);
-        e = cudaGetLastError();
-    }
-    GSM_CUDA_TRY(e);
+    GSM_CUDA_TRY(launch_queue_kernel<Pol>(a, smem, st, dry));
     return GSM_OK;
 }
 
@@ -2234,11 +1882,8 @@ gsm_status_t launch_batched(int count, const Plan *const *plans, const void *con
         a->hold = g_batch_hold.load();
         ++group;
         gsm_status_t s;
-        switch (plans[i]->opt.precision) {
-        case GSM_FP64: s = launch_queue_t<F64>(*a, grp, r.data(), w.data(), st, dry); break;
-        case GSM_FP32: s = launch_queue_t<F32>(*a, grp, r.data(), w.data(), st, dry); break;
-        default: s = launch_queue_t<DF64>(*a, grp, r.data(), w.data(), st, dry); break;
-        }
+        if (plans[i]->opt.precision == GSM_FP32) s = launch_queue_t<F32>(*a, grp, r.data(), w.data(), st, dry);
+        else s = launch_queue_t<FX>(*a, grp, r.data(), w.data(), st, dry);
         delete a;
         if (s != GSM_OK) return s;
     }

@@ -506,14 +506,8 @@ __global__ void k_multiplier_dip_full(DipFull dp, const double *__restrict__ mC,
     const double c = mC[((size_t)kx * (dp.n[1] + 1) + fy) * (dp.n[2] + 1) + fz];
     const double nm = dp.nv[0] * dp.mv[0] + dp.nv[1] * dp.mv[1] + dp.nv[2] * dp.mv[2];
     const double v = -nm * dp.norm + 3.0 * sym / (dp.L * dp.L) * c;
-    if (dp.prec == GSM_FP64) {
-        reinterpret_cast<double *>(out)[idx] = v;
-    } else if (dp.prec == GSM_FP32) {
-        reinterpret_cast<float *>(out)[idx] = (float)v;
-    } else {
-        const df a = df_from_double(v);
-        reinterpret_cast<float2 *>(out)[idx] = make_float2(a.hi, a.lo);
-    }
+    if (dp.prec == GSM_FP32) reinterpret_cast<float *>(out)[idx] = (float)v;
+    else reinterpret_cast<double *>(out)[idx] = v;   // then to fixed point (make_mult_rows)
 }
 }  // namespace
 
@@ -688,7 +682,8 @@ gsm_status_t build_plan_data(Plan *p, cudaStream_t st, const StoredPlanData *sto
     for (int a = 0; a < d; ++a) tot *= (size_t)(p->n[a] + 1);
     p->mult_elems = tot;
     GSM_CUDA_TRY(dev_alloc(&p->d_khat, sizeof(double) * tot));
-    GSM_CUDA_TRY(dev_alloc(&p->d_mult64, sizeof(double) * tot));
+    // the exponents of its rows follow it (fixed point)
+    GSM_CUDA_TRY(dev_alloc(&p->d_mult64, sizeof(double) * tot + sizeof(int) * (tot / (p->n[d - 1] + 1))));
     if (stored)
         GSM_CUDA_TRY(cudaMemcpyAsync(p->d_khat, stored->khat, sizeof(double) * tot, cudaMemcpyHostToDevice, st));
     else
@@ -754,11 +749,16 @@ gsm_status_t build_plan_data(Plan *p, cudaStream_t st, const StoredPlanData *sto
         dp.prec = p->opt.precision;
         const size_t full = (size_t)(p->n[0] + 1) * p->M[1] * p->M[2];
         const size_t eb = p->opt.precision == GSM_FP32 ? sizeof(float) : sizeof(double);
-        GSM_CUDA_TRY(dev_alloc(&p->d_mult, eb * full));
+        const size_t rows = full / p->M[2];
+        GSM_CUDA_TRY(dev_alloc(&p->d_mult, eb * full + sizeof(int) * rows));
         p->mult_full = true;
         p->mult_elems_pass = full;
         k_multiplier_dip_full<<<(full + 255) / 256, 256, 0, st>>>(dp, p->d_mult64, p->d_mult);
         GSM_CUDA_TRY(cudaGetLastError());
+        if (p->opt.precision != GSM_FP32) {
+            gsm_status_t s = make_mult_rows(p, p->d_mult, p->M[2], rows, st);
+            if (s != GSM_OK) return s;
+        }
         GSM_CUDA_TRY(cudaStreamSynchronize(st));
         return GSM_OK;
     }

@@ -1,0 +1,92 @@
+"""GPU tests of the block fixed-point transforms of the FP64 and FP32X2 passes:
+the accuracy of single lines against long double, and what one exponent per
+line has to carry (magnitudes far apart, scaling, zeros, subnormals,
+infinities and NaN)."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gsm():
+    import paper_1501_04438_gb300 as m
+    return m
+
+
+def _dft_long(x, sign):
+    """Rows of x transformed in long double (matrix product with a table of w_M^m)."""
+    M = x.shape[-1]
+    m = np.arange(M)
+    pi = np.longdouble("3.14159265358979323846264338327950288")
+    ang = sign * 2 * pi * m.astype(np.longdouble) / M
+    c, s = np.cos(ang), np.sin(ang)
+    idx = np.outer(m, m) % M
+    re, im = x.real.astype(np.longdouble), x.imag.astype(np.longdouble)
+    return re @ c[idx] - im @ s[idx], re @ s[idx] + im @ c[idx]
+
+
+# lengths around the kernels' edges: two stages, odd radices, the last length with one scale per
+# line (512) and the first rescaled after every stage (540), several threads groups
+@pytest.mark.parametrize("M", [16, 40, 100, 128, 320, 384, 512, 540, 1024, 2000])
+@pytest.mark.parametrize("sign", [-1, 1])
+def test_line_errors_are_those_of_fp64_or_less(gsm, M, sign):
+    """Relative rms error of a transform below 2^-53 sqrt(log2 M): the usual estimate of an FP64
+    FFT, u times the root of its number of radix-2 levels."""
+    import torch
+    rng = np.random.default_rng(M)
+    g = np.exp(-((np.arange(M) - 0.45 * M) / (0.06 * M)) ** 2)
+    x = np.stack([rng.standard_normal(M) + 1j * rng.standard_normal(M), g * (1 + 0.3j),
+                  (np.arange(M) == 3) * (1.0 + 0j), g * (1e-3 * rng.standard_normal(M) + 1j * rng.standard_normal(M)),
+                  np.where(np.arange(M) % 2 == 0, 1.0, 1e-14) * rng.standard_normal(M) + 0j])
+    re, im = _dft_long(x, sign)
+    got = gsm.fft_lines(torch.tensor(x, device="cuda"), sign, "fp64").cpu().numpy()
+    err = np.sqrt(np.sum((got.real - re) ** 2 + (got.imag - im) ** 2, axis=1) / np.sum(re ** 2 + im ** 2, axis=1))
+    assert np.all(err.astype(float) < 2.0 ** -53 * np.sqrt(np.log2(M))), err
+
+
+GRIDS = [("coulomb3d", (24, 20, 16)), ("poisson2d", (40, 54)), ("coulomb2d", (16, 2048)), ("coulomb2d", (2048, 16))]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32x2"])
+@pytest.mark.parametrize("kernel,n", GRIDS, ids=[f"{k}-{'x'.join(map(str, n))}" for k, n in GRIDS])
+def test_scaling_zeros_and_non_finite_values(gsm, kernel, n, precision):
+    """Powers of two scale the result exactly (exponents only), a density of zeros gives zeros,
+    subnormal results are rounded once more, an infinity or a NaN makes every output NaN."""
+    import torch
+    plan = gsm.Plan(kernel, 4.0, n, precision=precision)
+    rho = torch.tensor(np.random.default_rng(5).standard_normal(n[::-1]), device="cuda")
+    u = plan.apply(rho)
+    for k in (-600, 1, 600):
+        assert torch.equal(plan.apply(rho * 2.0 ** k), u * 2.0 ** k)
+    if kernel.startswith("coulomb"):
+        # the input's rounding to multiples of 2^-1074, half a unit each, through the (positive)
+        # kernel's row sums, and the output's own rounding
+        tiny = plan.apply(rho * 2.0 ** -500 * 2.0 ** -540)
+        rows = float(plan.apply(torch.ones_like(rho)).max())
+        err = (tiny - u * 2.0 ** -500 * 2.0 ** -540).abs().max() * 2.0 ** 500 * 2.0 ** 574
+        assert float(err) <= rows + 2.0
+    assert torch.equal(plan.apply(torch.zeros_like(rho)), torch.zeros_like(rho))
+    for bad in (float("nan"), float("inf"), -float("inf")):
+        r = rho.clone()
+        r.view(-1)[r.numel() // 3] = bad
+        assert bool(torch.isnan(plan.apply(r)).all())
+
+
+@pytest.mark.parametrize("kernel,n", GRIDS[:2], ids=["3d", "2d"])
+def test_lines_of_magnitudes_far_apart(gsm, kernel, n):
+    """Rows, columns and planes whose magnitudes differ by up to 1e30, against the oracle in the
+    relative max norm (FP64's own tolerance)."""
+    import torch
+    rng = np.random.default_rng(8)
+    rho = rng.standard_normal(n[::-1])
+    for axis, m in enumerate(rho.shape):
+        shape = [1] * rho.ndim
+        shape[axis] = m
+        rho = rho * (10.0 ** rng.uniform(-15, 0, size=m)).reshape(shape)
+    plan = gsm.Plan(kernel, 4.0, n)
+    u = plan.apply(torch.tensor(rho, device="cuda")).cpu().numpy()
+    uo, _ = oracle.apply(kernel, rho, 4.0, taylor_mode=1)
+    assert np.max(np.abs(u - uo)) / np.max(np.abs(uo)) < 1e-12
