@@ -252,10 +252,32 @@ GSM_HD void fx_bfly5(cx<long long> *v)
     v[3] = fx_subq<FWD>(p2, q2);
 }
 
+// Radix 6 = 2 x 3 without twiddles (prime factors: I. J. Good 1958): inputs
+// 3 n1 + 2 n2, outputs 3 k1 + 4 k2 mod 6.
+template <bool FWD>
+GSM_HD void fx_bfly6(cx<long long> *v)
+{
+    cx<long long> a[3], b[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        a[i] = fx_add(v[2 * i], v[(2 * i + 3) % 6]);
+        b[i] = fx_sub(v[2 * i], v[(2 * i + 3) % 6]);
+    }
+    fx_bfly3<FWD>(a);
+    fx_bfly3<FWD>(b);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        v[4 * k % 6] = a[k];
+        v[(3 + 4 * k) % 6] = b[k];
+    }
+}
+
 template <int RAD, bool FWD, int HALF>
 GSM_HD void fx_bfly(cx<long long> *v)
 {
-    if constexpr (RAD == 8) {
+    if constexpr (RAD == 6) {
+        fx_bfly6<FWD>(v);
+    } else if constexpr (RAD == 8) {
         fx_bfly8<FWD, HALF>(v);
     } else if constexpr (RAD == 4) {
         fx_bfly4<FWD, HALF>(v);

@@ -153,6 +153,11 @@ cudaError_t fx_launch_hook(const PassCfg &c, int nlines, int sign, const Sched &
 cudaError_t fx_raise_smem(const Plan *p, int pass, const PassCfg &c);
 cudaError_t fx_raise_conv_smem(const PassCfg &c);
 cudaError_t fx_raise_split_smem(bool conv, size_t smem);
+// the passes of padded lengths 64 R, R = 1, 2, 3, 4, 5, 6, 8 (gsm_fx3.cuh)
+template <int R>
+cudaError_t f3_raise_smem(const Plan *p);
+template <int R>
+void f3_launch(const FxCall &c, int pass);
 size_t fx_table_bytes(int M, int plain);
 void launch_fx_twiddles(const Sched &sc, int plain, int plain_m, void *out, cudaStream_t st);
 // largest CTA of the kernels with emax elements per thread

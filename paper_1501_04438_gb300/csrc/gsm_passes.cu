@@ -704,6 +704,8 @@ gsm_status_t configure_t(Plan *p)
         const PassCfg *c[3] = {&p->cfg_xf, &p->cfg_conv, &p->cfg_xi};
         for (int pass = 0; pass < 3; ++pass) chk(raise_pass_smem<Pol>(p, pass, *c[pass]));
     }
+    if constexpr (std::is_same<Pol, FX>::value)
+        for (int a = 0; a < d; ++a) with_f3(p->M[a], [&](auto R) { chk(f3_raise_smem<R()>(p)); });
     GSM_CUDA_TRY(e);
     // workspace
     const size_t cb = sizeof(S_t<Pol>);
@@ -831,13 +833,33 @@ void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cuda
     }
 }
 
-// Fixed point: the kernels are in gsm_fx.cu and gsm_fx_conv.cu.
+bool pass_uses_f3(const Plan *p, int pass);
+int f3_radix(int M);
+// Calls f(std::integral_constant<int, R>) with the R of padded length M.
+template <class F>
+void with_f3(int M, F &&f)
+{
+    switch (f3_radix(M)) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: f(std::integral_constant<int, 2>()); break;
+    case 3: f(std::integral_constant<int, 3>()); break;
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 5: f(std::integral_constant<int, 5>()); break;
+    case 6: f(std::integral_constant<int, 6>()); break;
+    case 8: f(std::integral_constant<int, 8>()); break;
+    default: break;
+    }
+}
+int pass_len(const Plan *p, int pass);
+
+// Fixed point: the kernels are in gsm_fx.cu, gsm_fx_conv.cu and gsm_fx3_*.cu.
 void launch_pass_fx(const Plan *p, int pass, const void *rho, void *u, cudaStream_t st)
 {
     const FxCall c{p,           fx_exps(p),   static_cast<const double *>(rho), static_cast<double *>(u), p->d_work1,
                    p->d_work2, p->d == 3 ? p->n[2] : 1, st};
     const int conv = p->d == 3 ? 2 : 1;
-    if (pass == conv && p->split_conv) fx_launch_split(c, true);
+    if (pass_uses_f3(p, pass)) with_f3(pass_len(p, pass), [&](auto R) { f3_launch<R()>(c, pass); });
+    else if (pass == conv && p->split_conv) fx_launch_split(c, true);
     else if (pass == 0 && p->split_x) fx_launch_split(c, false);
     else if (pass == conv) fx_launch_conv(c, p->cfg_conv);
     else fx_launch_xy(c, pass, *pass_cfg(const_cast<Plan *>(p), pass));
@@ -1027,6 +1049,57 @@ Sched fused_inverse(const Sched &f)
     return i;
 }
 
+// Default schedules of an axis: engine order; in fixed point the conv axis's
+// inverse starts with the forward's last radix (fused with the multiplication).
+Sched default_sched(const Plan *p, int axis, bool inverse)
+{
+    Sched sc;
+    make_sched(p->M[axis], &sc);
+    if (inverse && axis == p->d - 1 && p->opt.precision != GSM_FP32) return fused_inverse(sc);
+    return sc;
+}
+
+// R of the fixed-length kernels (gsm_fx3.cuh) for padded length M (0: none)
+int f3_radix(int M)
+{
+    const int R = M / 64;
+    return M % 64 == 0 && (R == 1 || R == 2 || R == 3 || R == 4 || R == 5 || R == 6 || R == 8) ? R : 0;
+}
+
+// Their stages: 8 8 R forward and in the inverse x and y passes, R 8 8 in the conv's inverse.
+Sched f3_sched(int M, bool conv_inverse)
+{
+    const int R = f3_radix(M);
+    Sched sc{};
+    sc.M = M;
+    sc.nst = R == 1 ? 2 : 3;
+    for (int i = 0; i < sc.nst; ++i) sc.r[i] = 8;
+    if (R > 1) sc.r[conv_inverse ? 0 : 2] = (unsigned char)R;
+    set_pad(&sc);
+    return sc;
+}
+
+// Whether the passes of (axis, inverse?) run them: fixed point, a length of
+// theirs, and the default schedules (schedules that were set or tuned run the
+// general kernels).  options.debug bit 2 turns them off, for comparisons.  The
+// conv pass takes both directions.
+bool uses_f3(const Plan *p, int axis, bool inverse)
+{
+    if (p->opt.precision == GSM_FP32 || (p->opt.debug & 4) != 0 || f3_radix(p->M[axis]) == 0) return false;
+    // (a conv inverse in engine order is what plans saved by earlier versions hold)
+    const bool f = same_sched(p->sched_f[axis], default_sched(p, axis, false));
+    const bool i = same_sched(p->sched_i[axis], default_sched(p, axis, true)) ||
+                   same_sched(p->sched_i[axis], default_sched(p, axis, false));
+    return axis == p->d - 1 ? f && i : inverse ? i : f;
+}
+bool pass_uses_f3(const Plan *p, int pass)
+{
+    int axis;
+    bool f, i;
+    pass_axis(p, pass, &axis, &f, &i);
+    return uses_f3(p, axis, i);
+}
+
 // Candidate (forward, inverse) schedules of pass `pass`, the current pair
 // first: single-direction passes vary their own direction over the
 // factorisations of M; the conv pass tries, for each factorisation, the
@@ -1154,6 +1227,11 @@ gsm_status_t autotune_t(Plan *p, cudaStream_t st, std::string *report)
                 *report += buf;
                 continue;
             }
+        }
+        if (pass_uses_f3(p, pass)) {
+            snprintf(buf, sizeof(buf), "pass %d M=%d fixed-length kernel (fixed schedule and shape)\n", pass, M);
+            *report += buf;
+            continue;
         }
         if (pass_is_split(p, pass)) {
             snprintf(buf, sizeof(buf), "pass %d M=%d split into two halves on a CTA pair (fixed shape)\n", pass, M);
@@ -1294,6 +1372,14 @@ size_t cplx_bytes(gsm_precision_t prec) { return prec == GSM_FP32 ? 8 : 16; }
 
 namespace {
 
+// The stages that the passes of (axis, inverse?) run: those of the schedule, or
+// those of the fixed-length kernels where they serve.
+Sched run_sched(const Plan *p, int axis, bool inverse)
+{
+    if (uses_f3(p, axis, inverse)) return f3_sched(p->M[axis], inverse && axis == p->d - 1);
+    return inverse ? p->sched_i[axis] : p->sched_f[axis];
+}
+
 // Whether the table made for (M, schedule a) serves (M, schedule b): equal M
 // and, in fixed point (whose tables are in stage order), equal schedules.
 bool table_serves(const Plan *p, const Sched &a, const Sched &b)
@@ -1304,13 +1390,13 @@ bool table_serves(const Plan *p, const Sched &a, const Sched &b)
 // The table of (axis, inverse?): an existing table that serves it, or a new one.
 gsm_status_t table_for(Plan *p, int axis, bool inverse, cudaStream_t st, void **out)
 {
-    const Sched &want = inverse ? p->sched_i[axis] : p->sched_f[axis];
+    const Sched want = run_sched(p, axis, inverse);
     for (int b = 0; b < p->d; ++b) {
-        if (p->d_tw[b] && table_serves(p, p->sched_f[b], want) && !(b == axis && inverse == false)) {
+        if (p->d_tw[b] && table_serves(p, run_sched(p, b, false), want) && !(b == axis && inverse == false)) {
             *out = p->d_tw[b];
             return GSM_OK;
         }
-        if (p->d_twi[b] && table_serves(p, p->sched_i[b], want) && !(b == axis && inverse == true)) {
+        if (p->d_twi[b] && table_serves(p, run_sched(p, b, true), want) && !(b == axis && inverse == true)) {
             *out = p->d_twi[b];
             return GSM_OK;
         }
@@ -1488,10 +1574,8 @@ gsm_status_t configure_passes(Plan *p)
             set_error("padded length 2n must be a product of 2, 3 and 5");
             return GSM_ERR_UNSUPPORTED_SIZE;
         }
-        p->sched_i[a] = p->sched_f[a];
+        p->sched_i[a] = default_sched(p, a, true);
     }
-    // fixed point: the conv axis's inverse starts with the forward's last radix
-    if (p->opt.precision != GSM_FP32) p->sched_i[p->d - 1] = fused_inverse(p->sched_f[p->d - 1]);
     return p->opt.precision == GSM_FP32 ? configure_t<F32>(p) : configure_t<FX>(p);
 }
 
@@ -1517,7 +1601,9 @@ gsm_status_t x_slabs_t(const Plan *p, bool inverse, int z0, int z1, const void *
                  z1 - z0, st};
         c.ex.xf += (size_t)z0 * ((ny + 1) / 2);
         c.ex.yi += (size_t)z0 * hx;
-        fx_launch_xy(c, inverse ? 4 : 0, inverse ? p->cfg_xi : p->cfg_xf);
+        const int pass = inverse ? 4 : 0;
+        if (pass_uses_f3(p, pass)) with_f3(p->M[0], [&](auto R) { f3_launch<R()>(c, pass); });
+        else fx_launch_xy(c, pass, inverse ? p->cfg_xi : p->cfg_xf);
         GSM_CUDA_TRY(cudaGetLastError());
         return GSM_OK;
     } else {
@@ -1739,6 +1825,10 @@ bool batch_eligible(const Plan *p)
         // a batch gives the same bits as gsm_apply
         if (p->opt.precision == GSM_FP32 && p->rr_conv && p->M[a] == 512) return false;
     }
+    // nor do plans with a pass on the fixed-length kernels, for speed
+    const int np = p->d == 3 ? 5 : 3;
+    for (int pass = 0; pass < np; ++pass)
+        if (pass_uses_f3(p, pass)) return false;
     return true;
 }
 

@@ -90,3 +90,31 @@ def test_lines_of_magnitudes_far_apart(gsm, kernel, n):
     u = plan.apply(torch.tensor(rho, device="cuda")).cpu().numpy()
     uo, _ = oracle.apply(kernel, rho, 4.0, taylor_mode=1)
     assert np.max(np.abs(u - uo)) / np.max(np.abs(uo)) < 1e-12
+
+
+# padded lengths 64 R with kernels of their own, as the x, y and z lines of grids whose other
+# axes leave the last CTA ragged, and 2D; general dipole axes take the half-spectrum multiplier
+FIXED = (32, 64, 96, 128, 160, 192, 256)
+ROLES = [("coulomb3d", lambda N: (N, 10, 8)), ("coulomb3d", lambda N: (10, N, 18)), ("dipolar3d", lambda N: (8, 10, N)),
+         ("coulomb2d", lambda N: (N, 54)), ("ds2d", lambda N: (18, N))]
+
+
+@pytest.mark.parametrize("role", range(len(ROLES)), ids=["x", "y", "z_full", "x2d", "y2d"])
+@pytest.mark.parametrize("N", FIXED)
+def test_fixed_length_kernels(gsm, N, role):
+    """The fixed-length kernels against the oracle and against the kernels of any length
+    (options.debug bit 2), whose lines take the same steps: relative differences of a few
+    roundings of the result, 2^-53 log2 of the padded volume."""
+    import torch
+    kernel, shape = ROLES[role]
+    n = shape(N)
+    kw = dict(dip_n=(0.6, 0.0, 0.8), dip_m=(0.0, 0.8, 0.6)) if kernel == "dipolar3d" else {}
+    rho = np.random.default_rng(N).standard_normal(n[::-1])
+    r = torch.tensor(rho, device="cuda")
+    u = gsm.Plan(kernel, 4.0, n, **kw).apply(r).cpu().numpy()
+    v = gsm.Plan(kernel, 4.0, n, debug=4, **kw).apply(r).cpu().numpy()
+    scale = np.max(np.abs(u))
+    assert np.max(np.abs(u - v)) / scale < 2.0 ** -53 * np.log2(np.prod([2.0 * m for m in n]))
+    if kernel != "ds2d":   # (ln r: see the split-conv test on white noise)
+        uo, _ = oracle.apply(kernel, rho, 4.0, taylor_mode=1, **kw)
+        assert np.max(np.abs(u - uo)) / np.max(np.abs(uo)) < 1e-12
