@@ -158,6 +158,13 @@ template <int R>
 cudaError_t f3_raise_smem(const Plan *p);
 template <int R>
 void f3_launch(const FxCall &c, int pass);
+// the same in FP32 (gsm_f3_f32.cuh), R <= 6
+template <int R>
+cudaError_t f3f_raise_smem(const Plan *p);
+template <int R>
+void f3f_launch(const Plan *p, int pass, const float *rho, float *u, float2 *W1, int nz, cudaStream_t st);
+// w^(j t) of a schedule's stages in stage order (fx_stage_table), FP32 (gsm_f3_f32.cu)
+void launch_f32_stage_twiddles(const Sched &sc, float2 *out, cudaStream_t st);
 size_t fx_table_bytes(int M, int plain);
 void launch_fx_twiddles(const Sched &sc, int plain, int plain_m, void *out, cudaStream_t st);
 // largest CTA of the kernels with emax elements per thread

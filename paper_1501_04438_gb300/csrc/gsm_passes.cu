@@ -496,19 +496,21 @@ __global__ void k_mult_convert(const double *in, size_t count, float *out)
 }
 
 // Twiddle table of a schedule in the precision of Pol: bytes, and its filling.
-// plain: entries w_plain_m^i appended for the split 2D passes (FX; the FP32
-// table is plain itself).
+// FX: in stage order, then `plain` entries w_plain_m^i for the split 2D passes;
+// FP32: the M twiddles in order, then, with plain = M, the same in stage order
+// for the fixed-length kernels.
 template <class Pol>
 size_t table_bytes(const Sched &sc, int plain)
 {
     if constexpr (std::is_same<Pol, FX>::value) return fx_table_bytes(sc.M, plain);
-    else return sizeof(float2) * sc.M;
+    else return sizeof(float2) * (sc.M + (size_t)plain);
 }
 template <class Pol>
 void fill_table(const Sched &sc, int plain, int plain_m, void *out, cudaStream_t st)
 {
     if constexpr (std::is_same<Pol, FX>::value) launch_fx_twiddles(sc, plain, plain_m, out, st);
     else k_twiddles<<<(sc.M + 255) / 256, 256, 0, st>>>(sc.M, static_cast<float2 *>(out));
+    if (std::is_same<Pol, F32>::value && plain > 0) launch_f32_stage_twiddles(sc, static_cast<float2 *>(out) + sc.M, st);
 }
 size_t plan_table_bytes(const Plan *p, const Sched &sc, int plain)
 {
@@ -704,8 +706,11 @@ gsm_status_t configure_t(Plan *p)
         const PassCfg *c[3] = {&p->cfg_xf, &p->cfg_conv, &p->cfg_xi};
         for (int pass = 0; pass < 3; ++pass) chk(raise_pass_smem<Pol>(p, pass, *c[pass]));
     }
-    if constexpr (std::is_same<Pol, FX>::value)
-        for (int a = 0; a < d; ++a) with_f3(p->M[a], [&](auto R) { chk(f3_raise_smem<R()>(p)); });
+    for (int a = 0; a < d; ++a)
+        with_f3(p->M[a], [&](auto R) {
+            if constexpr (std::is_same<Pol, FX>::value) chk(f3_raise_smem<R()>(p));
+            else if constexpr (R() != 8) chk(f3f_raise_smem<R()>(p));
+        });
     GSM_CUDA_TRY(e);
     // workspace
     const size_t cb = sizeof(S_t<Pol>);
@@ -725,6 +730,32 @@ gsm_status_t configure_t(Plan *p)
 
 // One pass of the apply: 3D passes 0..4 = xf, yf, conv, yi, xi; 2D 0..2 = xf, conv, xi.
 PassCfg *pass_cfg(Plan *p, int pass);
+bool pass_uses_f3(const Plan *p, int pass);
+int f3_radix(int M);
+int pass_len(const Plan *p, int pass);
+// Calls f(std::integral_constant<int, R>) with the R of padded length M.
+template <class F>
+void with_f3(int M, F &&f)
+{
+    switch (f3_radix(M)) {
+    case 1: f(std::integral_constant<int, 1>()); break;
+    case 2: f(std::integral_constant<int, 2>()); break;
+    case 3: f(std::integral_constant<int, 3>()); break;
+    case 4: f(std::integral_constant<int, 4>()); break;
+    case 5: f(std::integral_constant<int, 5>()); break;
+    case 6: f(std::integral_constant<int, 6>()); break;
+    case 8: f(std::integral_constant<int, 8>()); break;
+    default: break;
+    }
+}
+// FP32: R <= 6 (n = 256 has the register-resident kernels)
+void launch_f3f(const Plan *p, int pass, const float *rho, float *u, float2 *W1, int nz, cudaStream_t st)
+{
+    with_f3(pass_len(p, pass), [&](auto R) {
+        if constexpr (R() != 8) f3f_launch<R()>(p, pass, rho, u, W1, nz, st);
+    });
+}
+
 void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cudaStream_t st)
 {
     using Pol = F32;
@@ -742,6 +773,10 @@ void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cuda
     const tw *twxi = static_cast<const tw *>(p->d_twi[0]);
     const tw *twyi = static_cast<const tw *>(p->d_twi[1]);
     const int last = p->d == 3 ? 4 : 2;
+    if (pass_uses_f3(p, pass)) {
+        launch_f3f(p, pass, rho, u, W1, nz, st);
+        return;
+    }
     if constexpr (std::is_same<Pol, F32>::value) {
         if ((pass == 0 || pass == last) && p->M[0] == 512 && p->rr_conv) {
             if (pass == 0) launch_x_rr512_f32(false, rho, W1, ny, nz, twx, st);
@@ -832,25 +867,6 @@ void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cuda
         }
     }
 }
-
-bool pass_uses_f3(const Plan *p, int pass);
-int f3_radix(int M);
-// Calls f(std::integral_constant<int, R>) with the R of padded length M.
-template <class F>
-void with_f3(int M, F &&f)
-{
-    switch (f3_radix(M)) {
-    case 1: f(std::integral_constant<int, 1>()); break;
-    case 2: f(std::integral_constant<int, 2>()); break;
-    case 3: f(std::integral_constant<int, 3>()); break;
-    case 4: f(std::integral_constant<int, 4>()); break;
-    case 5: f(std::integral_constant<int, 5>()); break;
-    case 6: f(std::integral_constant<int, 6>()); break;
-    case 8: f(std::integral_constant<int, 8>()); break;
-    default: break;
-    }
-}
-int pass_len(const Plan *p, int pass);
 
 // Fixed point: the kernels are in gsm_fx.cu, gsm_fx_conv.cu and gsm_fx3_*.cu.
 void launch_pass_fx(const Plan *p, int pass, const void *rho, void *u, cudaStream_t st)
@@ -1049,8 +1065,8 @@ Sched fused_inverse(const Sched &f)
     return i;
 }
 
-// Default schedules of an axis: engine order; in fixed point the conv axis's
-// inverse starts with the forward's last radix (fused with the multiplication).
+// Default schedules of an axis: engine order; the conv axis's inverse starts
+// with the forward's last radix (fused with the multiplication) in fixed point.
 Sched default_sched(const Plan *p, int axis, bool inverse)
 {
     Sched sc;
@@ -1079,13 +1095,15 @@ Sched f3_sched(int M, bool conv_inverse)
     return sc;
 }
 
-// Whether the passes of (axis, inverse?) run them: fixed point, a length of
-// theirs, and the default schedules (schedules that were set or tuned run the
+// Whether the passes of (axis, inverse?) run them: a length of theirs and the
+// default schedules (schedules that were set or tuned run the
 // general kernels).  options.debug bit 2 turns them off, for comparisons.  The
 // conv pass takes both directions.
 bool uses_f3(const Plan *p, int axis, bool inverse)
 {
-    if (p->opt.precision == GSM_FP32 || (p->opt.debug & 4) != 0 || f3_radix(p->M[axis]) == 0) return false;
+    if ((p->opt.debug & 4) != 0 || f3_radix(p->M[axis]) == 0) return false;
+    // FP32: n = 256 has the register-resident kernels, or the shared-memory engine asked for
+    if (p->opt.precision == GSM_FP32 && (p->M[axis] == 512 || !p->rr_conv)) return false;
     // (a conv inverse in engine order is what plans saved by earlier versions hold)
     const bool f = same_sched(p->sched_f[axis], default_sched(p, axis, false));
     const bool i = same_sched(p->sched_i[axis], default_sched(p, axis, true)) ||
@@ -1381,29 +1399,38 @@ Sched run_sched(const Plan *p, int axis, bool inverse)
 }
 
 // Whether the table made for (M, schedule a) serves (M, schedule b): equal M
-// and, in fixed point (whose tables are in stage order), equal schedules.
+// and, where tables are in stage order, equal schedules.
 bool table_serves(const Plan *p, const Sched &a, const Sched &b)
 {
-    return a.M == b.M && (p->opt.precision == GSM_FP32 || same_sched(a, b));
+    return a.M == b.M && ((p->opt.precision == GSM_FP32 && (f3_radix(a.M) == 0 || a.M == 512)) || same_sched(a, b));
+}
+
+// Entries after the first M of the table of (axis, inverse?), see fill_table:
+// FP32, the stage-ordered ones of the fixed-length kernels; fixed point, the
+// first M / 2 twiddles in order for the split 2D passes.
+int table_plain(const Plan *p, int axis, bool inverse)
+{
+    const int M = p->M[axis];
+    if (p->opt.precision == GSM_FP32) return uses_f3(p, axis, inverse) ? M : 0;
+    return p->d == 2 && M >= kSplitMinM ? M / 2 : 0;
 }
 
 // The table of (axis, inverse?): an existing table that serves it, or a new one.
 gsm_status_t table_for(Plan *p, int axis, bool inverse, cudaStream_t st, void **out)
 {
     const Sched want = run_sched(p, axis, inverse);
+    const int plain = table_plain(p, axis, inverse);
     for (int b = 0; b < p->d; ++b) {
-        if (p->d_tw[b] && table_serves(p, run_sched(p, b, false), want) && !(b == axis && inverse == false)) {
+        if (p->d_tw[b] && table_serves(p, run_sched(p, b, false), want) && table_plain(p, b, false) >= plain && !(b == axis && inverse == false)) {
             *out = p->d_tw[b];
             return GSM_OK;
         }
-        if (p->d_twi[b] && table_serves(p, run_sched(p, b, true), want) && !(b == axis && inverse == true)) {
+        if (p->d_twi[b] && table_serves(p, run_sched(p, b, true), want) && table_plain(p, b, true) >= plain && !(b == axis && inverse == true)) {
             *out = p->d_twi[b];
             return GSM_OK;
         }
     }
     const int M = want.M;
-    // the split 2D passes also need the first M / 2 of the M twiddles in order
-    const int plain = p->d == 2 && M >= kSplitMinM ? M / 2 : 0;
     void *t = nullptr;
     GSM_CUDA_TRY(dev_alloc(&t, plan_table_bytes(p, want, plain)));
     fill_plan_table(p, want, plain, M, t, st);
@@ -1607,6 +1634,14 @@ gsm_status_t x_slabs_t(const Plan *p, bool inverse, int z0, int z1, const void *
         GSM_CUDA_TRY(cudaGetLastError());
         return GSM_OK;
     } else {
+    if constexpr (std::is_same<Pol, F32>::value) {
+        const int pass = inverse ? 4 : 0;
+        if (pass_uses_f3(p, pass)) {
+            launch_f3f(p, pass, static_cast<const io *>(rho_v) + in_off, static_cast<io *>(u_v) + in_off, W1, z1 - z0, st);
+            GSM_CUDA_TRY(cudaGetLastError());
+            return GSM_OK;
+        }
+    }
     if constexpr (std::is_same<Pol, F32>::value) {
         if (p->M[0] == 512 && p->rr_conv) {
             if (!inverse) launch_x_rr512_f32(false, static_cast<const io *>(rho_v) + in_off, W1, ny, z1 - z0, twx, st);
