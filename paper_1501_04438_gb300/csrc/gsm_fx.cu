@@ -1,50 +1,8 @@
 // gsm_fx.cu -- fixed point: the x and y passes, the FFT hook and the tables.
-#include "gsm_fx_passes.cuh"
+#include "gsm_fx_kernels.cuh"
 
 namespace gsm {
 namespace {
-
-// ------------------------------------------------------------------ kernels
-template <int EMAX>
-__global__ void __launch_bounds__(fx_threads(EMAX), fx_ctas(EMAX))
-    k_fx_xf(const double *__restrict__ rho, fxc *__restrict__ W1, FxExps ex, int nx, int ny, int hx, Sched sc, int nl,
-            const int4 *__restrict__ tw)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int red[kFxRedWords];
-    fx_body_xf<EMAX>(fx_thread(), rho, W1, ex, nx, ny, hx, sc, nl, tw, blockIdx.x, blockIdx.y, smem_raw, red);
-}
-
-template <int EMAX>
-__global__ void __launch_bounds__(fx_threads(EMAX), fx_ctas(EMAX))
-    k_fx_yf(const fxc *__restrict__ W1, fxc *__restrict__ W2, FxExps ex, int ny, int nz, int hx, Sched sc, int nl,
-            const int4 *__restrict__ tw)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int red[kFxRedWords];
-    fx_body_yf<EMAX, false>(fx_thread(), W1, W2, ex, ny, nz, hx, sc, nl, tw, blockIdx.x, blockIdx.y, smem_raw, red);
-}
-
-template <int EMAX>
-__global__ void __launch_bounds__(fx_threads(EMAX), fx_ctas(EMAX))
-    k_fx_yi(const fxc *__restrict__ W2, fxc *__restrict__ W1, FxExps ex, int ny, int nz, int hx, Sched sc, int nl,
-            const int4 *__restrict__ tw)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int red[kFxRedWords];
-    fx_body_yi<EMAX, false>(fx_thread(), W2, W1, ex, ny, nz, hx, sc, nl, tw, blockIdx.x, blockIdx.y, smem_raw, red);
-}
-
-template <int EMAX>
-__global__ void __launch_bounds__(fx_threads(EMAX), fx_ctas(EMAX))
-    k_fx_xi(const fxc *__restrict__ W1, double *__restrict__ u, const int *__restrict__ ek, int ek_stride, int nx,
-            int ny, int hx, Sched sc, int nl, const int4 *__restrict__ tw)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int red[kFxRedWords];
-    fx_body_xi<EMAX, false>(fx_thread(), W1, u, ek + (size_t)blockIdx.y * ek_stride, nx, ny, hx, sc, nl, tw, blockIdx.x,
-                            blockIdx.y, smem_raw, red);
-}
 
 // ------------------------------------------------------------------ FFT test hook
 struct FxFromPairs : FxDoubles {
@@ -206,13 +164,14 @@ gsm_status_t make_mult_rows(Plan *p, void *table, int len, size_t rows, cudaStre
 cudaError_t fx_raise_smem(const Plan *p, int pass, const PassCfg &c)
 {
     const int last = p->d == 3 ? 4 : 2;
-    if (pass == (p->d == 3 ? 2 : 1)) return fx_raise_conv_smem(c);
-    cudaError_t e = cudaSuccess;
+    if (pass == (p->d == 3 ? 2 : 1)) return fx_raise_conv_smem(p, c);
+    cudaError_t e = fixed_raise(p, pass, c);
+    if (e != cudaSuccess) return e;
     with_emax(c, [&](auto E) {
-        if (pass == 0) e = raise_smem(k_fx_xf<E()>, c.smem);
-        else if (pass == last) e = raise_smem(k_fx_xi<E()>, c.smem);
-        else if (pass == 1) e = raise_smem(k_fx_yf<E()>, c.smem);
-        else e = raise_smem(k_fx_yi<E()>, c.smem);
+        if (pass == 0) e = raise_smem(k_fx_xf<E(), Sched>, c.smem);
+        else if (pass == last) e = raise_smem(k_fx_xi<E(), Sched>, c.smem);
+        else if (pass == 1) e = raise_smem(k_fx_yf<E(), Sched>, c.smem);
+        else e = raise_smem(k_fx_yi<E(), Sched>, c.smem);
     });
     return e;
 }
@@ -220,6 +179,7 @@ cudaError_t fx_raise_smem(const Plan *p, int pass, const PassCfg &c)
 // x forward (pass 0), y forward (1), y inverse (3), x inverse (the last)
 void fx_launch_xy(const FxCall &a, int pass, const PassCfg &c)
 {
+    if (fixed_launch(a, pass, c)) return;
     const Plan *p = a.p;
     const int nx = p->n[0], ny = p->n[1], nz = a.nz, hx = nx + 1, last = p->d == 3 ? 4 : 2;
     fxc *W1 = static_cast<fxc *>(a.W1), *W2 = static_cast<fxc *>(a.W2);
@@ -228,14 +188,14 @@ void fx_launch_xy(const FxCall &a, int pass, const PassCfg &c)
     const dim3 gx((ny + 2 * c.nl - 1) / (2 * c.nl), nz), gy((nz + c.nl - 1) / c.nl, hx), b = fx_block(c);
     with_emax(c, [&](auto E) {
         if (pass == 0)
-            k_fx_xf<E()><<<gx, b, c.smem, a.st>>>(a.rho, W1, a.ex, nx, ny, hx, p->sched_f[0], c.nl, tw(0));
+            k_fx_xf<E(), Sched><<<gx, b, c.smem, a.st>>>(a.rho, W1, a.ex, nx, ny, hx, p->sched_f[0], c.nl, tw(0));
         else if (pass == last)
-            k_fx_xi<E()><<<gx, b, c.smem, a.st>>>(W1, a.u, p->d == 3 ? a.ex.yi : a.ex.cv, hx, nx, ny, hx, p->sched_i[0],
-                                                  c.nl, twi(0));
+            k_fx_xi<E(), Sched><<<gx, b, c.smem, a.st>>>(W1, a.u, p->d == 3 ? a.ex.yi : a.ex.cv, hx, nx, ny, hx,
+                                                         p->sched_i[0], c.nl, twi(0));
         else if (pass == 1)
-            k_fx_yf<E()><<<gy, b, c.smem, a.st>>>(W1, W2, a.ex, ny, nz, hx, p->sched_f[1], c.nl, tw(1));
+            k_fx_yf<E(), Sched><<<gy, b, c.smem, a.st>>>(W1, W2, a.ex, ny, nz, hx, p->sched_f[1], c.nl, tw(1));
         else
-            k_fx_yi<E()><<<gy, b, c.smem, a.st>>>(W2, W1, a.ex, ny, nz, hx, p->sched_i[1], c.nl, twi(1));
+            k_fx_yi<E(), Sched><<<gy, b, c.smem, a.st>>>(W2, W1, a.ex, ny, nz, hx, p->sched_i[1], c.nl, twi(1));
     });
 }
 

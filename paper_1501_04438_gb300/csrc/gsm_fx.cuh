@@ -320,6 +320,11 @@ GSM_HD int fx_reduce(int v, const Group &g, int *buf)
     const int nw = g.T >> 5, w0 = threadIdx.y * nw;
     if ((g.t & 31) == 0) buf[w0 + (g.t >> 5)] = v;
     group_sync(g);
+    if (nw > 4) {   // one load and one more warp reduction
+        const int lane = g.t & 31;
+        v = lane < nw ? buf[w0 + lane] : MAX ? INT_MIN : 0;
+        return MAX ? __reduce_max_sync(0xffffffffu, v) : (int)__reduce_add_sync(0xffffffffu, (unsigned)v);
+    }
     v = buf[w0];
     for (int i = 1; i < nw; ++i) v = MAX ? max(v, buf[w0 + i]) : (int)((unsigned)v + (unsigned)buf[w0 + i]);
     return v;
@@ -359,13 +364,83 @@ GSM_HD int fx_shift_of(unsigned acc, const FxLine &ln, const Group &g, int *buf)
     return s > 0 ? s : 0;
 }
 
+// ---------------------------------------------------------------- schedules
+// A schedule known at compile time: the default order of make_sched (INV: the
+// fused inverse, the last radix first).  The functions below take it in the
+// place of a Sched; strides, tests, barriers' counts and loops are then
+// constants.
+template <int M_, bool INV = false>
+struct FixedSched {
+    struct List {
+        int n, r[kMaxStages];
+    };
+    static constexpr List list()
+    {
+        List l{};
+        int m = M_;
+        const int order[5] = {8, 4, 2, 5, 3};
+        for (int k = 0; k < 5; ++k)
+            for (; m % order[k] == 0; m /= order[k]) l.r[l.n++] = order[k];
+        if (INV) {
+            const int last = l.r[l.n - 1];
+            for (int i = l.n - 1; i > 0; --i) l.r[i] = l.r[i - 1];
+            l.r[0] = last;
+        }
+        return l;
+    }
+    static constexpr int padding()   // set_pad
+    {
+        const List l = list();
+        int Ns = 1, pad = 3;
+        for (int st = 0; st < l.n; ++st) {
+            if (st > 0 && (M_ / l.r[st]) % 8 != 0) pad = 31;
+            Ns *= l.r[st];
+            if (st + 1 < l.n && 8 % Ns != 0 && Ns % 8 != 0) pad = 31;
+        }
+        return pad;
+    }
+    static constexpr int M = M_, nst = list().n, pad = padding();
+    template <int ST>
+    static constexpr int radix() { return list().r[ST]; }
+    static constexpr int product(int st)   // of the radices before stage st
+    {
+        const List l = list();
+        int Ns = 1;
+        for (int i = 0; i < st; ++i) Ns *= l.r[i];
+        return Ns;
+    }
+    static bool is(const Sched &s)
+    {
+        const List l = list();
+        if (s.M != M || s.nst != nst || s.pad != pad) return false;
+        for (int i = 0; i < nst; ++i)
+            if (s.r[i] != l.r[i]) return false;
+        return true;
+    }
+};
+template <class SC>
+struct is_fixed_sched {
+    static constexpr bool value = true;
+};
+template <>
+struct is_fixed_sched<Sched> {
+    static constexpr bool value = false;
+};
+template <class SC>
+GSM_HD int first_radix(const SC &sc)
+{
+    if constexpr (is_fixed_sched<SC>::value) return SC::template radix<0>();
+    else return sc.r[0];
+}
+
 // ---------------------------------------------------------------- stages
 // First radix of the stage-ordered table: the twiddles of stage st (radix R
 // after stages of product Ns) are exp(-2 pi i j t / (R Ns)), j < Ns, t = 1..R-1,
 // at offset Ns - r0 + (t - 1) Ns + j: consecutive j, the threads of a warp,
 // read consecutive entries (a table indexed by j t scattered them over as many
 // 128-byte lines as threads).  M - r0 entries for the whole transform.
-GSM_HD const int4 *fx_stage_table(const int4 *tw, const Sched &sc, int Ns) { return tw + (Ns - sc.r[0]); }
+template <class SC>
+GSM_HD const int4 *fx_stage_table(const int4 *tw, const SC &sc, int Ns) { return tw + (Ns - first_radix(sc)); }
 
 GSM_HD int fx_mod(int b, int Ns) { return (Ns & (Ns - 1)) == 0 ? (b & (Ns - 1)) : b % Ns; }
 
@@ -388,8 +463,8 @@ GSM_HD int fx_pos(int i, int pad) { return i + (i >> pad); }
 //   out(b, off, v)        takes an output of the transform
 //   Out::kSmem            stores it in the line's own shared memory
 // First stage (radix RAD, untwiddled), HALF = 1: inputs t >= RAD/2 are zero.
-template <int RAD, bool FWD, int NB, int HALF, class In, class Out>
-GSM_HD void fx_first(fxc *s, const Sched &sc, const Group &g, FxLine &ln, In in, Out out)
+template <int RAD, bool FWD, int NB, int HALF, class SC, class In, class Out>
+GSM_HD void fx_first(fxc *s, const SC &sc, const Group &g, FxLine &ln, In in, Out out)
 {
     constexpr int NIN = HALF == 1 ? RAD / 2 : RAD;
     const int nb = sc.M / RAD;
@@ -539,6 +614,20 @@ GSM_HD void fx_stage(fxc *s, int M, int Ns, bool last, const int4 *__restrict__ 
 // The stages [st_begin, st_end) (st_end < 0: to the last) after the first, in
 // the order 8, 4, 2, 5, 3, each radix one loop of its own; the transform's
 // last stage hands its outputs to `out`.
+template <bool FWD, int EMAX, bool CROP, int ST, int END, class SC, class Out>
+GSM_HD void fx_rest_fixed(fxc *s, const int4 *__restrict__ tw, const Group &g, FxLine &ln, Out out)
+{
+    if constexpr (ST < END) {
+        constexpr int RAD = SC::template radix<ST>(), Ns = SC::product(ST);
+        fx_stage<RAD, FWD, (EMAX + RAD - 1) / RAD, CROP>(s, SC::M, Ns, ST == SC::nst - 1, fx_stage_table(tw, SC{}, Ns), g,
+                                                         ln, out);
+        fx_rest_fixed<FWD, EMAX, CROP, ST + 1, END, SC>(s, tw, g, ln, out);
+    }
+}
+// MID: up to the last stage, which is fused with the multiplication
+template <bool FWD, int EMAX, bool CROP, bool MID, class SC, class Out>
+GSM_HD void fx_rest_of(fxc *s, const SC &sc, const int4 *__restrict__ tw, const Group &g, FxLine &ln, Out out);
+
 template <bool FWD, int EMAX, bool CROP, class Out>
 GSM_HD void fx_rest(fxc *s, const Sched &sc, const int4 *__restrict__ tw, const Group &g, FxLine &ln, int st_begin,
                     int st_end, Out out)
@@ -556,37 +645,48 @@ GSM_HD void fx_rest(fxc *s, const Sched &sc, const int4 *__restrict__ tw, const 
     GSM_FX_STAGES(3);
 #undef GSM_FX_STAGES
 }
+template <bool FWD, int EMAX, bool CROP, bool MID, class SC, class Out>
+GSM_HD void fx_rest_of(fxc *s, const SC &sc, const int4 *__restrict__ tw, const Group &g, FxLine &ln, Out out)
+{
+    if constexpr (is_fixed_sched<SC>::value) fx_rest_fixed<FWD, EMAX, CROP, 1, MID ? SC::nst - 1 : SC::nst, SC>(s, tw, g, ln, out);
+    else fx_rest<FWD, EMAX, CROP>(s, sc, tw, g, ln, 1, MID ? sc.nst - 1 : -1, out);
+}
 
 // First stage by the schedule's first radix.  ZPAD: the second half of the
 // line is zero (forward transforms; their first radix is even).
-template <bool FWD, int EMAX, bool ZPAD, class In, class Out>
-GSM_HD void fx_begin(fxc *s, const Sched &sc, const Group &g, FxLine &ln, In in, Out out)
+template <bool FWD, int EMAX, bool ZPAD, class SC, class In, class Out>
+GSM_HD void fx_begin(fxc *s, const SC &sc, const Group &g, FxLine &ln, In in, Out out)
 {
     constexpr int H = ZPAD ? 1 : 0;
-    const int r = sc.r[0];
-    if (r == 8) fx_first<8, FWD, (EMAX + 7) / 8, H>(s, sc, g, ln, in, out);
-    else if (r == 4) fx_first<4, FWD, (EMAX + 3) / 4, H>(s, sc, g, ln, in, out);
-    else if (r == 2) fx_first<2, FWD, (EMAX + 1) / 2, H>(s, sc, g, ln, in, out);
-    else if constexpr (!ZPAD) {
-        if (r == 5) fx_first<5, FWD, (EMAX + 4) / 5, 0>(s, sc, g, ln, in, out);
-        else fx_first<3, FWD, (EMAX + 2) / 3, 0>(s, sc, g, ln, in, out);
+    if constexpr (is_fixed_sched<SC>::value) {
+        constexpr int RAD = SC::template radix<0>();
+        fx_first<RAD, FWD, (EMAX + RAD - 1) / RAD, H>(s, sc, g, ln, in, out);
+    } else {
+        const int r = sc.r[0];
+        if (r == 8) fx_first<8, FWD, (EMAX + 7) / 8, H>(s, sc, g, ln, in, out);
+        else if (r == 4) fx_first<4, FWD, (EMAX + 3) / 4, H>(s, sc, g, ln, in, out);
+        else if (r == 2) fx_first<2, FWD, (EMAX + 1) / 2, H>(s, sc, g, ln, in, out);
+        else if constexpr (!ZPAD) {
+            if (r == 5) fx_first<5, FWD, (EMAX + 4) / 5, 0>(s, sc, g, ln, in, out);
+            else fx_first<3, FWD, (EMAX + 2) / 3, 0>(s, sc, g, ln, in, out);
+        }
     }
 }
 
-template <bool FWD, int EMAX, bool ZPAD, bool CROP, class In, class Out>
-GSM_HD void fx_transform(fxc *s, const Sched &sc, const int4 *__restrict__ tw, const Group &g, FxLine &ln, In in,
+template <bool FWD, int EMAX, bool ZPAD, bool CROP, class SC, class In, class Out>
+GSM_HD void fx_transform(fxc *s, const SC &sc, const int4 *__restrict__ tw, const Group &g, FxLine &ln, In in,
                          Out out)
 {
     ln.pad = sc.pad;
     fx_begin<FWD, EMAX, ZPAD>(s, sc, g, ln, in, out);
-    fx_rest<FWD, EMAX, CROP>(s, sc, tw, g, ln, 1, -1, out);
+    fx_rest_of<FWD, EMAX, CROP, false>(s, sc, tw, g, ln, out);
 }
 
 // The forward's last stage (radix R), the multiplication by mult(k) (entries of
 // a row in units of 2^erow), the scaling of the product and the inverse's
 // first stage, in registers (see fft_fused_mid).
-template <int R, int NB, class MultF>
-GSM_HD void fx_mid(fxc *s, const Sched &scf, const Sched &sci, const int4 *__restrict__ tw, const Group &g, FxLine &ln,
+template <int R, int NB, class SC, class SCI, class MultF>
+GSM_HD void fx_mid(fxc *s, const SC &scf, const SCI &sci, const int4 *__restrict__ tw, const Group &g, FxLine &ln,
                    MultF mult, int erow)
 {
     const int M = scf.M, nb = M / R;
@@ -648,6 +748,24 @@ GSM_HD void fx_mid(fxc *s, const Sched &scf, const Sched &sci, const int4 *__res
         }
     }
     fx_sync(g);
+}
+
+// The same by the inverse's first radix.
+template <int EMAX, class SC, class SCI, class MultF>
+GSM_HD void fx_mid_of(fxc *s, const SC &scf, const SCI &sci, const int4 *__restrict__ tw, const Group &g, FxLine &ln,
+                      MultF mult, int erow)
+{
+    if constexpr (is_fixed_sched<SCI>::value) {
+        constexpr int R = SCI::template radix<0>();
+        fx_mid<R, (EMAX + R - 1) / R>(s, scf, sci, tw, g, ln, mult, erow);
+    } else {
+        const int fr = sci.r[0];
+        if (fr == 8) fx_mid<8, (EMAX + 7) / 8>(s, scf, sci, tw, g, ln, mult, erow);
+        else if (fr == 4) fx_mid<4, (EMAX + 3) / 4>(s, scf, sci, tw, g, ln, mult, erow);
+        else if (fr == 2) fx_mid<2, (EMAX + 1) / 2>(s, scf, sci, tw, g, ln, mult, erow);
+        else if (fr == 5) fx_mid<5, (EMAX + 4) / 5>(s, scf, sci, tw, g, ln, mult, erow);
+        else fx_mid<3, (EMAX + 2) / 3>(s, scf, sci, tw, g, ln, mult, erow);
+    }
 }
 
 // ---------------------------------------------------------------- doubles

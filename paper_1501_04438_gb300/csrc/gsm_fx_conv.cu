@@ -1,22 +1,24 @@
 // gsm_fx_conv.cu -- fixed point: the conv pass and the split passes of long 2D lines.
-#include "gsm_fx_passes.cuh"
+#include "gsm_fx_kernels.cuh"
 
 namespace gsm {
 namespace {
 
-template <int EMAX>
-__global__ void __launch_bounds__(fx_threads(EMAX), fx_ctas(EMAX))
-    k_fx_conv(fxc *__restrict__ W, const int2 *__restrict__ mult, const int *__restrict__ mrow_exp, FxExps ex,
-              int nlines, int n, int is3d, int My, int ny1, Sched sc, Sched sci, int nl,
-              const int4 *__restrict__ tw, const int4 *__restrict__ twi, int full)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int red[kFxRedWords];
-    fx_body_conv<EMAX, false>(fx_thread(), W, mult, mrow_exp, ex, nlines, n, is3d, My, ny1, sc, sci, nl, tw, twi, blockIdx.x,
-                              blockIdx.y, smem_raw, full != 0, red);
-}
-
 // ------------------------------------------------------------------ conv, long 2D lines
+// Threads of a half line and CTAs per SM: a length known at compile time has 8
+// values per thread (64 registers), any other 16.  4096^2 FP64, xf, conv, xi in ms:
+// whole lines 0.390, 1.264, 0.492; halves of any length 0.351, 1.324, 0.418; of a
+// length known at compile time 0.291, 1.037, 0.351 (2048^2: 0.124, 0.363, 0.146 ->
+// 0.074, 0.248, 0.089).  What bounds them is integer issue.
+template <class SC>
+constexpr int split_threads()
+{
+    if constexpr (is_fixed_sched<SC>::value) return SC::M / 8;
+    else return kSplitThreads;
+}
+template <class SC>
+constexpr int split_ctas() { return is_fixed_sched<SC>::value ? 1024 / split_threads<SC>() : 2; }
+
 // A conv line of padded length M = 2 Mh holds Mh values x and zeros; its even
 // and odd frequencies are two transforms of length Mh, X[2k] = FFT_Mh(x)[k],
 // X[2k + 1] = FFT_Mh(x w_M^n)[k], and the cropped inverse is
@@ -61,10 +63,10 @@ struct FxMultHalf {   // output k' of a half is frequency 2 k' + rank
     __device__ __forceinline__ int2 at(int b, int t, int nb) const { return m(2 * (b + t * nb) + rank); }
 };
 
-template <int EMAX>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSplitThreads, 2)
+template <int EMAX, class SC, class SCI>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<SC>(), split_ctas<SC>())
     k_fx_conv_split(fxc *__restrict__ W, const int2 *__restrict__ mult, const int *__restrict__ mrow_exp, FxExps ex,
-                    int nlines, int ny1, Sched sc, Sched sci, const int4 *__restrict__ tw,
+                    int nlines, int ny1, SC sc, SCI sci, const int4 *__restrict__ tw,
                     const int4 *__restrict__ twi, const int4 *__restrict__ twM, int full)
 {
     namespace cg = cooperative_groups;
@@ -75,7 +77,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSplitThreads, 2)
     const int rank = (int)cl.block_rank();
     const int line = blockIdx.x >> 1;
     const int Mh = sc.M, M = 2 * Mh;
-    const Group g = fx_thread().g;
+    const Group g = fx_thread_of<SC>().g;
     fxc *s = reinterpret_cast<fxc *>(smem_raw);
     fxc *w = W + (size_t)line * Mh;
     const bool active = line < nlines;   // every CTA of a cluster reaches both cluster barriers
@@ -90,15 +92,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSplitThreads, 2)
         // the half's schedules always fuse (make_split_tables)
         ln.pad = sc.pad;
         fx_begin<true, EMAX, false>(s, sc, g, ln, in, FxNoOut{});
-        fx_rest<true, EMAX, false>(s, sc, tw, g, ln, 1, sc.nst - 1, FxNoOut{});
-        const FxMultHalf mh{m, rank};
-        const int fr = sci.r[0], er = mrow_exp[line];
-        if (fr == 8) fx_mid<8, (EMAX + 7) / 8>(s, sc, sci, tw, g, ln, mh, er);
-        else if (fr == 4) fx_mid<4, (EMAX + 3) / 4>(s, sc, sci, tw, g, ln, mh, er);
-        else if (fr == 2) fx_mid<2, (EMAX + 1) / 2>(s, sc, sci, tw, g, ln, mh, er);
-        else if (fr == 5) fx_mid<5, (EMAX + 4) / 5>(s, sc, sci, tw, g, ln, mh, er);
-        else fx_mid<3, (EMAX + 2) / 3>(s, sc, sci, tw, g, ln, mh, er);
-        fx_rest<false, EMAX, false>(s, sci, twi, g, ln, 1, -1, FxHalfToSmem{s, twM, rank});
+        fx_rest_of<true, EMAX, false, true>(s, sc, tw, g, ln, FxNoOut{});
+        fx_mid_of<EMAX>(s, sc, sci, tw, g, ln, FxMultHalf{m, rank}, mrow_exp[line]);
+        fx_rest_of<false, EMAX, false, false>(s, sci, twi, g, ln, FxHalfToSmem{s, twM, rank});
         if (threadIdx.x == 0) line_e = ln.E;
     }
     cl.sync();   // both halves transformed
@@ -142,16 +138,16 @@ struct FxFromRowsRot : FxDoubles {
     }
 };
 
-template <int EMAX>
-__global__ void __launch_bounds__(kSplitThreads, 2)
-    k_fx_xf_split(const double *__restrict__ rho, fxc *__restrict__ W1, FxExps ex, int nx, int ny, Sched sc,
+template <int EMAX, class SC>
+__global__ void __launch_bounds__(split_threads<SC>(), split_ctas<SC>())
+    k_fx_xf_split(const double *__restrict__ rho, fxc *__restrict__ W1, FxExps ex, int nx, int ny, SC sc,
                   const int4 *__restrict__ tw, const int4 *__restrict__ twM)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int red[kFxRedWords];
     const int rank = blockIdx.x & 1, ya = 2 * (blockIdx.x >> 1);
     const int Mh = sc.M;   // == nx
-    const Group g = fx_thread().g;
+    const Group g = fx_thread_of<SC>().g;
     fxc *s = reinterpret_cast<fxc *>(smem_raw);
     FxLine ln{0, 0, Mh > kFxLongM, red};
     FxFromRowsRot in;
@@ -177,52 +173,163 @@ __global__ void __launch_bounds__(kSplitThreads, 2)
     }
 }
 
+// ------------------------------------------------------------------ x inverse, long 2D lines
+// The halves of the inverse x line (two real rows), on a cluster of two CTAs as
+// in the conv: the Hermitian fill pairs Z[k] with Z[M - k], of the parity of k,
+// so each CTA reads the rows of its own parity only; the halves of the cropped
+// line are added through distributed shared memory, and each CTA stores one
+// half of both rows.
+struct FxFromSmemHalf : FxInts {   // element i of a half is frequency 2 i + rank
+    const fxc *s;
+    const int *e;
+    int M, rank, pad;
+    __device__ __forceinline__ raw load(int b, int off) const
+    {
+        const int i = b + off, f = 2 * i + rank;
+        return {s[fx_pos(i, pad)], e[min(f, M - f)]};
+    }
+};
+
+template <int EMAX, class SC>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<SC>(), split_ctas<SC>())
+    k_fx_xi_split(const fxc *__restrict__ W1, double *__restrict__ u, const int *__restrict__ ek, int nx, int ny,
+                  SC sc, const int4 *__restrict__ tw, const int4 *__restrict__ twM)
+{
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int red[kFxRedWords];
+    __shared__ int line_e;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), ya = 2 * (blockIdx.x >> 1);   // ya < ny
+    const int Mh = sc.M, M = 2 * Mh;   // Mh == nx, even
+    const Group g = fx_thread_of<SC>().g;
+    const bool two = ya + 1 < ny;
+    fxc *s = reinterpret_cast<fxc *>(smem_raw);
+    struct AB {
+        longlong2 a, b;
+    };
+    // the frequencies k = 2 k' + rank <= nx; M - k sits at Mh - k' - rank
+    gather_smem<4, AB>(
+        (int)threadIdx.x, (int)blockDim.x, rank ? nx / 2 : nx / 2 + 1,
+        [&](int kp) {
+            const longlong2 *q = reinterpret_cast<const longlong2 *>(W1 + (size_t)(2 * kp + rank) * ny + ya);
+            AB v{q[0], {0, 0}};
+            if (two) v.b = q[1];
+            return v;
+        },
+        [&](int kp, const AB &v) {
+            const int k = 2 * kp + rank;
+            const bool real = k == 0 || k == nx;
+            const long long ai = real ? 0 : v.a.y, bi = real ? 0 : v.b.y;
+            s[fx_pos(kp, sc.pad)] = {rsub(v.a.x, bi), radd(ai, v.b.x)};
+            if (!real) s[fx_pos(Mh - kp - rank, sc.pad)] = {radd(v.a.x, bi), rsub(v.b.x, ai)};
+        });
+    __syncthreads();
+    FxLine ln{0, 0, Mh > kFxLongM, red};
+    FxFromSmemHalf in;
+    in.s = s;
+    in.e = ek;
+    in.M = M;
+    in.rank = rank;
+    in.pad = sc.pad;
+    fx_transform<false, EMAX, false, false>(s, sc, tw, g, ln, in, FxHalfToSmem{s, twM, rank});
+    if (threadIdx.x == 0) line_e = ln.E;
+    cl.sync();   // both halves transformed
+    const fxc *peer = cl.map_shared_rank(s, rank ^ 1);
+    const int e0 = line_e, e1 = *cl.map_shared_rank(&line_e, rank ^ 1);
+    const int e = max(e0, e1) + 1, d0 = min(e - e0, 62), d1 = min(e - e1, 62);
+    const int h = Mh / 2;
+    double *row = u + (size_t)ya * nx;
+    for (int i = threadIdx.x; i < h; i += blockDim.x) {
+        const int n = rank * h + i, p = pidx<FX>(n);
+        const cx<long long> v = fx_add(fx_shift(fx_ld(s[p]), d0), fx_shift(fx_ld(peer[p]), d1));
+        row[n] = fx_out_double(v.re, e);
+        if (two) row[nx + n] = fx_out_double(v.im, e);
+    }
+    cl.sync();   // the peer has read this CTA's half: its shared memory may go
+}
+
+// Calls f(EMAX, forward, inverse) with the types and values that a half line's
+// kernels are launched with: schedules known at compile time for 4096 and 2048.
+template <class F>
+void with_split(const Plan *p, const Sched &f, const Sched *i, F &&fn)
+{
+    const bool fixed = (p->opt.debug & 4) == 0;
+    using E8 = std::integral_constant<int, 8>;
+    if (fixed && FixedSched<4096>::is(f) && (!i || FixedSched<4096, true>::is(*i))) fn(E8(), FixedSched<4096>(), FixedSched<4096, true>());
+    else if (fixed && FixedSched<2048>::is(f) && (!i || FixedSched<2048, true>::is(*i))) fn(E8(), FixedSched<2048>(), FixedSched<2048, true>());
+    else fn(std::integral_constant<int, 16>(), f, i ? *i : f);
+}
+template <class SC>
+int split_block(const PassCfg &c) { return is_fixed_sched<SC>::value ? split_threads<SC>() : c.nthr; }
 }  // namespace
 
-cudaError_t fx_raise_conv_smem(const PassCfg &c)
+cudaError_t fx_raise_conv_smem(const Plan *p, const PassCfg &c)
 {
-    cudaError_t e = cudaSuccess;
-    with_emax(c, [&](auto E) { e = raise_smem(k_fx_conv<E()>, c.smem); });
+    cudaError_t e = fixed_raise(p, p->d == 3 ? 2 : 1, c);
+    with_emax(c, [&](auto E) { if (e == cudaSuccess) e = raise_smem(k_fx_conv<E(), Sched, Sched>, c.smem); });
     return e;
 }
 
 cudaError_t fx_raise_split_smem(bool conv, size_t smem)
 {
-    return conv ? raise_smem(k_fx_conv_split<16>, smem) : raise_smem(k_fx_xf_split<16>, smem);
+    cudaError_t e = cudaSuccess;
+    auto raise = [&](auto E, auto sc, auto sci) {
+        using SC = decltype(sc);
+        using SCI = decltype(sci);
+        if (conv) {
+            if (e == cudaSuccess) e = raise_smem(k_fx_conv_split<E(), SC, SCI>, smem);
+        } else {
+            if (e == cudaSuccess) e = raise_smem(k_fx_xf_split<E(), SC>, smem);
+            if (e == cudaSuccess) e = raise_smem(k_fx_xi_split<E(), SC>, smem);
+        }
+    };
+    raise(std::integral_constant<int, 16>(), Sched(), Sched());
+    if (smem == pass_smem<FX>(4096, 1)) raise(std::integral_constant<int, 8>(), FixedSched<4096>(), FixedSched<4096, true>());
+    if (smem == pass_smem<FX>(2048, 1)) raise(std::integral_constant<int, 8>(), FixedSched<2048>(), FixedSched<2048, true>());
+    return e;
 }
 
 void fx_launch_conv(const FxCall &a, const PassCfg &c)
 {
     const Plan *p = a.p;
+    if (fixed_launch(a, p->d == 3 ? 2 : 1, c)) return;
     const int z = p->d - 1, ny = p->n[1], hx = p->n[0] + 1, My = p->d == 3 ? p->M[1] : 1;
     const int2 *mult = static_cast<const int2 *>(p->d_mult);
     const int4 *tw = static_cast<const int4 *>(p->d_tw[z]), *twi = static_cast<const int4 *>(p->d_twi[z]);
     fxc *W = static_cast<fxc *>(p->d == 3 ? a.W2 : a.W1);
     const dim3 g = p->d == 3 ? dim3((My + c.nl - 1) / c.nl, hx) : dim3((hx + c.nl - 1) / c.nl), b(c.gthr, c.nl);
     with_emax(c, [&](auto E) {
-        k_fx_conv<E()><<<g, b, c.smem, a.st>>>(W, mult, p->d_mrow, a.ex, p->d == 3 ? hx * My : hx, p->n[z], p->d == 3,
-                                               My, ny + 1, p->sched_f[z], p->sched_i[z], c.nl, tw, twi,
-                                               p->mult_full ? 1 : 0);
+        k_fx_conv<E(), Sched, Sched><<<g, b, c.smem, a.st>>>(
+            W, mult, p->d_mrow, a.ex, p->d == 3 ? hx * My : hx, p->n[z], p->d == 3, My, ny + 1, p->sched_f[z],
+            p->sched_i[z], c.nl, tw, twi, p->mult_full ? 1 : 0);
     });
 }
 
-// The split conv (conv) or the split x forward pass of a 2D plan.
-void fx_launch_split(const FxCall &a, bool conv)
+// A split pass (0 xf, 1 conv, 2 xi) of a 2D plan.
+void fx_launch_split(const FxCall &a, int pass)
 {
     const Plan *p = a.p;
+    const bool conv = pass == 1;
     const int nx = p->n[0], ny = p->n[1], hx = nx + 1;
     fxc *W1 = static_cast<fxc *>(a.W1);
     const int4 *twM = static_cast<const int4 *>(p->d_tw[conv ? 1 : 0]) + p->M[conv ? 1 : 0];   // the plain entries
-    if (conv) {
-        const PassCfg &c = p->cfg_split;
-        k_fx_conv_split<16><<<2 * hx, c.nthr, c.smem, a.st>>>(
-            W1, static_cast<const int2 *>(p->d_mult), p->d_mrow, a.ex, hx, ny + 1, p->sched_hf, p->sched_hi,
-            static_cast<const int4 *>(p->d_twh), static_cast<const int4 *>(p->d_twhi), twM, p->mult_full ? 1 : 0);
-    } else {
-        const PassCfg &c = p->cfg_xsplit;
-        k_fx_xf_split<16><<<2 * ((ny + 1) / 2), c.nthr, c.smem, a.st>>>(
-            a.rho, W1, a.ex, nx, ny, p->sched_xh, static_cast<const int4 *>(p->d_twxh), twM);
-    }
+    const PassCfg &c = conv ? p->cfg_split : p->cfg_xsplit;
+    const Sched &f = conv ? p->sched_hf : p->sched_xh;
+    with_split(p, f, conv ? &p->sched_hi : nullptr, [&](auto E, auto sc, auto sci) {
+        using SC = decltype(sc);
+        using SCI = decltype(sci);
+        const int b = split_block<SC>(c);
+        const int4 *tw = static_cast<const int4 *>(conv ? p->d_twh : p->d_twxh);
+        if (conv)
+            k_fx_conv_split<E(), SC, SCI><<<2 * hx, b, c.smem, a.st>>>(
+                W1, static_cast<const int2 *>(p->d_mult), p->d_mrow, a.ex, hx, ny + 1, sc, sci, tw,
+                static_cast<const int4 *>(p->d_twhi), twM, p->mult_full ? 1 : 0);
+        else if (pass == 0)
+            k_fx_xf_split<E(), SC><<<2 * ((ny + 1) / 2), b, c.smem, a.st>>>(a.rho, W1, a.ex, nx, ny, sc, tw, twM);
+        else
+            k_fx_xi_split<E(), SC><<<2 * ((ny + 1) / 2), b, c.smem, a.st>>>(W1, a.u, a.ex.cv, nx, ny, sc, tw, twM);
+    });
 }
 
 }  // namespace gsm

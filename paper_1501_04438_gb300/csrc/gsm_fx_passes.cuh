@@ -44,6 +44,19 @@ __device__ __forceinline__ FxThread fx_thread()
     th.tid = threadIdx.y * blockDim.x + threadIdx.x;
     return th;
 }
+// the same for a schedule known at compile time: 8 values per thread
+template <class SC>
+constexpr int fixed_threads() { return ((SC::M + 7) / 8 + 31) / 32 * 32; }
+template <class SC>
+__device__ __forceinline__ FxThread fx_thread_of()
+{
+    FxThread th = fx_thread();
+    if constexpr (is_fixed_sched<SC>::value) {
+        th.g.T = fixed_threads<SC>();
+        if (fixed_threads<SC>() == 32) th.g.bar = -1;
+    }
+    return th;
+}
 // one warp per line in a one-dimensional CTA
 __device__ __forceinline__ FxThread fx_warp_line()
 {
@@ -140,9 +153,9 @@ __device__ __forceinline__ void fx_copy_wait()
 }
 
 // ------------------------------------------------------------------ x forward
-template <int EMAX>
+template <int EMAX, class SC>
 __device__ __forceinline__ void fx_body_xf(const FxThread &th, const double *__restrict__ rho, fxc *__restrict__ W1, const FxExps &ex,
-                                           int nx, int ny, int hx, const Sched &sc, int nl,
+                                           int nx, int ny, int hx, const SC &sc, int nl,
                                            const int4 *__restrict__ tw, int bx, int by, unsigned char *smem_raw,
                                            int *red)
 {
@@ -177,9 +190,9 @@ __device__ __forceinline__ void fx_body_xf(const FxThread &th, const double *__r
 }
 
 // ------------------------------------------------------------------ y forward
-template <int EMAX, bool CG>
+template <int EMAX, bool CG, class SC>
 __device__ __forceinline__ void fx_body_yf(const FxThread &th, const fxc *__restrict__ W1, fxc *__restrict__ W2, const FxExps &ex, int ny,
-                                           int nz, int hx, const Sched &sc, int nl,
+                                           int nz, int hx, const SC &sc, int nl,
                                            const int4 *__restrict__ tw, int bx, int by, unsigned char *smem_raw,
                                            int *red)
 {
@@ -236,24 +249,21 @@ struct FxMulToSmem {
 
 // Forward, multiplication and inverse of the line whose inputs `in` gives;
 // the outputs go to `out`.
-template <int EMAX, bool ZPAD, bool CROP, class In, class MultF, class MulOut, class Out>
-__device__ __forceinline__ void fx_convolve(fxc *s, const Sched &sc, const Sched &sci, const int4 *__restrict__ tw,
+template <int EMAX, bool ZPAD, bool CROP, class SC, class SCI, class In, class MultF, class MulOut, class Out>
+__device__ __forceinline__ void fx_convolve(fxc *s, const SC &sc, const SCI &sci, const int4 *__restrict__ tw,
                                             const int4 *__restrict__ twi, const Group &g, FxLine &ln, In in,
                                             MultF mult, int erow, MulOut mul_out, Out out)
 {
-    const int fr = fused_radix(sc, sci);
+    bool fused = true;
+    if constexpr (!is_fixed_sched<SC>::value) fused = fused_radix(sc, sci) != 0;
     ln.pad = sc.pad;
     fx_begin<true, EMAX, ZPAD>(s, sc, g, ln, in, mul_out);
-    if (fr != 0) {
-        fx_rest<true, EMAX, false>(s, sc, tw, g, ln, 1, sc.nst - 1, FxNoOut{});
-        if (fr == 8) fx_mid<8, (EMAX + 7) / 8>(s, sc, sci, tw, g, ln, mult, erow);
-        else if (fr == 4) fx_mid<4, (EMAX + 3) / 4>(s, sc, sci, tw, g, ln, mult, erow);
-        else if (fr == 2) fx_mid<2, (EMAX + 1) / 2>(s, sc, sci, tw, g, ln, mult, erow);
-        else if (fr == 5) fx_mid<5, (EMAX + 4) / 5>(s, sc, sci, tw, g, ln, mult, erow);
-        else fx_mid<3, (EMAX + 2) / 3>(s, sc, sci, tw, g, ln, mult, erow);
-        fx_rest<false, EMAX, CROP>(s, sci, twi, g, ln, 1, -1, out);
-    } else {
-        fx_rest<true, EMAX, false>(s, sc, tw, g, ln, 1, -1, mul_out);
+    if (fused) {
+        fx_rest_of<true, EMAX, false, true>(s, sc, tw, g, ln, FxNoOut{});
+        fx_mid_of<EMAX>(s, sc, sci, tw, g, ln, mult, erow);
+        fx_rest_of<false, EMAX, CROP, false>(s, sci, twi, g, ln, out);
+    } else if constexpr (!is_fixed_sched<SC>::value) {
+        fx_rest_of<true, EMAX, false, false>(s, sc, tw, g, ln, mul_out);
         group_sync(g);
         FxFromSmem<false> back;
         back.s = s;
@@ -265,10 +275,10 @@ __device__ __forceinline__ void fx_convolve(fxc *s, const Sched &sc, const Sched
     }
 }
 
-template <int EMAX, bool CG>
+template <int EMAX, bool CG, class SC, class SCI>
 __device__ __forceinline__ void fx_body_conv(const FxThread &th, fxc *__restrict__ W, const int2 *__restrict__ mult,
                                              const int *__restrict__ mrow_exp, const FxExps &ex, int nlines, int n,
-                                             int is3d, int My, int ny1, const Sched &sc, const Sched &sci, int nl,
+                                             int is3d, int My, int ny1, const SC &sc, const SCI &sci, int nl,
                                              const int4 *__restrict__ tw, const int4 *__restrict__ twi,
                                              int bx, int by, unsigned char *smem_raw, bool full, int *red)
 {
@@ -300,9 +310,9 @@ __device__ __forceinline__ void fx_body_conv(const FxThread &th, fxc *__restrict
 }
 
 // ------------------------------------------------------------------ y inverse
-template <int EMAX, bool CG>
+template <int EMAX, bool CG, class SC>
 __device__ __forceinline__ void fx_body_yi(const FxThread &th, const fxc *__restrict__ W2, fxc *__restrict__ W1, const FxExps &ex, int ny,
-                                           int nz, int hx, const Sched &sc, int nl,
+                                           int nz, int hx, const SC &sc, int nl,
                                            const int4 *__restrict__ tw, int bx, int by, unsigned char *smem_raw,
                                            int *red)
 {
@@ -336,9 +346,9 @@ __device__ __forceinline__ void fx_body_yi(const FxThread &th, const fxc *__rest
 
 // ------------------------------------------------------------------ x inverse
 // ek: exponents of the kx rows of this slab (3D: yi[z], 2D: cv)
-template <int EMAX, bool CG>
+template <int EMAX, bool CG, class SC>
 __device__ __forceinline__ void fx_body_xi(const FxThread &th, const fxc *__restrict__ W1, double *__restrict__ u,
-                                           const int *__restrict__ ek, int nx, int ny, int hx, const Sched &sc, int nl,
+                                           const int *__restrict__ ek, int nx, int ny, int hx, const SC &sc, int nl,
                                            const int4 *__restrict__ tw, int bx, int by,
                                            unsigned char *smem_raw, int *red)
 {

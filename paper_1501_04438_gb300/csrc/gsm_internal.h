@@ -76,8 +76,8 @@ struct Plan {
     Sched sched_hf, sched_hi;
     void *d_twh = nullptr, *d_twhi = nullptr;   // tables of the half length
     PassCfg cfg_split;
-    // 2D x forward pass of padded length >= kSplitMinM: each line as two
-    // half-length transforms on two CTAs (k_xf_split)
+    // 2D x passes of padded length >= kSplitMinM: each line as two half-length
+    // transforms on two CTAs (k_xf_split, k_fx_xf_split, k_fx_xi_split)
     bool split_x = false;
     Sched sched_xh;                 // length M[0] / 2
     void *d_twxh = nullptr;         // its tables
@@ -147,11 +147,11 @@ struct FxCall {
 // limits of their kernels; twiddle tables (gsm_fx.cu, gsm_fx_conv.cu).
 void fx_launch_xy(const FxCall &c, int pass, const PassCfg &cfg);
 void fx_launch_conv(const FxCall &c, const PassCfg &cfg);
-void fx_launch_split(const FxCall &c, bool conv);
+void fx_launch_split(const FxCall &c, int pass);
 cudaError_t fx_launch_hook(const PassCfg &c, int nlines, int sign, const Sched &sc, const double *in, double *out,
                            const void *tw, cudaStream_t st);
 cudaError_t fx_raise_smem(const Plan *p, int pass, const PassCfg &c);
-cudaError_t fx_raise_conv_smem(const PassCfg &c);
+cudaError_t fx_raise_conv_smem(const Plan *p, const PassCfg &c);
 cudaError_t fx_raise_split_smem(bool conv, size_t smem);
 // the passes of padded lengths 64 R, R = 1, 2, 3, 4, 5, 6, 8 (gsm_fx3.cuh)
 template <int R>

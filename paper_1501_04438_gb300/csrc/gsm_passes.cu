@@ -731,6 +731,7 @@ gsm_status_t configure_t(Plan *p)
 // One pass of the apply: 3D passes 0..4 = xf, yf, conv, yi, xi; 2D 0..2 = xf, conv, xi.
 PassCfg *pass_cfg(Plan *p, int pass);
 bool pass_uses_f3(const Plan *p, int pass);
+bool pass_is_split(const Plan *p, int pass);
 int f3_radix(int M);
 int pass_len(const Plan *p, int pass);
 // Calls f(std::integral_constant<int, R>) with the R of padded length M.
@@ -875,8 +876,7 @@ void launch_pass_fx(const Plan *p, int pass, const void *rho, void *u, cudaStrea
                    p->d_work2, p->d == 3 ? p->n[2] : 1, st};
     const int conv = p->d == 3 ? 2 : 1;
     if (pass_uses_f3(p, pass)) with_f3(pass_len(p, pass), [&](auto R) { f3_launch<R()>(c, pass); });
-    else if (pass == conv && p->split_conv) fx_launch_split(c, true);
-    else if (pass == 0 && p->split_x) fx_launch_split(c, false);
+    else if (pass_is_split(p, pass)) fx_launch_split(c, pass);
     else if (pass == conv) fx_launch_conv(c, p->cfg_conv);
     else fx_launch_xy(c, pass, *pass_cfg(const_cast<Plan *>(p), pass));
 }
@@ -1006,10 +1006,16 @@ bool pass_uses_rr(const Plan *p, int pass)
     return p->opt.precision == GSM_FP32 && p->rr_conv && p->M[axis] == 512;
 }
 
-// The split 2D passes have a fixed launch shape and half-length schedules of their own.
+// The split 2D passes have a fixed launch shape and half-length schedules of
+// their own.  The inverse x pass is split in fixed point only (a whole FP32 line
+// takes half the shared memory), and not with a schedule that was set or tuned.
 bool pass_is_split(const Plan *p, int pass)
 {
-    return p->d == 2 && ((pass == 1 && p->split_conv) || (pass == 0 && p->split_x));
+    if (p->d != 2) return false;
+    Sched def;
+    if (pass == 2)
+        return p->split_x && p->opt.precision != GSM_FP32 && make_sched(p->M[0], &def) && same_sched(p->sched_i[0], def);
+    return pass == 1 ? p->split_conv : p->split_x;
 }
 
 // Factorisations of M into radices 8, 4, 2, 5, 3 in the order fft_line runs

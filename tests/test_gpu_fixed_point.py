@@ -124,3 +124,33 @@ def test_fixed_length_kernels(gsm, N, role, precision):
         uo, _ = oracle.apply(kernel, r.double().cpu().numpy(), 4.0, taylor_mode=1, **kw)
         bound = unit * np.log2(2 * max(n)) if precision == "fp32" else 1e-12
         assert np.max(np.abs(u - uo)) / np.max(np.abs(uo)) < bound
+
+
+# every length whose default schedule is compiled in, as x, y and z lines of grids whose other axes
+# have none, with the octant and (general dipole axes) the half-spectrum multiplier; n = 216 has none
+COMPILED = [24, 30, 36, 40, 48, 50, 54, 60, 72, 80, 90, 100, 108, 120, 144, 150, 162, 180, 200, 216, 240, 250]
+LONG = [(512, 18), (18, 512), (1024, 10), (10, 1024), (2048, 18), (18, 2048), (4096, 10), (12, 4096)]
+CASES = ([("coulomb3d", s) for N in COMPILED for s in ((N, 10, 18), (10, N, 18), (10, 18, N))] +
+         [("dipolar3d", (10, 18, N)) for N in COMPILED] + [("ds2d", s) for s in LONG])
+
+
+@pytest.mark.parametrize("kernel,n", CASES, ids=[k[0] + "x".join(map(str, s)) for k, s in CASES])
+def test_schedules_known_at_compile_time(gsm, kernel, n):
+    """The kernels of a compiled-in schedule run the integer operations of the kernels of any
+    schedule (options.debug bit 2) in the same order: equal bits."""
+    import torch
+    kw = dict(dip_n=(0.6, 0.0, 0.8), dip_m=(0.0, 0.8, 0.6)) if kernel == "dipolar3d" else {}
+    r = torch.tensor(np.random.default_rng(sum(n)).standard_normal(n[::-1]), device="cuda")
+    assert torch.equal(gsm.Plan(kernel, 4.0, n, **kw).apply(r), gsm.Plan(kernel, 4.0, n, debug=4, **kw).apply(r))
+
+
+@pytest.mark.parametrize("n", [(2048, 18), (2160, 10), (4096, 10)], ids=lambda n: "x".join(map(str, n)))
+def test_split_inverse_x(gsm, n):
+    """Long x lines as two halves on a CTA pair against whole lines (debug bit 1): a few roundings of
+    the result, u log2 of the padded size."""
+    import torch
+    r = torch.tensor(np.random.default_rng(n[0]).standard_normal(n[::-1]), device="cuda")
+    u = gsm.Plan("coulomb2d", 4.0, n).apply(r)
+    for debug in (2, 6):
+        v = gsm.Plan("coulomb2d", 4.0, n, debug=debug).apply(r)
+        assert float((u - v).abs().max() / v.abs().max()) < 2.0 ** -53 * np.log2(4.0 * n[0] * n[1])
