@@ -44,14 +44,17 @@ __device__ __forceinline__ void body_xf(const typename Pol::io_t *__restrict__ r
     const int ya = y0 + 2 * l;
     const typename Pol::io_t *slab = rho + (size_t)z * ny * nx;
     // x >= nx is zero padding
-    for (int x = g.t; x < M; x += g.T) {
-        R a = Pol::zero(), b = Pol::zero();
-        if (x < nx) {
-            if (ya < ny) a = Pol::from_io(slab[(size_t)ya * nx + x]);
-            if (ya + 1 < ny) b = Pol::from_io(slab[(size_t)(ya + 1) * nx + x]);
-        }
-        s[pidx<Pol>(x)] = Pol::st(cx<R>{a, b});
-    }
+    gather_smem<4, cx<R>>(
+        g.t, g.T, M,
+        [&](int x) {
+            cx<R> v{Pol::zero(), Pol::zero()};
+            if (x < nx) {
+                if (ya < ny) v.re = Pol::from_io(slab[(size_t)ya * nx + x]);
+                if (ya + 1 < ny) v.im = Pol::from_io(slab[(size_t)(ya + 1) * nx + x]);
+            }
+            return v;
+        },
+        [&](int x, const cx<R> &v) { s[pidx<Pol>(x)] = Pol::st(v); });
     group_sync(g);
     fft_line<Pol, true, EMAX>(s, sc, tw, g);
     __syncthreads();
@@ -60,11 +63,11 @@ __device__ __forceinline__ void body_xf(const typename Pol::io_t *__restrict__ r
     // is removed by the multiplier.
     const S_t<Pol> *s0 = reinterpret_cast<const S_t<Pol> *>(smem_raw);
     S_t<Pol> *out = W1 + (size_t)z * hx * ny;
-    for (int i = threadIdx.x; i < hx * nl; i += blockDim.x) {
-        const int k = i / nl, ll = i - k * nl;
+    // (a thread keeps its line: the CTA's nl gthr threads are whole rows of nl)
+    const int ll = threadIdx.x % nl, yy = y0 + 2 * ll;
+    for (int k = threadIdx.x / nl; k < hx; k += gthr) {
         const cx<R> zk = Pol::ld(s0[ll * LS + pidx<Pol>(k)]);
         const cx<R> zm = cconj(Pol::ld(s0[ll * LS + pidx<Pol>(k == 0 ? 0 : M - k)]));
-        const int yy = y0 + 2 * ll;
         if (yy < ny) out[(size_t)k * ny + yy] = Pol::st(cadd(zk, zm));
         if (yy + 1 < ny) out[(size_t)k * ny + yy + 1] = Pol::st(cmul_negi(csub(zk, zm)));
     }
@@ -95,7 +98,7 @@ __device__ __forceinline__ void body_yf(const S_t<Pol> *__restrict__ W1, S_t<Pol
     const int z0 = bx * nl;
     const int z = z0 + l;
     const S_t<Pol> *in = W1 + ((size_t)z * hx + kx) * ny;
-    gather_smem<1, S_t<Pol>>(   // y >= ny: zero padding
+    gather_smem<4, S_t<Pol>>(   // y >= ny: zero padding
         g.t, g.T, M,
         [&](int y) {
             S_t<Pol> v = Pol::st(cx<R>{Pol::zero(), Pol::zero()});
@@ -108,11 +111,9 @@ __device__ __forceinline__ void body_yf(const S_t<Pol> *__restrict__ W1, S_t<Pol
     __syncthreads();
     const S_t<Pol> *s0 = reinterpret_cast<const S_t<Pol> *>(smem_raw);
     S_t<Pol> *out = W2 + (size_t)kx * M * nz;
-    for (int i = threadIdx.x; i < M * nl; i += blockDim.x) {
-        const int ky = i / nl, ll = i - ky * nl;
-        const int zz = z0 + ll;
-        if (zz < nz) out[(size_t)ky * nz + zz] = s0[ll * LS + pidx<Pol>(ky)];
-    }
+    const int ll = threadIdx.x % nl, zz = z0 + ll;
+    if (zz < nz)
+        for (int ky = threadIdx.x / nl; ky < M; ky += gthr) out[(size_t)ky * nz + zz] = s0[ll * LS + pidx<Pol>(ky)];
 }
 
 template <class Pol, int EMAX>
@@ -146,11 +147,9 @@ __device__ __forceinline__ void body_conv(S_t<Pol> *__restrict__ W, const typena
     const int line = bx * nl + l;
     if (line >= nlines) return;   // the whole group leaves; no CTA barrier follows
     S_t<Pol> *w = W + (size_t)line * n;
-    for (int z = g.t; z < M; z += g.T) {   // z >= n: zero padding
-        S_t<Pol> v = Pol::st(cx<R>{Pol::zero(), Pol::zero()});
-        if (z < n) v = ldw<CG>(w + z);
-        s[pidx<Pol>(z)] = v;
-    }
+    gather_smem<4, S_t<Pol>>(   // z >= n: zero padding
+        g.t, g.T, M, [&](int z) { return z < n ? ldw<CG>(w + z) : Pol::st(cx<R>{Pol::zero(), Pol::zero()}); },
+        [&](int z, const S_t<Pol> &v) { s[pidx<Pol>(z)] = v; });
     group_sync(g);
     // multiplier of frequency k: the whole half spectrum is stored (full), or
     // the octant, read at min(k, M - k) (the multiplier is even)
@@ -215,18 +214,11 @@ __device__ __forceinline__ void body_yi(const S_t<Pol> *__restrict__ W2, S_t<Pol
     const int kx = by;
     const int z0 = bx * nl;
     const S_t<Pol> *in = W2 + (size_t)kx * M * nz;
-    gather_smem<1, S_t<Pol>>(
-        threadIdx.x, blockDim.x, M * nl,
-        [&](int i) {
-            const int ky = i / nl, ll = i - ky * nl;
-            S_t<Pol> v{};
-            if (z0 + ll < nz) v = ldw<CG>(in + (size_t)ky * nz + z0 + ll);
-            return v;
-        },
-        [&](int i, const S_t<Pol> &v) {
-            const int ky = i / nl, ll = i - ky * nl;
-            if (z0 + ll < nz) s0[ll * LS + pidx<Pol>(ky)] = v;
-        });
+    const int ll = threadIdx.x % nl;
+    if (z0 + ll < nz)
+        gather_smem<4, S_t<Pol>>(
+            threadIdx.x / nl, gthr, M, [&](int ky) { return ldw<CG>(in + (size_t)ky * nz + z0 + ll); },
+            [&](int ky, const S_t<Pol> &v) { s0[ll * LS + pidx<Pol>(ky)] = v; });
     __syncthreads();
     const int z = z0 + l;
     fft_line<Pol, false, EMAX>(s, sc, tw, g);
@@ -266,18 +258,16 @@ __device__ __forceinline__ void body_xi(const S_t<Pol> *__restrict__ W1, typenam
     struct AB {
         S_t<Pol> a, b;
     };
-    gather_smem<1, AB>(
-        threadIdx.x, blockDim.x, hx * nl,
-        [&](int i) {
-            const int k = i / nl, ll = i - k * nl;
-            const int yy = y0 + 2 * ll;
+    const int ll = threadIdx.x % nl, yy = y0 + 2 * ll;
+    gather_smem<4, AB>(
+        threadIdx.x / nl, gthr, hx,
+        [&](int k) {
             AB v{Pol::st(cx<R>{Pol::zero(), Pol::zero()}), Pol::st(cx<R>{Pol::zero(), Pol::zero()})};
             if (yy < ny) v.a = ldw<CG>(in + (size_t)k * ny + yy);
             if (yy + 1 < ny) v.b = ldw<CG>(in + (size_t)k * ny + yy + 1);
             return v;
         },
-        [&](int i, const AB &v) {
-            const int k = i / nl, ll = i - k * nl;
+        [&](int k, const AB &v) {
             cx<R> A = Pol::ld(v.a), B = Pol::ld(v.b);
             if (k == 0 || k == nx) {
                 A.im = Pol::zero();
