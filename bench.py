@@ -34,8 +34,6 @@ sys.path.insert(0, ROOT)
 METRIC = "3D Coulomb 256^3 FP64 Mpts/s at <=1e-12 rel err; HBM roofline fraction"
 UNIT = "Mpts/s"
 L_BOX = 12.0
-FP64_PEAK_TFLOPS = 1.25     # 152 SMs x 2 FP64 FMA/clk x 2 flop x 2.07 GHz (nominal)
-FP32_PEAK_TFLOPS = 80.5     # 152 SMs x 128 FP32 FMA/clk x 2 flop x 2.07 GHz (nominal)
 PASS_NAMES_3D = ["xf", "yf", "conv", "yi", "xi"]
 
 
@@ -320,21 +318,14 @@ def main():
     else:
         alg_flops, alg_bytes = None, None
     dom_s = avg_pass[dom] / 1e3
-    if prec == "fp32":
-        roof = {"bound": "hbm", "achieved": (alg_bytes or b_app) / dom_s / 1e9, "peak": hbm_peak,
-                "unit": "GB/s"}
-    else:
-        peak = FP64_PEAK_TFLOPS if prec == "fp64" else FP32_PEAK_TFLOPS
-        roof = {"bound": "alu", "achieved": (alg_flops or f_app) / dom_s / 1e12, "peak": peak,
-                "unit": "TFLOP/s"}
+    roof = {"bound": "hbm", "achieved": (alg_bytes or b_app) / dom_s / 1e9, "peak": hbm_peak, "unit": "GB/s"}
     roof["frac"] = roof["achieved"] / roof["peak"]
+    # radix-2 model; FP64 and FP32x2 compute in 64-bit integers, so no floating-point peak applies
+    roof["model_tflops"] = (alg_flops or f_app) / dom_s / 1e12
     roof["traffic"] = profiled_traffic(dom_name, prec)
     roof["kernel"] = f"k_{dom_name} (pass {dom} of {npass})"
-    roof["peak_source"] = ("FP64 pipe: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz (recipe nominal 1.25 TFLOP/s); "
-                           "measured DFMA probe 1.20 TFLOP/s at 2.0 GHz" if prec == "fp64" else
-                           ("FP32 pipe nominal (double-float arithmetic)" if prec == "fp32x2" else
-                            ("measured HBM copy, MEASURED_PEAKS.json" if "hbm_gbs" in peaks else
-                             "fallback HBM figure 6.8 TB/s (no MEASURED_PEAKS.json)")))
+    roof["peak_source"] = ("measured HBM copy, MEASURED_PEAKS.json" if "hbm_gbs" in peaks else
+                           "fallback HBM figure 6.8 TB/s (no MEASURED_PEAKS.json)")
     # the five passes as built move 12 (instead of 8) half-spectrum slabs
     b_5 = b_app + 4 * cbytes * (n + 1) * n * n
     hbm_whole = {"bytes_model": b_app, "achieved_gbs": b_app / (ms_per_step / 1e3) / 1e9, "peak_gbs": hbm_peak,
