@@ -38,6 +38,13 @@ struct F3 {
     static constexpr int BC = M / RC, NSC = BC;
     static constexpr int KC = (BC * LG + SG - 1) / SG;      // of them per thread
     static constexpr size_t SMEM = (size_t)NL * LS * sizeof(fxc);
+    // Words of the shared arrays r0, r1 (F3Shared): each line has its own, for the
+    // reduction of its threads (SEG of them) and the conv's sums of two warps
+    // alike, so that a sync group touches no other group's words: nothing but its
+    // own barriers orders the two uses.
+    static constexpr int LW = SEG > 2 ? SEG : 2;
+    __host__ __device__ static constexpr int reduce_word(int line, int seg) { return line * LW + seg; }
+    __host__ __device__ static constexpr int conv_word(int line, int half) { return line * LW + half; }
     static_assert(SG % NB == 0 && THREADS % SG == 0 && SG % 32 == 0, "whole lines and warps per sync group");
 };
 template <int R>
@@ -65,7 +72,7 @@ struct F3Thread {
         *bc = q % F::BC;
         return F::BC * F::LG % F::SG == 0 || q < F::BC * F::LG;
     }
-    // maximum or sum over the threads of the line; buf: NL * SEG words
+    // maximum or sum over the threads of the line; buf: NL * LW words
     template <bool MAX>
     __device__ __forceinline__ int reduce(int v, int *buf) const
     {
@@ -80,12 +87,12 @@ struct F3Thread {
             }
         }
         if constexpr (F::SEG == 1) return v;
-        if (b % F::W == 0) buf[line * F::SEG + b / F::W] = v;
+        if (b % F::W == 0) buf[F::reduce_word(line, b / F::W)] = v;
         sync();
-        v = buf[line * F::SEG];
+        v = buf[F::reduce_word(line, 0)];
 #pragma unroll
         for (int i = 1; i < F::SEG; ++i) {
-            const int w = buf[line * F::SEG + i];
+            const int w = buf[F::reduce_word(line, i)];
             v = MAX ? max(v, w) : (int)((unsigned)v + (unsigned)w);
         }
         return v;
@@ -95,11 +102,11 @@ struct F3Thread {
 // shared words of the reductions and line exponents
 template <int R>
 struct F3Shared {
-    int r0[F3<R>::NL * (F3<R>::SEG > 2 ? F3<R>::SEG : 2)], r1[F3<R>::NL * (F3<R>::SEG > 2 ? F3<R>::SEG : 2)];
+    int r0[F3<R>::NL * F3<R>::LW], r1[F3<R>::NL * F3<R>::LW];
     int e[F3<R>::NL];
 };
 
-// padded position; f3_off: of a compile-time offset that does not carry into it
+// padded position
 __device__ __forceinline__ constexpr int f3_pos(int i) { return i + (i >> 3); }
 
 __device__ __forceinline__ int f3_norm(int acc, int top_bits)
@@ -335,7 +342,7 @@ __device__ __forceinline__ void f3_body_conv(fxc *__restrict__ Wd, const int2 *_
             for (int o = 4; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
         } else {
             acc[k] = __reduce_add_sync(0xffffffffu, acc[k]);
-            if (have && (bc & 31) == 0) sh.r1[ln * 2 + (bc >> 5)] = (int)acc[k];
+            if (have && (bc & 31) == 0) sh.r1[F::conv_word(ln, bc >> 5)] = (int)acc[k];
         }
     }
     th.sync();
@@ -344,7 +351,7 @@ __device__ __forceinline__ void f3_body_conv(fxc *__restrict__ Wd, const int2 *_
     for (int k = 0; k < F::KC; ++k) {
         int ln, bc;
         if (!th.last_bfly(k, &ln, &bc)) break;
-        const unsigned a = F::TWO ? acc[k] : (unsigned)sh.r1[ln * 2] + (unsigned)sh.r1[ln * 2 + 1];
+        const unsigned a = F::TWO ? acc[k] : (unsigned)sh.r1[F::conv_word(ln, 0)] + (unsigned)sh.r1[F::conv_word(ln, 1)];
         const int sn = f3_norm((int)a, kFxTop - 44);
         if (bc == 0 && r0 + ln < rows) ex.cv[base + r0 + ln] = sh.e[ln] + er[k] + sn;
         if (sn > 0) {

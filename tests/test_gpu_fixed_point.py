@@ -154,3 +154,15 @@ def test_split_inverse_x(gsm, n):
     for debug in (2, 6):
         v = gsm.Plan("coulomb2d", 4.0, n, debug=debug).apply(r)
         assert float((u - v).abs().max() / v.abs().max()) < 2.0 ** -53 * np.log2(4.0 * n[0] * n[1])
+
+
+@pytest.mark.parametrize("N", [96, 160, 192])
+def test_conv_of_several_sync_groups_repeats_its_bits(gsm, N):
+    """The conv lines of a CTA whose sync groups are not ordered against one another (three to six
+    warps each): 200 applies with equal bits."""
+    import torch
+    r = torch.tensor(np.random.default_rng(N).standard_normal((N, 60, 64)), device="cuda")
+    plan = gsm.Plan("coulomb3d", 4.0, (64, 60, N))
+    u = plan.apply(r)
+    for _ in range(200):
+        assert torch.equal(plan.apply(r), u)
