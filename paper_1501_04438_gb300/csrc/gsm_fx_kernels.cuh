@@ -80,58 +80,73 @@ __global__ void __launch_bounds__(fx_threads(EMAX), fx_ctas(EMAX))
 
 }  // namespace
 
+// The passes of padded length M.  Defined in the translation unit that the length
+// belongs to and nowhere else: the kernels have internal linkage, so a second copy
+// would have shared-memory limits of its own.
 template <int M>
 struct FixedPasses {
+    static bool serves(const Plan *p, int axis, bool fwd, bool inv, const PassCfg &c);
+    // kernels' shared-memory limits for shape c (any that serves() may accept)
+    static cudaError_t raise(const Plan *p, int pass, const PassCfg &c);
+    // false: not served
+    static bool launch(const FxCall &a, int pass, const PassCfg &c);
+};
+
+#ifdef GSM_FX_LENGTH_UNIT
+template <int M>
+bool FixedPasses<M>::serves(const Plan *p, int axis, bool fwd, bool inv, const PassCfg &c)
+{
     using F = FixedSched<M>;
     using I = FixedSched<M, true>;
-    static constexpr int T = fixed_threads<F>();
-    static bool serves(const Plan *p, int axis, bool fwd, bool inv, const PassCfg &c)
-    {
-        const bool conv = fwd && inv;
-        return c.emax == 8 && c.gthr == T && (!fwd || F::is(p->sched_f[axis])) &&
-               (!inv || (conv ? I::is(p->sched_i[axis]) : F::is(p->sched_i[axis])));
+    const bool conv = fwd && inv;
+    return c.emax == 8 && c.gthr == fixed_threads<F>() && (!fwd || F::is(p->sched_f[axis])) &&
+           (!inv || (conv ? I::is(p->sched_i[axis]) : F::is(p->sched_i[axis])));
+}
+template <int M>
+cudaError_t FixedPasses<M>::raise(const Plan *p, int pass, const PassCfg &c)
+{
+    using F = FixedSched<M>;
+    using I = FixedSched<M, true>;
+    const int last = p->d == 3 ? 4 : 2, conv = p->d == 3 ? 2 : 1;
+    if (c.emax != 8) return cudaSuccess;
+    if (pass == 0) return raise_smem(k_fx_xf<8, F>, c.smem);
+    if (pass == last) return raise_smem(k_fx_xi<8, F>, c.smem);
+    if (pass == conv) return raise_smem(k_fx_conv<8, F, I>, c.smem);
+    if constexpr (M <= kFxLongM) return pass == 1 ? raise_smem(k_fx_yf<8, F>, c.smem) : raise_smem(k_fx_yi<8, F>, c.smem);
+    return cudaSuccess;
+}
+template <int M>
+bool FixedPasses<M>::launch(const FxCall &a, int pass, const PassCfg &c)
+{
+    using F = FixedSched<M>;
+    using I = FixedSched<M, true>;
+    const Plan *p = a.p;
+    const int last = p->d == 3 ? 4 : 2, conv = p->d == 3 ? 2 : 1;
+    const int axis = pass == 0 || pass == last ? 0 : pass == conv ? p->d - 1 : 1;
+    if (!serves(p, axis, pass <= conv, pass >= conv, c)) return false;
+    if constexpr (M > kFxLongM)
+        if (pass != 0 && pass != last && pass != conv) return false;
+    const int nx = p->n[0], ny = p->n[1], nz = a.nz, hx = nx + 1;
+    fxc *W1 = static_cast<fxc *>(a.W1), *W2 = static_cast<fxc *>(a.W2);
+    const int4 *tw = static_cast<const int4 *>(p->d_tw[axis]), *twi = static_cast<const int4 *>(p->d_twi[axis]);
+    const dim3 gx((ny + 2 * c.nl - 1) / (2 * c.nl), nz), gy((nz + c.nl - 1) / c.nl, hx), b(c.gthr, c.nl);
+    if (pass == 0) {
+        k_fx_xf<8, F><<<gx, b, c.smem, a.st>>>(a.rho, W1, a.ex, nx, ny, hx, F(), c.nl, tw);
+    } else if (pass == last) {
+        k_fx_xi<8, F><<<gx, b, c.smem, a.st>>>(W1, a.u, p->d == 3 ? a.ex.yi : a.ex.cv, hx, nx, ny, hx, F(), c.nl, twi);
+    } else if (pass == conv) {
+        const int My = p->d == 3 ? p->M[1] : 1;
+        const dim3 g = p->d == 3 ? dim3((My + c.nl - 1) / c.nl, hx) : dim3((hx + c.nl - 1) / c.nl);
+        k_fx_conv<8, F, I><<<g, b, c.smem, a.st>>>(p->d == 3 ? W2 : W1, static_cast<const int2 *>(p->d_mult), p->d_mrow,
+                                                   a.ex, p->d == 3 ? hx * My : hx, p->n[axis], p->d == 3, My, ny + 1,
+                                                   F(), I(), c.nl, tw, twi, p->mult_full ? 1 : 0);
+    } else if constexpr (M <= kFxLongM) {
+        if (pass == 1) k_fx_yf<8, F><<<gy, b, c.smem, a.st>>>(W1, W2, a.ex, ny, nz, hx, F(), c.nl, tw);
+        else k_fx_yi<8, F><<<gy, b, c.smem, a.st>>>(W2, W1, a.ex, ny, nz, hx, F(), c.nl, twi);
     }
-    // kernels' shared-memory limits for shape c (any that serves() may accept)
-    static cudaError_t raise(const Plan *p, int pass, const PassCfg &c)
-    {
-        const int last = p->d == 3 ? 4 : 2, conv = p->d == 3 ? 2 : 1;
-        if (c.emax != 8) return cudaSuccess;
-        if (pass == 0) return raise_smem(k_fx_xf<8, F>, c.smem);
-        if (pass == last) return raise_smem(k_fx_xi<8, F>, c.smem);
-        if (pass == conv) return raise_smem(k_fx_conv<8, F, I>, c.smem);
-        if constexpr (M <= kFxLongM) return pass == 1 ? raise_smem(k_fx_yf<8, F>, c.smem) : raise_smem(k_fx_yi<8, F>, c.smem);
-        return cudaSuccess;
-    }
-    // false: not served
-    static bool launch(const FxCall &a, int pass, const PassCfg &c)
-    {
-        const Plan *p = a.p;
-        const int last = p->d == 3 ? 4 : 2, conv = p->d == 3 ? 2 : 1;
-        const int axis = pass == 0 || pass == last ? 0 : pass == conv ? p->d - 1 : 1;
-        if (!serves(p, axis, pass <= conv, pass >= conv, c)) return false;
-        if constexpr (M > kFxLongM)
-            if (pass != 0 && pass != last && pass != conv) return false;
-        const int nx = p->n[0], ny = p->n[1], nz = a.nz, hx = nx + 1;
-        fxc *W1 = static_cast<fxc *>(a.W1), *W2 = static_cast<fxc *>(a.W2);
-        const int4 *tw = static_cast<const int4 *>(p->d_tw[axis]), *twi = static_cast<const int4 *>(p->d_twi[axis]);
-        const dim3 gx((ny + 2 * c.nl - 1) / (2 * c.nl), nz), gy((nz + c.nl - 1) / c.nl, hx), b(c.gthr, c.nl);
-        if (pass == 0) {
-            k_fx_xf<8, F><<<gx, b, c.smem, a.st>>>(a.rho, W1, a.ex, nx, ny, hx, F(), c.nl, tw);
-        } else if (pass == last) {
-            k_fx_xi<8, F><<<gx, b, c.smem, a.st>>>(W1, a.u, p->d == 3 ? a.ex.yi : a.ex.cv, hx, nx, ny, hx, F(), c.nl, twi);
-        } else if (pass == conv) {
-            const int My = p->d == 3 ? p->M[1] : 1;
-            const dim3 g = p->d == 3 ? dim3((My + c.nl - 1) / c.nl, hx) : dim3((hx + c.nl - 1) / c.nl);
-            k_fx_conv<8, F, I><<<g, b, c.smem, a.st>>>(p->d == 3 ? W2 : W1, static_cast<const int2 *>(p->d_mult), p->d_mrow,
-                                                       a.ex, p->d == 3 ? hx * My : hx, p->n[axis], p->d == 3, My, ny + 1,
-                                                       F(), I(), c.nl, tw, twi, p->mult_full ? 1 : 0);
-        } else if constexpr (M <= kFxLongM) {
-            if (pass == 1) k_fx_yf<8, F><<<gy, b, c.smem, a.st>>>(W1, W2, a.ex, ny, nz, hx, F(), c.nl, tw);
-            else k_fx_yi<8, F><<<gy, b, c.smem, a.st>>>(W2, W1, a.ex, ny, nz, hx, F(), c.nl, twi);
-        }
-        return true;
-    }
-};
+    return true;
+}
+#endif
 
 // The lengths of each translation unit (gsm_fx_len_*.cu).
 #define GSM_FX_LENGTHS_A(X) X(48) X(60) X(72) X(80) X(96) X(100) X(108)
@@ -141,12 +156,8 @@ struct FixedPasses {
 #define GSM_FX_LENGTHS_E(X) X(1024) X(2048)
 #define GSM_FX_LENGTHS(X) \
     GSM_FX_LENGTHS_A(X) GSM_FX_LENGTHS_B(X) GSM_FX_LENGTHS_C(X) GSM_FX_LENGTHS_D(X) GSM_FX_LENGTHS_E(X)
-#define GSM_FX_EXTERN(M) extern template struct FixedPasses<M>;
 #define GSM_FX_DEFINE(M) template struct FixedPasses<M>;
 #ifndef GSM_FX_LENGTH_UNIT
-GSM_FX_LENGTHS(GSM_FX_EXTERN)
-#endif
-
 inline int fixed_axis(const Plan *p, int pass)
 {
     return pass == 0 || pass == (p->d == 3 ? 4 : 2) ? 0 : pass == (p->d == 3 ? 2 : 1) ? p->d - 1 : 1;
@@ -167,5 +178,6 @@ inline cudaError_t fixed_raise(const Plan *p, int pass, const PassCfg &c)
 #undef GSM_FX_CASE
     return cudaSuccess;
 }
+#endif
 
 }  // namespace gsm
