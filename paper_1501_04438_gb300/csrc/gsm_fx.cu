@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(fx_threads(EMAX), fx_ctas(EMAX))
     fxc *s = reinterpret_cast<fxc *>(smem_raw) + l * line_stride<FX>(M);
     const int line = blockIdx.x * nl + l;
     if (line >= nlines) return;
-    FxLine ln{0, 0, M > kFxLongM, red};
+    FxLine ln{0, 0, M > kFxLongM, red, 0};
     FxFromPairs src;
     src.p = in + (size_t)line * M;
     fx_transform<FWD, EMAX, false, false>(s, sc, tw, g, ln, src, FxToPairs{out + (size_t)line * M, &ln});
@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(128) k_fx_mult_rows(const double *in, int2 *ou
     if (m > 0.0) frexp(m, &e);
     if (threadIdx.x == 0) row_exp[blockIdx.x] = e;
     for (int i = threadIdx.x; i < len; i += blockDim.x)
-        out[(size_t)blockIdx.x * len + i] = m > 0.0 ? fx_factor(ldexp(r[i], -e), 0.0) : make_int2(0, 0);
+        out[(size_t)blockIdx.x * len + i] = m > 0.0 ? fx_mult_factor(ldexp(r[i], -e)) : make_int2(0, 0);
 }
 
 // thread x of a line's group, line y of the CTA

@@ -7,24 +7,28 @@
 // is a block of 64-bit integers with one common exponent:
 //   value = (re + i im) 2^E,   re, im: signed 64-bit, E one per line.
 // A complex addition is two 64-bit integer additions (4 instructions), a
-// rotation 14 multiply-adds on 31-bit halves.  Measured per warp and SM
-// sub-partition (2.0 GHz): a 64-bit addition 2.4 cycles, a 32 x 32 + 64
-// multiply-add 4, a DFMA 64; a twiddled radix-8 butterfly 680 cycles here, 66
-// DFMA = 4200 in FP64, 820 with pairs of floats.  What bounds the passes is the
-// integer issue rate (60 % of the issue slots busy, DRAM at 7-20 %).  FP64 apply
-// at 256^3 (five passes): 8.88 ms in FP64 arithmetic, 2.32 ms here; the pairs of
-// floats that FP32X2 used before took 2.92 ms.
+// rotation 12 multiply-adds on 32-bit halves and two 64-bit shifts.  Measured per
+// warp and SM sub-partition (2.0 GHz): a 64-bit addition 2.4 cycles, a 32 x 32 + 64
+// multiply-add 4, a DFMA 64.  FP64 apply at 256^3: 8.88 ms in FP64 arithmetic,
+// 1.80 ms here (1.67 ms before the products and shifts were rounded without bias
+// and the multiplier had exponents of its own, see below).
 //
-// Accuracy.  A line is scaled when it is loaded so that the sum of
-// |re| + |im| over the line is below 2^61: every value of every stage is a
+// Accuracy.  A line is scaled when it is loaded, and again after the
+// multiplication, so that the sum of |re| + |im| over the line is below 2^62 (2^61
+// if outputs are added in pairs after it): every value of every stage is a
 // partial sum of the inputs with factors of modulus one, so nothing overflows
-// and the full range is used, with an absolute rounding of about one unit per
-// product, 2^-61 of that sum, where FP64 rounds every operation to 2^-53 of
+// and the full range is used, with an absolute rounding of half a unit or so per
+// product, 2^-62 of that sum, where FP64 rounds every operation to 2^-53 of
 // its result.  Lines longer than kFxLongM, whose sum is far above their
 // values, are rescaled from their actual maximum after every stage instead
-// (block floating point).  Both are compared with long double on the host over all lengths,
-// for smooth, single-point and random lines: rms errors 0.02 to 0.6 of an FP64
-// radix-2 FFT's, up to equal for random full lines of 360 to 512.
+// (block floating point).  Roundings have no preferred side: a bias of half a unit
+// per value adds up to M/2 units in one output, and where that is frequency zero
+// the multiplier makes it the result's error.  Multiplied lines (forward, 1/k^2,
+// inverse) against long double, maximum norm, here and with a plain FFT in doubles:
+// smooth 1.1e-16 / 2.6e-16 (n = 256), 1.1e-16 / 3.3e-16 (n = 2048); a point 9e-17 /
+// 2.7e-16, 1.8e-16 / 2.7e-16; white noise 2.2e-16 / 5.6e-16, 2.1e-16 / 5.9e-16;
+// Gaussian times a wave at 0.9 of Nyquist 2.6e-14 / 7.6e-14, 1.8e-13 / 1.7e-12.  A
+// host test holds such lines to the error of doubles.
 //
 // The functions here compile for the host too (one thread per line), which is
 // what those comparisons run.
@@ -57,8 +61,7 @@ struct FX {
 // Line exponents: beyond +-kFxBig they mark a line whose input held an
 // infinity or a NaN (its outputs are NaN) and a line that is not there (zeros).
 constexpr int kFxNan = 1 << 28, kFxZero = -(1 << 28), kFxBig = 1 << 27;
-constexpr int kFxTop = 61;         // bound of a line's sum, as a power of two
-constexpr int kFxStage = 58;       // bound of re, im before a stage of a long line
+constexpr int kFxTop = 62;         // bound of a line's sum, as a power of two (FxLine::paired: one less)
 constexpr int kFxLongM = 512;      // lines longer than this are rescaled after every stage
 
 // ---------------------------------------------------------------- arithmetic
@@ -66,19 +69,22 @@ GSM_HD long long radd(long long a, long long b) { return (long long)((unsigned l
 GSM_HD long long rsub(long long a, long long b) { return (long long)((unsigned long long)a - (unsigned long long)b); }
 GSM_HD long long rneg(long long a) { return rsub(0, a); }
 
-// x = h 2^31 + l with 0 <= l < 2^31 (|x| < 2^62, so h fits)
+// x = h 2^32 + l with -2^31 <= l < 2^31: l is x's low word, so that the part of
+// a product that is dropped below has no preferred sign
 struct fxh {
     int h, l;
 };
-GSM_HD fxh fx_split(long long x) { return {(int)(x >> 31), (int)((unsigned)x & 0x7fffffffu)}; }
+GSM_HD fxh fx_split(long long x) { return {(int)(x >> 32) + (int)((unsigned)x >> 31), (int)x}; }
 
-// A factor c, |c| <= 1, is (h, l) with c = h 2^-31 + l 2^-62, |l| <= 2^30 (the
-// factors +-1 are +-(1 - 2^-62)).  x c = hx hc + (hx lc + lx hc) 2^-31 up to half
-// a unit; the cross terms are rounded to their high word (kFxHalf) and doubled,
-// within one unit, and 0 c = 0.
-constexpr long long kFxHalf = 1ll << 31;
-// a b + c, one instruction (spelled out: the compiler knows that l is not
-// negative and would widen it unsigned, which makes the product a 64 x 64-bit one)
+// A factor c, |c| <= 1, is (h, l) with c = h 2^-30 + l 2^-62, |l| < 2^31, so that
+// 1 is exact.  x c = 4 hx hc + (hx lc + lx hc) 2^-30 + lx lc 2^-62; the cross
+// terms are rounded (kFxHalf), the last term, one unit at most, is dropped.  A
+// factor of 1, -1, i or -i is exact, and no product leans to one side: a bias of
+// half a unit per product would add up in the output of frequency zero of what
+// follows, where the multiplier is largest.
+constexpr long long kFxHalf = 1ll << 29;
+// a b + c, one instruction (spelled out: the compiler would widen a factor that
+// it knows not to be negative unsigned, which makes the product a 64 x 64-bit one)
 GSM_HD long long fx_mad(int a, int b, long long c)
 {
 #ifdef __CUDA_ARCH__
@@ -89,7 +95,7 @@ GSM_HD long long fx_mad(int a, int b, long long c)
     return (long long)a * b + c;
 #endif
 }
-GSM_HD long long fx_join(long long acc, long long mid) { return fx_mad((int)(mid >> 32), 2, acc); }
+GSM_HD long long fx_join(long long acc, long long mid) { return radd((long long)((unsigned long long)acc << 2), mid >> 30); }
 GSM_HD long long fx_mul(fxh x, int ch, int cl)
 {
     return fx_join(fx_mad(x.h, ch, 0), fx_mad(x.l, ch, fx_mad(x.h, cl, kFxHalf)));
@@ -98,8 +104,8 @@ GSM_HD long long fx_mul(fxh x, int ch, int cl)
 template <long long K62>
 GSM_HD long long fx_mulc(long long x)
 {
-    constexpr int h = (int)((K62 + (1ll << 30)) >> 31);
-    constexpr int l = (int)(K62 - h * (1ll << 31));
+    constexpr int h = (int)((K62 + (1ll << 31)) >> 32);
+    constexpr int l = (int)(K62 - h * (1ll << 32));
     return fx_mul(fx_split(x), h, l);
 }
 
@@ -129,13 +135,16 @@ GSM_HD cx<long long> fx_subq(cx<long long> a, cx<long long> b) { return fx_addq<
 GSM_HD cx<long long> fx_ld(const fxc &v) { return {v.re, v.im}; }
 GSM_HD fxc fx_st(cx<long long> a) { return {a.re, a.im}; }
 
-// x 2^-s, 0 <= s <= 62, rounded (half up)
-GSM_HD long long fx_shift(long long x, int s, long long half) { return (x + half) >> s; }
-GSM_HD cx<long long> fx_shift(cx<long long> a, int s)
+// x 2^-s, 0 < s <= 62, rounded to nearest, ties to even (a preferred side would
+// add up like the products' above)
+GSM_HD long long fx_shift(long long x, int s)
 {
-    const long long half = s > 0 ? 1ll << (s - 1) : 0;
-    return {fx_shift(a.re, s, half), fx_shift(a.im, s, half)};
+    return (x + ((1ll << (s - 1)) - 1) + ((unsigned)(x >> s) & 1u)) >> s;
 }
+GSM_HD cx<long long> fx_shift(cx<long long> a, int s) { return {fx_shift(a.re, s), fx_shift(a.im, s)}; }
+// x 2^-s for either sign of s, |s| <= 62 (x 2^-s must fit)
+GSM_HD long long fx_scale2(long long x, int s) { return s > 0 ? fx_shift(x, s) : (long long)((unsigned long long)x << -s); }
+GSM_HD cx<long long> fx_scale2(cx<long long> a, int s) { return {fx_scale2(a.re, s), fx_scale2(a.im, s)}; }
 
 GSM_HD unsigned fx_abs_high(long long x)
 {
@@ -341,26 +350,33 @@ struct FxLine {
     int pad;      // layout in shared memory (fx_pos)
     bool longm;   // rescale after every stage
     int *red;     // two buffers of one word per warp of the CTA
+    int paired;   // 1: sums and differences of two outputs are formed from them
 };
 constexpr int kFxRedWarps = 16;
 constexpr int kFxRedWords = 2 * kFxRedWarps;
 
+// Bound (as a power of two) of re and im before a stage of a long line that adds
+// `terms` values: its outputs, terms sqrt(2) times that at most, stay below 2^63
+// or, out > 0 (1 + FxLine::paired), those of a line's last stage below 2^(63 - out).
+// So every value in the workspace, pairs included, is below 2^62 (see FxInts).
+GSM_HD constexpr int fx_bound(int terms, int out) { return (terms > 5 ? 59 : terms > 2 ? 60 : 61) - out; }
+
 // The shift that brings a line into range, from the group's sum of
 // (|high word| >> 12) + 1 over re and im (kFxTop), or from its maximum high
-// word (kFxStage, long lines); the same for every thread of the group.
-// fx_weight: one value's part of that bound.
+// word (long lines: 2^bound); the same for every thread of the group.
+// fx_weight: one value's part of that sum or maximum.
 GSM_HD unsigned fx_weight(cx<long long> x, bool longm)
 {
     const unsigned a = fx_abs_high(x.re), b = fx_abs_high(x.im);
     return longm ? (a > b ? a : b) : (a >> 12) + (b >> 12) + 2u;
 }
 GSM_HD unsigned fx_weigh(unsigned acc, unsigned w, bool longm) { return longm ? (acc > w ? acc : w) : acc + w; }
-GSM_HD int fx_shift_of(unsigned acc, const FxLine &ln, const Group &g, int *buf)
+GSM_HD int fx_shift_of(unsigned acc, const FxLine &ln, const Group &g, int *buf, int bound)
 {
     // sum: below acc 2^44, so acc - 1 < 2^b gives sum <= 2^(44 + b); maximum: high word + 1
     int s;
-    if (ln.longm) s = fx_bits((unsigned)fx_reduce<true>((int)acc, g, buf)) - (kFxStage - 32);
-    else s = fx_bits((unsigned)fx_reduce<false>((int)acc, g, buf)) - (kFxTop - 44);
+    if (ln.longm) s = fx_bits((unsigned)fx_reduce<true>((int)acc, g, buf)) - (bound - 32);
+    else s = fx_bits((unsigned)fx_reduce<false>((int)acc, g, buf)) - (kFxTop - ln.paired - 44);
     return s > 0 ? s : 0;
 }
 
@@ -432,6 +448,13 @@ GSM_HD int first_radix(const SC &sc)
     if constexpr (is_fixed_sched<SC>::value) return SC::template radix<0>();
     else return sc.r[0];
 }
+// bound of a long line before stage ST (Sched: st); out: see fx_bound, should it be the last
+template <int ST, class SC>
+GSM_HD int fx_bound_before(const SC &sc, int st, int out)
+{
+    if constexpr (is_fixed_sched<SC>::value) return fx_bound(SC::template radix<(ST < SC::nst ? ST : 0)>(), ST == SC::nst - 1 ? out : 0);
+    else return fx_bound(sc.r[st], st == sc.nst - 1 ? out : 0);
+}
 
 // ---------------------------------------------------------------- stages
 // First radix of the stage-ordered table: the twiddles of stage st (radix R
@@ -458,13 +481,14 @@ GSM_HD int fx_pos(int i, int pad) { return i + (i >> pad); }
 // same for all threads:
 //   in.load(b, off)       raw element (In::raw) of the line
 //   in.exponent(r)        its exponent
-//   in.align(r, e)        it as integers of exponent e >= its own
+//   in.align(r, e, longm) it as integers of exponent e >= its own
 //   in.line_exponent(e)   exponent of the line whose largest is e
 //   out(b, off, v)        takes an output of the transform
 //   Out::kSmem            stores it in the line's own shared memory
 // First stage (radix RAD, untwiddled), HALF = 1: inputs t >= RAD/2 are zero.
+// next: bound of a long line before the second stage.
 template <int RAD, bool FWD, int NB, int HALF, class SC, class In, class Out>
-GSM_HD void fx_first(fxc *s, const SC &sc, const Group &g, FxLine &ln, In in, Out out)
+GSM_HD void fx_first(fxc *s, const SC &sc, const Group &g, FxLine &ln, int next, In in, Out out)
 {
     constexpr int NIN = HALF == 1 ? RAD / 2 : RAD;
     const int nb = sc.M / RAD;
@@ -498,13 +522,13 @@ GSM_HD void fx_first(fxc *s, const SC &sc, const Group &g, FxLine &ln, In in, Ou
             if (g.t + i * g.T < nb) {
 #pragma unroll
                 for (int t = 0; t < NIN; ++t) {
-                    v[i][t] = in.align(raw[i][t], em);
+                    v[i][t] = in.align(raw[i][t], em, ln.longm);
                     acc = fx_weigh(acc, fx_weight(v[i][t], ln.longm), ln.longm);
                 }
             }
         }
     }
-    const int sn = fx_shift_of(acc, ln, g, ln.red + kFxRedWarps);
+    const int sn = fx_shift_of(acc, ln, g, ln.red + kFxRedWarps, fx_bound(NIN, last ? 1 + ln.paired : 0));
     ln.E = in.line_exponent(em) + sn;
     acc = 0;
 #pragma unroll
@@ -523,7 +547,7 @@ GSM_HD void fx_first(fxc *s, const SC &sc, const Group &g, FxLine &ln, In in, Ou
     }
     int sh = 0;
     if (ln.longm && !last) {
-        sh = fx_shift_of(acc, ln, g, ln.red);
+        sh = fx_shift_of(acc, ln, g, ln.red, next);
         ln.E += sh;
     } else if (g.bar < 0) {
         fx_sync(g);   // one warp: the reductions passed no barrier since the line was read
@@ -549,10 +573,10 @@ GSM_HD void fx_first(fxc *s, const SC &sc, const Group &g, FxLine &ln, In in, Ou
 
 // Stage of radix RAD after stages of product Ns > 1: s -> s, or -> out when it
 // is the last one.  CROP: of the last stage only the outputs t < RAD/2 (even
-// radices).
+// radices).  next: bound of a long line before the next stage.
 template <int RAD, bool FWD, int NB, bool CROP, class Out>
 GSM_HD void fx_stage(fxc *s, int M, int Ns, bool last, const int4 *__restrict__ tws, const Group &g, FxLine &ln,
-                     Out out)
+                     int next, Out out)
 {
     const int nb = M / RAD;
     cx<long long> v[NB][RAD];
@@ -589,7 +613,7 @@ GSM_HD void fx_stage(fxc *s, int M, int Ns, bool last, const int4 *__restrict__ 
     }
     int sh = 0;
     if (ln.longm) {   // several warps: the reduction passes a barrier
-        sh = fx_shift_of(acc, ln, g, ln.red + kFxRedWarps);
+        sh = fx_shift_of(acc, ln, g, ln.red + kFxRedWarps, next);
         ln.E += sh;
     } else {
         fx_sync(g);
@@ -614,14 +638,14 @@ GSM_HD void fx_stage(fxc *s, int M, int Ns, bool last, const int4 *__restrict__ 
 // The stages [st_begin, st_end) (st_end < 0: to the last) after the first, in
 // the order 8, 4, 2, 5, 3, each radix one loop of its own; the transform's
 // last stage hands its outputs to `out`.
-template <bool FWD, int EMAX, bool CROP, int ST, int END, class SC, class Out>
+template <bool FWD, int EMAX, bool CROP, bool MID, int ST, int END, class SC, class Out>
 GSM_HD void fx_rest_fixed(fxc *s, const int4 *__restrict__ tw, const Group &g, FxLine &ln, Out out)
 {
     if constexpr (ST < END) {
         constexpr int RAD = SC::template radix<ST>(), Ns = SC::product(ST);
         fx_stage<RAD, FWD, (EMAX + RAD - 1) / RAD, CROP>(s, SC::M, Ns, ST == SC::nst - 1, fx_stage_table(tw, SC{}, Ns), g,
-                                                         ln, out);
-        fx_rest_fixed<FWD, EMAX, CROP, ST + 1, END, SC>(s, tw, g, ln, out);
+                                                         ln, fx_bound_before<ST + 1>(SC{}, 0, MID ? 0 : 1 + ln.paired), out);
+        fx_rest_fixed<FWD, EMAX, CROP, MID, ST + 1, END, SC>(s, tw, g, ln, out);
     }
 }
 // MID: up to the last stage, which is fused with the multiplication
@@ -630,14 +654,15 @@ GSM_HD void fx_rest_of(fxc *s, const SC &sc, const int4 *__restrict__ tw, const 
 
 template <bool FWD, int EMAX, bool CROP, class Out>
 GSM_HD void fx_rest(fxc *s, const Sched &sc, const int4 *__restrict__ tw, const Group &g, FxLine &ln, int st_begin,
-                    int st_end, Out out)
+                    int st_end, int out_bound, Out out)
 {
     const int last = sc.nst - 1, nend = st_end < 0 ? sc.nst : st_end;
     int Ns = 1, st = st_begin;
     for (int i = 0; i < st_begin; ++i) Ns *= sc.r[i];
 #define GSM_FX_STAGES(RAD)                                                                      \
     for (; st < nend && sc.r[st] == RAD; ++st, Ns *= RAD)                                       \
-        fx_stage<RAD, FWD, (EMAX + RAD - 1) / RAD, CROP>(s, sc.M, Ns, st == last, fx_stage_table(tw, sc, Ns), g, ln, out)
+        fx_stage<RAD, FWD, (EMAX + RAD - 1) / RAD, CROP>(s, sc.M, Ns, st == last, fx_stage_table(tw, sc, Ns), g, ln, \
+                                                         st < last ? fx_bound_before<0>(sc, st + 1, out_bound) : 0, out)
     GSM_FX_STAGES(8);
     GSM_FX_STAGES(4);
     GSM_FX_STAGES(2);
@@ -648,27 +673,29 @@ GSM_HD void fx_rest(fxc *s, const Sched &sc, const int4 *__restrict__ tw, const 
 template <bool FWD, int EMAX, bool CROP, bool MID, class SC, class Out>
 GSM_HD void fx_rest_of(fxc *s, const SC &sc, const int4 *__restrict__ tw, const Group &g, FxLine &ln, Out out)
 {
-    if constexpr (is_fixed_sched<SC>::value) fx_rest_fixed<FWD, EMAX, CROP, 1, MID ? SC::nst - 1 : SC::nst, SC>(s, tw, g, ln, out);
-    else fx_rest<FWD, EMAX, CROP>(s, sc, tw, g, ln, 1, MID ? sc.nst - 1 : -1, out);
+    if constexpr (is_fixed_sched<SC>::value) fx_rest_fixed<FWD, EMAX, CROP, MID, 1, MID ? SC::nst - 1 : SC::nst, SC>(s, tw, g, ln, out);
+    else fx_rest<FWD, EMAX, CROP>(s, sc, tw, g, ln, 1, MID ? sc.nst - 1 : -1, MID ? 0 : 1 + ln.paired, out);
 }
 
 // First stage by the schedule's first radix.  ZPAD: the second half of the
-// line is zero (forward transforms; their first radix is even).
-template <bool FWD, int EMAX, bool ZPAD, class SC, class In, class Out>
+// line is zero (forward transforms; their first radix is even).  MID: the last
+// stage is fused with the multiplication.
+template <bool FWD, int EMAX, bool ZPAD, bool MID, class SC, class In, class Out>
 GSM_HD void fx_begin(fxc *s, const SC &sc, const Group &g, FxLine &ln, In in, Out out)
 {
     constexpr int H = ZPAD ? 1 : 0;
+    const int next = sc.nst > 1 ? fx_bound_before<1>(sc, 1, MID ? 0 : 1 + ln.paired) : 0;
     if constexpr (is_fixed_sched<SC>::value) {
         constexpr int RAD = SC::template radix<0>();
-        fx_first<RAD, FWD, (EMAX + RAD - 1) / RAD, H>(s, sc, g, ln, in, out);
+        fx_first<RAD, FWD, (EMAX + RAD - 1) / RAD, H>(s, sc, g, ln, next, in, out);
     } else {
         const int r = sc.r[0];
-        if (r == 8) fx_first<8, FWD, (EMAX + 7) / 8, H>(s, sc, g, ln, in, out);
-        else if (r == 4) fx_first<4, FWD, (EMAX + 3) / 4, H>(s, sc, g, ln, in, out);
-        else if (r == 2) fx_first<2, FWD, (EMAX + 1) / 2, H>(s, sc, g, ln, in, out);
+        if (r == 8) fx_first<8, FWD, (EMAX + 7) / 8, H>(s, sc, g, ln, next, in, out);
+        else if (r == 4) fx_first<4, FWD, (EMAX + 3) / 4, H>(s, sc, g, ln, next, in, out);
+        else if (r == 2) fx_first<2, FWD, (EMAX + 1) / 2, H>(s, sc, g, ln, next, in, out);
         else if constexpr (!ZPAD) {
-            if (r == 5) fx_first<5, FWD, (EMAX + 4) / 5, 0>(s, sc, g, ln, in, out);
-            else fx_first<3, FWD, (EMAX + 2) / 3, 0>(s, sc, g, ln, in, out);
+            if (r == 5) fx_first<5, FWD, (EMAX + 4) / 5, 0>(s, sc, g, ln, next, in, out);
+            else fx_first<3, FWD, (EMAX + 2) / 3, 0>(s, sc, g, ln, next, in, out);
         }
     }
 }
@@ -678,8 +705,35 @@ GSM_HD void fx_transform(fxc *s, const SC &sc, const int4 *__restrict__ tw, cons
                          Out out)
 {
     ln.pad = sc.pad;
-    fx_begin<FWD, EMAX, ZPAD>(s, sc, g, ln, in, out);
+    fx_begin<FWD, EMAX, ZPAD, false>(s, sc, g, ln, in, out);
     fx_rest_of<FWD, EMAX, CROP, false>(s, sc, tw, g, ln, out);
+}
+
+// A multiplier entry is a factor of at least 1/2 in modulus, of 56 bits, and in its
+// low six bits the distance d of its exponent from the row's, so that a small
+// entry keeps its bits, and so does the product: a line whose weight sits where
+// the multiplier is small (an oscillating density) is scaled up by it.
+GSM_HD int fx_mult_exp(int2 m) { return m.y & 63; }
+
+// The product p 2^-d of a line's value and an entry: what it has for the maximum
+// over the line, all products being below 2^(32 + T) with T the bits of that, and
+// for the sum (T >= kFxProductT), whose unit is 2^(14 + T).
+constexpr int kFxProductT = 18;
+GSM_HD unsigned fx_product_top(cx<long long> p, int d)
+{
+    const unsigned a = fx_abs_high(p.re) | fx_abs_high(p.im);
+    return d < 32 ? a >> d : 0;
+}
+GSM_HD unsigned fx_product_weight(cx<long long> p, int d, int T)
+{
+    const int s = d + T - kFxProductT;
+    return s < 32 ? ((fx_abs_high(p.re) + fx_abs_high(p.im) + 2u) >> s) + 1u : 1u;
+}
+// shift of a product of exponent distance d in a line of total shift sn
+GSM_HD int fx_product_shift(int sn, int d)
+{
+    const int s = sn + d;
+    return s > 62 ? 62 : s < -62 ? -62 : s;
 }
 
 // The forward's last stage (radix R), the multiplication by mult(k) (entries of
@@ -692,7 +746,8 @@ GSM_HD void fx_mid(fxc *s, const SC &scf, const SCI &sci, const int4 *__restrict
     const int M = scf.M, nb = M / R;
     const int4 *tws = fx_stage_table(tw, scf, nb);
     cx<long long> v[NB][R];
-    unsigned acc = 0;
+    int d[NB][R];
+    unsigned tops = 0;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         const int b = g.t + i * g.T;
@@ -706,20 +761,33 @@ GSM_HD void fx_mid(fxc *s, const SC &scf, const SCI &sci, const int4 *__restrict
             for (int t = 0; t < R; ++t) {
                 const int2 m = mult.template at<R>(b, t, nb);
                 v[i][t] = {fx_mul(fx_split(v[i][t].re), m.x, m.y), fx_mul(fx_split(v[i][t].im), m.x, m.y)};
-                acc = fx_weigh(acc, fx_weight(v[i][t], ln.longm), ln.longm);
+                d[i][t] = fx_mult_exp(m);
+                tops = fx_weigh(tops, fx_product_top(v[i][t], d[i][t]), true);
             }
         }
     }
-    const int sn = fx_shift_of(acc, ln, g, ln.red);
+    int top = fx_bits((unsigned)fx_reduce<true>((int)tops, g, ln.red)), sn;
+    if (ln.longm) {
+        sn = top + 32 - fx_bound(R, 0);
+    } else {
+        top = top > kFxProductT ? top : kFxProductT;
+        unsigned acc = 0;
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            if (g.t + i * g.T < nb) {
+#pragma unroll
+                for (int t = 0; t < R; ++t) acc += fx_product_weight(v[i][t], d[i][t], top);
+            }
+        }
+        sn = top + 14 + fx_bits((unsigned)fx_reduce<false>((int)acc, g, ln.red + kFxRedWarps)) - (kFxTop - ln.paired);
+    }
     ln.E += erow + sn;
-    acc = 0;
+    unsigned acc = 0;
 #pragma unroll
     for (int i = 0; i < NB; ++i) {
         if (g.t + i * g.T < nb) {
-            if (sn > 0) {
 #pragma unroll
-                for (int t = 0; t < R; ++t) v[i][t] = fx_shift(v[i][t], sn);
-            }
+            for (int t = 0; t < R; ++t) v[i][t] = fx_scale2(v[i][t], fx_product_shift(sn, d[i][t]));
             fx_bfly<R, false, 0>(v[i]);
             if (ln.longm) {
 #pragma unroll
@@ -729,7 +797,7 @@ GSM_HD void fx_mid(fxc *s, const SC &scf, const SCI &sci, const int4 *__restrict
     }
     int sh = 0;
     if (ln.longm) {
-        sh = fx_shift_of(acc, ln, g, ln.red + kFxRedWarps);
+        sh = fx_shift_of(acc, ln, g, ln.red + kFxRedWarps, fx_bound_before<1>(sci, 1, 1 + ln.paired));
         ln.E += sh;
     }
     if (g.bar < 0) fx_sync(g);   // one warp: the reductions passed no barrier
@@ -742,9 +810,9 @@ GSM_HD void fx_mid(fxc *s, const SC &scf, const SCI &sci, const int4 *__restrict
 #pragma unroll
                 for (int t = 0; t < R; ++t) v[i][t] = fx_shift(v[i][t], sh);
             }
-            fxc *d = s + fx_pos(R * b, ln.pad);
+            fxc *o = s + fx_pos(R * b, ln.pad);
 #pragma unroll
-            for (int t = 0; t < R; ++t) d[t] = fx_st(v[i][t]);
+            for (int t = 0; t < R; ++t) o[t] = fx_st(v[i][t]);
         }
     }
     fx_sync(g);
@@ -780,7 +848,7 @@ GSM_HD int fx_field(double x)   // biased exponent, sign dropped
 #endif
 }
 
-// x as an integer of exponent e - 1083, e >= the field of x and >= 1 (|result| < 2^61)
+// x as an integer of exponent e - 1083, rounded, e >= the field of x and >= 1 (|result| < 2^61)
 GSM_HD long long fx_from_double(double x, int e)
 {
     unsigned long long u;
@@ -793,7 +861,7 @@ GSM_HD long long fx_from_double(double x, int e)
     const unsigned long long m = (u & 0xfffffffffffffull) | (f ? 1ull << 52 : 0ull);
     int s = e - (f ? f : 1);
     s = s < 63 ? s : 63;
-    const long long a = (long long)((m << 8) >> s), sg = (long long)u >> 63;
+    const long long a = (long long)(((m << 8) + ((1ull << s) >> 1)) >> s), sg = (long long)u >> 63;
     return (a ^ sg) - sg;
 }
 constexpr int kFxDoubleBias = 1083;
@@ -854,7 +922,7 @@ struct FxDoubles {
         const int p = fx_field(r.a), q = fx_field(r.b);
         return p > q ? p : q;
     }
-    static GSM_HD cx<long long> align(const raw &r, int e)
+    static GSM_HD cx<long long> align(const raw &r, int e, bool)
     {
         if (e == 0x7ff) return {0, 0};
         e = e < 1 ? 1 : e;
@@ -866,18 +934,22 @@ struct FxDoubles {
     }
 };
 
-// Raw complex value of integers with their own exponent.
+// Raw complex value of integers below 2^62 with their own exponent.  Aligned, they
+// are rounded in long lines: dropping the bits lowers every value by half a unit,
+// which the transform adds up, up to 2^11 units of a line whose largest value may
+// be 2^61 (an FP64 sum has that much from 2^8 units on); short lines stay below.
 struct FxInts {
     struct raw {
         fxc v;
         int e;
     };
     static GSM_HD int exponent(const raw &r) { return r.e; }
-    static GSM_HD cx<long long> align(const raw &r, int e)
+    static GSM_HD cx<long long> align(const raw &r, int e, bool longm)
     {
         int s = e - r.e;
         s = s < 63 ? s : 63;
-        return {r.v.re >> s, r.v.im >> s};
+        const long long half = longm ? (long long)((1ull << s) >> 1) : 0;
+        return {(r.v.re + half) >> s, (r.v.im + half) >> s};
     }
     static GSM_HD int line_exponent(int em) { return em; }
 };
@@ -886,11 +958,21 @@ struct FxInts {
 GSM_HD int2 fx_factor(double hi, double lo)
 {
     long long T = llrint(hi * 4611686018427387904.0) + llrint(lo * 4611686018427387904.0);
-    const long long top = (1ll << 62) - 1;
+    const long long top = 1ll << 62;
     T = T > top ? top : T < -top ? -top : T;
-    long long h = (T + (1ll << 30)) >> 31;
-    h = h > 0x7fffffffll ? 0x7fffffffll : h < -0x7fffffffll ? -0x7fffffffll : h;   // -h must exist too
-    return make_int2((int)h, (int)(T - (h << 31)));
+    const long long h = (T + (1ll << 31)) >> 32, l = T - h * (1ll << 32);
+    return make_int2((int)h, l == INT_MIN ? INT_MIN + 1 : (int)l);   // -l must exist too
+}
+
+// Multiplier entry c in units of its row's 2^e (|c| <= 1), see fx_mult_exp.
+GSM_HD int2 fx_mult_factor(double c)
+{
+    if (c == 0.0) return make_int2(0, 0);
+    int x;
+    frexp(c, &x);
+    const int d = x > 0 ? 0 : x < -63 ? 63 : -x;
+    const long long T = (llrint(ldexp(c, d + 62)) & ~63ll) + d, h = (T + (1ll << 31)) >> 32;
+    return make_int2((int)h, (int)(T - h * (1ll << 32)));
 }
 
 }  // namespace gsm

@@ -109,15 +109,9 @@ struct F3Shared {
 // padded position
 __device__ __forceinline__ constexpr int f3_pos(int i) { return i + (i >> 3); }
 
-__device__ __forceinline__ int f3_norm(int acc, int top_bits)
-{
-    const int s = fx_bits((unsigned)acc) - top_bits;
-    return s > 0 ? s : 0;
-}
-
-// First stage: radix 8, HALF = 1: inputs t >= 4 are zero.  In as in gsm_fx.cuh.
+// First stage: radix 8, HALF = 1: inputs t >= 4 are zero.  In and PAIRED as in gsm_fx.cuh.
 // Leaves the line's exponent in sh.e (read it after the next sync).
-template <int R, bool FWD, int HALF, class In>
+template <int R, bool FWD, int HALF, bool PAIRED, class In>
 __device__ __forceinline__ void f3_first(fxc *s, const F3Thread<R> &th, F3Shared<R> &sh, const In &in)
 {
     using F = F3<R>;
@@ -133,10 +127,10 @@ __device__ __forceinline__ void f3_first(fxc *s, const F3Thread<R> &th, F3Shared
     unsigned acc = 0;
 #pragma unroll
     for (int t = 0; t < NIN; ++t) {
-        v[t] = in.align(raw[t], em);
+        v[t] = in.align(raw[t], em, false);
         acc += fx_weight(v[t], false);
     }
-    const int sn = f3_norm(th.template reduce<false>((int)acc, sh.r1), kFxTop - 44);
+    const int sn = max(0, fx_bits((unsigned)th.template reduce<false>((int)acc, sh.r1)) - (kFxTop - PAIRED - 44));
     if (th.b == 0) sh.e[th.line] = in.line_exponent(em) + sn;
     if (sn > 0) {
 #pragma unroll
@@ -233,7 +227,7 @@ __device__ __forceinline__ void f3_body_xf(const double *__restrict__ rho, fxc *
     FxFromRows in;
     in.a = ya < ny ? slab + (size_t)ya * nx : nullptr;
     in.b = ya + 1 < ny ? slab + (size_t)(ya + 1) * nx : nullptr;
-    f3_first<R, true, 1>(s, th, sh, in);
+    f3_first<R, true, 1, true>(s, th, sh, in);
     f3_second<R, true>(s, th, tw);
     f3_last<R, true, false>(s, th, tw, F3ToSmem<R>{s});
     if (th.b == 0 && ya < ny) ex.xf[(size_t)z * ((ny + 1) >> 1) + (ya >> 1)] = sh.e[th.line];
@@ -269,7 +263,7 @@ __device__ __forceinline__ void f3_body_yf(const fxc *__restrict__ W1, fxc *__re
     in.p = z < nz ? W1 + ((size_t)z * hx + kx) * ny : nullptr;
     in.e = ex.xf + (size_t)z * (ny / 2);
     in.shift = 1;
-    f3_first<R, true, 1>(s, th, sh, in);
+    f3_first<R, true, 1, false>(s, th, sh, in);
     f3_second<R, true>(s, th, tw);
     f3_last<R, true, false>(s, th, tw, F3ToSmem<R>{s});
     if (th.b == 0 && z < nz) ex.yf[(size_t)kx * nz + z] = sh.e[th.line];
@@ -303,19 +297,19 @@ __device__ __forceinline__ void f3_body_conv(fxc *__restrict__ Wd, const int2 *_
         in.p = row < rows ? Wd + (size_t)line * n : nullptr;
         in.e = IS3D ? ex.yf + (size_t)by * n : ex.xf + (row & 1) * ex.xf_par;
         in.shift = IS3D ? 0 : 1;
-        f3_first<R, true, 1>(s, th, sh, in);
+        f3_first<R, true, 1, false>(s, th, sh, in);
     }
     f3_second<R, true>(s, th, tw);
-    // last forward stage, multiplier, scaling, first inverse stage
+    // last forward stage, multiplier, scaling, first inverse stage (see fx_mid)
     constexpr int RC = F::RC, BC = F::BC;
     cx<long long> v[F::KC][RC];
-    unsigned acc[F::KC];
-    int er[F::KC];
+    int d[F::KC][RC], T[F::KC], er[F::KC];
+    unsigned top[F::KC], acc[F::KC];
 #pragma unroll
     for (int k = 0; k < F::KC; ++k) {
         int ln, bc;
         const bool have = th.last_bfly(k, &ln, &bc);
-        acc[k] = 0;
+        top[k] = 0;
         er[k] = 0;
         if (have) {
             f3_last_in<R, true>(v[k], s + ln * F::LS, bc, tw);
@@ -333,10 +327,32 @@ __device__ __forceinline__ void f3_body_conv(fxc *__restrict__ Wd, const int2 *_
                 else if (2 * t >= RC) f = __ldg(mm - t * F::NSC);
                 else f = __ldg(2 * (bc + t * F::NSC) <= M ? m + t * F::NSC : mm - t * F::NSC);   // middle of an odd radix
                 v[k][t] = {fx_mul(fx_split(v[k][t].re), f.x, f.y), fx_mul(fx_split(v[k][t].im), f.x, f.y)};
-                acc[k] += fx_weight(v[k][t], false);
+                d[k][t] = fx_mult_exp(f);
+                top[k] = max(top[k], fx_product_top(v[k][t], d[k][t]));
             }
         }
         // 32 lanes of one line (two warps per line), or 8 lanes (R = 1)
+        if constexpr (F::TWO) {
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) top[k] = max(top[k], __shfl_xor_sync(0xffffffffu, top[k], o));
+        } else {
+            top[k] = __reduce_max_sync(0xffffffffu, top[k]);
+            if (have && (bc & 31) == 0) sh.r0[F::conv_word(ln, bc >> 5)] = (int)top[k];
+        }
+    }
+    if constexpr (!F::TWO) th.sync();
+#pragma unroll
+    for (int k = 0; k < F::KC; ++k) {
+        int ln, bc;
+        const bool have = th.last_bfly(k, &ln, &bc);
+        acc[k] = 0;
+        T[k] = kFxProductT;
+        if (have) {
+            if constexpr (!F::TWO) top[k] = (unsigned)max(sh.r0[F::conv_word(ln, 0)], sh.r0[F::conv_word(ln, 1)]);
+            T[k] = max(kFxProductT, fx_bits(top[k]));
+#pragma unroll
+            for (int t = 0; t < RC; ++t) acc[k] += fx_product_weight(v[k][t], d[k][t], T[k]);
+        }
         if constexpr (F::TWO) {
 #pragma unroll
             for (int o = 4; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
@@ -352,16 +368,14 @@ __device__ __forceinline__ void f3_body_conv(fxc *__restrict__ Wd, const int2 *_
         int ln, bc;
         if (!th.last_bfly(k, &ln, &bc)) break;
         const unsigned a = F::TWO ? acc[k] : (unsigned)sh.r1[F::conv_word(ln, 0)] + (unsigned)sh.r1[F::conv_word(ln, 1)];
-        const int sn = f3_norm((int)a, kFxTop - 44);
+        const int sn = T[k] + 14 + fx_bits(a) - (kFxTop - (IS3D ? 0 : 1));
         if (bc == 0 && r0 + ln < rows) ex.cv[base + r0 + ln] = sh.e[ln] + er[k] + sn;
-        if (sn > 0) {
 #pragma unroll
-            for (int t = 0; t < RC; ++t) v[k][t] = fx_shift(v[k][t], sn);
-        }
+        for (int t = 0; t < RC; ++t) v[k][t] = fx_scale2(v[k][t], fx_product_shift(sn, d[k][t]));
         fx_bfly<RC, false, 0>(v[k]);
-        fxc *d = s + ln * F::LS + (PAD ? f3_pos(RC * bc) : RC * bc);
+        fxc *o = s + ln * F::LS + (PAD ? f3_pos(RC * bc) : RC * bc);
 #pragma unroll
-        for (int t = 0; t < RC; ++t) d[t] = fx_st(v[k][t]);
+        for (int t = 0; t < RC; ++t) o[t] = fx_st(v[k][t]);
     }
     th.sync();
     fxc *l = s + th.line * F::LS;
@@ -456,7 +470,7 @@ __device__ __forceinline__ void f3_body_yi(const fxc *__restrict__ W2, fxc *__re
     F3FromSmem<R, CG, false> in;
     in.l = s + th.line * F::LS;
     in.e = ex.cv + (size_t)kx * F::M;
-    f3_first<R, false, 0>(s, th, sh, in);
+    f3_first<R, false, 0, true>(s, th, sh, in);
     f3_second<R, false>(s, th, tw);
     F3ToLines<R> out{W1 + ((size_t)z0 * hx + kx) * ny, (size_t)hx * ny, nz - z0};
     f3_last<R, false, true>(s, th, tw, out);
@@ -514,7 +528,7 @@ __device__ __forceinline__ void f3_body_xi(const fxc *__restrict__ W1, double *_
     F3FromSmem<R, CG, true> in;
     in.l = s + th.line * F::LS;
     in.e = ek;
-    f3_first<R, false, 0>(s, th, sh, in);
+    f3_first<R, false, 0, false>(s, th, sh, in);
     f3_second<R, false>(s, th, tw);
     F3ToRows<R> out{u + ((size_t)z * ny + y0) * nx, ny - y0, sh.e};
     f3_last<R, false, true>(s, th, tw, out);

@@ -38,13 +38,11 @@ struct FxFromGlobalRot : FxInts {
     int rank;
     __device__ __forceinline__ raw load(int b, int off) const { return {p[b + off], e[(b + off) >> 1], b + off}; }
     __device__ __forceinline__ int exponent(const raw &r) const { return r.e; }
-    __device__ __forceinline__ cx<long long> align(const raw &r, int em) const
+    __device__ __forceinline__ cx<long long> align(const raw &r, int em, bool longm) const
     {
-        // the x pass leaves values below 2^63: halved before a rotation
-        const cx<long long> x = FxInts::align({r.v, r.e}, em + rank);
+        const cx<long long> x = FxInts::align({r.v, r.e}, em, longm);
         return rank ? fx_rot<true>(x, twM[r.i]) : x;
     }
-    __device__ __forceinline__ int line_exponent(int em) const { return em + rank; }
 };
 struct FxHalfToSmem {
     static constexpr bool kSmem = true;
@@ -82,7 +80,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<SC>(),
     fxc *w = W + (size_t)line * Mh;
     const bool active = line < nlines;   // every CTA of a cluster reaches both cluster barriers
     if (active) {
-        FxLine ln{0, 0, Mh > kFxLongM, red};
+        FxLine ln{0, 0, Mh > kFxLongM, red, 1};
         FxFromGlobalRot in;
         in.p = w;
         in.e = ex.xf + (line & 1) * ex.xf_par;
@@ -91,7 +89,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<SC>(),
         const FxMultRow m{mult + (size_t)line * (full ? M : ny1), M, full};
         // the half's schedules always fuse (make_split_tables)
         ln.pad = sc.pad;
-        fx_begin<true, EMAX, false>(s, sc, g, ln, in, FxNoOut{});
+        fx_begin<true, EMAX, false, true>(s, sc, g, ln, in, FxNoOut{});
         fx_rest_of<true, EMAX, false, true>(s, sc, tw, g, ln, FxNoOut{});
         fx_mid_of<EMAX>(s, sc, sci, tw, g, ln, FxMultHalf{m, rank}, mrow_exp[line]);
         fx_rest_of<false, EMAX, false, false>(s, sci, twi, g, ln, FxHalfToSmem{s, twM, rank});
@@ -131,9 +129,9 @@ struct FxFromRowsRot : FxDoubles {
         return {pa != nullptr ? pa[i] : 0.0, pb != nullptr ? pb[i] : 0.0, i};
     }
     __device__ __forceinline__ int exponent(const raw &r) const { return FxDoubles::exponent({r.a, r.b}); }
-    __device__ __forceinline__ cx<long long> align(const raw &r, int em) const
+    __device__ __forceinline__ cx<long long> align(const raw &r, int em, bool longm) const
     {
-        const cx<long long> x = FxDoubles::align({r.a, r.b}, em);
+        const cx<long long> x = FxDoubles::align({r.a, r.b}, em, longm);
         return rank ? fx_rot<true>(x, twM[r.i]) : x;
     }
 };
@@ -149,7 +147,7 @@ __global__ void __launch_bounds__(split_threads<SC>(), split_ctas<SC>())
     const int Mh = sc.M;   // == nx
     const Group g = fx_thread_of<SC>().g;
     fxc *s = reinterpret_cast<fxc *>(smem_raw);
-    FxLine ln{0, 0, Mh > kFxLongM, red};
+    FxLine ln{0, 0, Mh > kFxLongM, red, 1};
     FxFromRowsRot in;
     in.pa = ya < ny ? rho + (size_t)ya * nx : nullptr;
     in.pb = ya + 1 < ny ? rho + (size_t)(ya + 1) * nx : nullptr;
@@ -225,7 +223,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(split_threads<SC>(),
             if (!real) s[fx_pos(Mh - kp - rank, sc.pad)] = {radd(v.a.x, bi), rsub(v.b.x, ai)};
         });
     __syncthreads();
-    FxLine ln{0, 0, Mh > kFxLongM, red};
+    FxLine ln{0, 0, Mh > kFxLongM, red, 0};
     FxFromSmemHalf in;
     in.s = s;
     in.e = ek;

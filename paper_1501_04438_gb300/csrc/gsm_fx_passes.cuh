@@ -124,18 +124,18 @@ struct FxFromGlobal : FxInts {
         return r;
     }
 };
-// the line's own shared memory, exponent of element i at e[min(i, fold - i)] (e == NULL: e0 for all)
+// the line's own shared memory, exponent of element i at e[min(i, fold - i)]
 template <bool CG>
 struct FxFromSmem : FxInts {
     const fxc *s;
     const int *e;
-    int fold, e0, pad;
+    int fold, pad;
     __device__ __forceinline__ raw load(int b, int off) const
     {
         const int i = b + off;
         raw r;
         r.v = s[fx_pos(i, pad)];
-        r.e = e == nullptr ? e0 : ldw<CG>(e + min(i, fold - i));
+        r.e = ldw<CG>(e + min(i, fold - i));
         return r;
     }
 };
@@ -165,7 +165,7 @@ __device__ __forceinline__ void fx_body_xf(const FxThread &th, const double *__r
     fxc *s = reinterpret_cast<fxc *>(smem_raw) + l * LS;
     const int z = by, y0 = bx * 2 * nl, ya = y0 + 2 * l;
     const double *slab = rho + (size_t)z * ny * nx;
-    FxLine ln{0, 0, M > kFxLongM, red};
+    FxLine ln{0, 0, M > kFxLongM, red, 1};
     FxFromRows in;
     in.a = ya < ny ? slab + (size_t)ya * nx : nullptr;
     in.b = ya + 1 < ny ? slab + (size_t)(ya + 1) * nx : nullptr;
@@ -201,7 +201,7 @@ __device__ __forceinline__ void fx_body_yf(const FxThread &th, const fxc *__rest
     const int l = th.l;
     fxc *s = reinterpret_cast<fxc *>(smem_raw) + l * LS;
     const int kx = by, z0 = bx * nl, z = z0 + l;
-    FxLine ln{0, 0, M > kFxLongM, red};
+    FxLine ln{0, 0, M > kFxLongM, red, 0};
     FxFromGlobal<CG> in;
     in.p = z < nz ? W1 + ((size_t)z * hx + kx) * ny : nullptr;
     in.e = ex.xf + (size_t)z * ((ny + 1) >> 1);
@@ -234,7 +234,7 @@ struct FxMultRow {
     }
 };
 // output k of the forward, multiplied, back to the line (schedules whose
-// middle stages are not fused)
+// middle stages are not fused), and from there, scaled to its largest product
 struct FxMulToSmem {
     static constexpr bool kSmem = true;
     fxc *s;
@@ -247,6 +247,25 @@ struct FxMulToSmem {
     }
 };
 
+struct FxFromProducts : FxInts {
+    const fxc *s;
+    FxMultRow m;
+    int e0, pad;
+    __device__ __forceinline__ raw load(int b, int off) const
+    {
+        return {s[fx_pos(b + off, pad)], -fx_mult_exp(m(b + off))};
+    }
+    static __device__ __forceinline__ int exponent(const raw &r)
+    {
+        return fx_bits(fx_abs_high(r.v.re) | fx_abs_high(r.v.im)) + r.e;
+    }
+    static __device__ __forceinline__ cx<long long> align(const raw &r, int em, bool)   // below 2^62
+    {
+        return fx_scale2(cx<long long>{r.v.re, r.v.im}, fx_product_shift(em - 30, -r.e));
+    }
+    __device__ __forceinline__ int line_exponent(int em) const { return e0 + em - 30; }
+};
+
 // Forward, multiplication and inverse of the line whose inputs `in` gives;
 // the outputs go to `out`.
 template <int EMAX, bool ZPAD, bool CROP, class SC, class SCI, class In, class MultF, class MulOut, class Out>
@@ -257,7 +276,7 @@ __device__ __forceinline__ void fx_convolve(fxc *s, const SC &sc, const SCI &sci
     bool fused = true;
     if constexpr (!is_fixed_sched<SC>::value) fused = fused_radix(sc, sci) != 0;
     ln.pad = sc.pad;
-    fx_begin<true, EMAX, ZPAD>(s, sc, g, ln, in, mul_out);
+    fx_begin<true, EMAX, ZPAD, true>(s, sc, g, ln, in, mul_out);
     if (fused) {
         fx_rest_of<true, EMAX, false, true>(s, sc, tw, g, ln, FxNoOut{});
         fx_mid_of<EMAX>(s, sc, sci, tw, g, ln, mult, erow);
@@ -265,10 +284,9 @@ __device__ __forceinline__ void fx_convolve(fxc *s, const SC &sc, const SCI &sci
     } else if constexpr (!is_fixed_sched<SC>::value) {
         fx_rest_of<true, EMAX, false, false>(s, sc, tw, g, ln, mul_out);
         group_sync(g);
-        FxFromSmem<false> back;
+        FxFromProducts back;
         back.s = s;
-        back.e = nullptr;
-        back.fold = sc.M;
+        back.m = mult;
         back.e0 = ln.E + erow;
         back.pad = ln.pad;
         fx_transform<false, EMAX, false, CROP>(s, sci, twi, g, ln, back, out);
@@ -303,7 +321,7 @@ __device__ __forceinline__ void fx_body_conv(const FxThread &th, fxc *__restrict
         in.shift = 1;
     }
     const FxMultRow m{mult + row * (full ? M : n + 1), M, full ? 1 : 0};
-    FxLine ln{0, 0, M > kFxLongM, red};
+    FxLine ln{0, 0, M > kFxLongM, red, is3d ? 0 : 1};
     fx_convolve<EMAX, true, true>(s, sc, sci, tw, twi, g, ln, in, m, mrow_exp[row], FxMulToSmem{s, m, &ln},
                                   FxToGlobal{w, n});
     if (g.t == 0) ex.cv[line] = ln.E;
@@ -333,12 +351,11 @@ __device__ __forceinline__ void fx_body_yi(const FxThread &th, const fxc *__rest
     __syncthreads();
     const int z = z0 + l;
     if (z >= nz) return;          // whole groups; no CTA barrier follows
-    FxLine ln{0, 0, M > kFxLongM, red};
+    FxLine ln{0, 0, M > kFxLongM, red, 1};
     FxFromSmem<CG> in;
     in.s = s;
     in.e = ex.cv + (size_t)kx * M;
     in.fold = INT_MAX;
-    in.e0 = 0;
     in.pad = pad;
     fx_transform<false, EMAX, false, true>(s, sc, tw, g, ln, in, FxToGlobal{W1 + ((size_t)z * hx + kx) * ny, ny});
     if (g.t == 0) ex.yi[(size_t)z * hx + kx] = ln.E;
@@ -385,12 +402,11 @@ __device__ __forceinline__ void fx_body_xi(const FxThread &th, const fxc *__rest
     const int ya = y0 + 2 * l;
     if (ya >= ny) return;         // whole groups; no CTA barrier follows
     double *slab = u + (size_t)z * ny * nx;
-    FxLine ln{0, 0, M > kFxLongM, red};
+    FxLine ln{0, 0, M > kFxLongM, red, 0};
     FxFromSmem<CG> in;
     in.s = s;
     in.e = ek;
     in.fold = M;
-    in.e0 = 0;
     in.pad = pad;
     FxToRows out{slab + (size_t)ya * nx, ya + 1 < ny ? slab + (size_t)(ya + 1) * nx : nullptr, nx, &ln};
     fx_transform<false, EMAX, false, true>(s, sc, tw, g, ln, in, out);

@@ -27,3 +27,12 @@ def test_sync_groups_of_the_64r_kernels_have_words_of_their_own(tmp_path):
     word of the shared reduction arrays."""
     out = subprocess.run([compile_host(tmp_path, "fx_host")], check=True, capture_output=True, text=True).stdout
     assert out.split() == ["0"] * 7
+
+
+def test_multiplied_lines_are_no_worse_than_in_doubles(tmp_path):
+    """Maximum error of one multiplied line (smooth, a point, white noise, a wave near Nyquist, a point
+    over a floor, alternating; short and long lines) at most that of a plain FFT in doubles."""
+    out = subprocess.run([compile_host(tmp_path, "fx_accuracy")], check=True, capture_output=True, text=True).stdout
+    lines = [line.split() for line in out.splitlines()]
+    assert len(lines) == 36
+    assert not [line for line in lines if float(line[2]) > float(line[3])], out
