@@ -158,7 +158,7 @@ __device__ __forceinline__ void f3_second(fxc *s, const F3Thread<R> &th, const i
 #pragma unroll
     for (int t = 0; t < 8; ++t) v[t] = fx_ld(p[t * 9 * R]);
 #pragma unroll
-    for (int t = 1; t < 8; ++t) v[t] = fx_rot<FWD>(v[t], w[(t - 1) * 8]);
+    for (int t = 1; t < 8; ++t) v[t] = fx_rot<FWD>(v[t], fx_tw(w + (t - 1) * 8));
     fx_bfly8<FWD, 0>(v);
     th.sync();
     fxc *d = l + 72 * (th.b >> 3) + j;
@@ -177,7 +177,7 @@ __device__ __forceinline__ void f3_last_in(cx<long long> *v, const fxc *l, int b
 #pragma unroll
     for (int t = 0; t < F::RC; ++t) v[t] = fx_ld(p[t * (F::NSC + F::NSC / 8)]);
 #pragma unroll
-    for (int t = 1; t < F::RC; ++t) v[t] = fx_rot<FWD>(v[t], w[(t - 1) * F::NSC]);
+    for (int t = 1; t < F::RC; ++t) v[t] = fx_rot<FWD>(v[t], fx_tw(w + (t - 1) * F::NSC));
 }
 
 // Last stage; out(line, i, t, v) takes output i + t NSC of a line.  CROP: only
@@ -388,7 +388,7 @@ __device__ __forceinline__ void f3_body_conv(fxc *__restrict__ Wd, const int2 *_
 #pragma unroll
         for (int t = 0; t < 8; ++t) x[t] = fx_ld(p[t * (PAD ? 9 * R : 8 * R)]);
 #pragma unroll
-        for (int t = 1; t < 8; ++t) x[t] = fx_rot<false>(x[t], w[(t - 1) * R]);
+        for (int t = 1; t < 8; ++t) x[t] = fx_rot<false>(x[t], fx_tw(w + (t - 1) * R));
         fx_bfly8<false, 0>(x);
         th.sync();
         const int d0 = (th.b - j) * 8 + j;
@@ -405,7 +405,7 @@ __device__ __forceinline__ void f3_body_conv(fxc *__restrict__ Wd, const int2 *_
 #pragma unroll
         for (int t = 0; t < 8; ++t) x[t] = fx_ld(p[t * (P ? 9 * R : 8 * R)]);
 #pragma unroll
-        for (int t = 1; t < 8; ++t) x[t] = fx_rot<false>(x[t], w[(t - 1) * F::NB]);
+        for (int t = 1; t < 8; ++t) x[t] = fx_rot<false>(x[t], fx_tw(w + (t - 1) * F::NB));
         fx_bfly8<false, 2>(x);
         if (r0 + th.line < rows) {
             fxc *o = Wd + (size_t)(base + r0 + th.line) * n + th.b;

@@ -41,7 +41,7 @@ struct FxFromGlobalRot : FxInts {
     __device__ __forceinline__ cx<long long> align(const raw &r, int em, bool longm) const
     {
         const cx<long long> x = FxInts::align({r.v, r.e}, em, longm);
-        return rank ? fx_rot<true>(x, twM[r.i]) : x;
+        return rank ? fx_rot<true>(x, fx_tw(twM + r.i)) : x;
     }
 };
 struct FxHalfToSmem {
@@ -51,7 +51,7 @@ struct FxHalfToSmem {
     int rank;
     __device__ __forceinline__ void operator()(int b, int off, cx<long long> v) const
     {
-        s[pidx<FX>(b + off)] = fx_st(rank ? fx_rot<false>(v, twM[b + off]) : v);
+        s[pidx<FX>(b + off)] = fx_st(rank ? fx_rot<false>(v, fx_tw(twM + b + off)) : v);
     }
 };
 struct FxMultHalf {   // output k' of a half is frequency 2 k' + rank
@@ -132,7 +132,7 @@ struct FxFromRowsRot : FxDoubles {
     __device__ __forceinline__ cx<long long> align(const raw &r, int em, bool longm) const
     {
         const cx<long long> x = FxDoubles::align({r.a, r.b}, em, longm);
-        return rank ? fx_rot<true>(x, twM[r.i]) : x;
+        return rank ? fx_rot<true>(x, fx_tw(twM + r.i)) : x;
     }
 };
 

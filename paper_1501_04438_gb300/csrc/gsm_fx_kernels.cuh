@@ -11,12 +11,12 @@
 // 378, 230 -> 150, 240, 1176, 257, 167; 2D (xf, conv, xi) 1024^2 27, 68, 33 -> 25,
 // 54, 27; 512^2 15, 27, 31 -> 13, 21, 15.
 //
-// They are compiled for the even n up to 256 that are products of 2, 3 and 5, but
-// for the lengths of gsm_fx3.cuh (faster still) and n = 216: its kernels as built
-// by nvcc 13.0 were 1e-10 off where the general ones and the same source on the
-// host are 4e-15 off (all others give the general kernels' bits, and a test holds
-// every one of them to that); and for n = 512 and 1024.  Schedules or launch
-// shapes that were set or tuned to something else keep the general kernels.
+// They are compiled for the even n from 24 to 256 that are products of 2, 3 and 5,
+// but for the lengths of gsm_fx3.cuh (faster still), and for n = 512 and 1024; in
+// two halves (gsm_fx_conv.cu) for n = 2048 and 4096: up to 256 every length a 3D
+// grid usually has, beyond it the powers of two, as each length costs five
+// kernels.  All give the general kernels' bits.  Schedules or launch shapes that
+// were set or tuned to something else keep the general kernels.
 #pragma once
 
 #include "gsm_fx_passes.cuh"
@@ -152,7 +152,7 @@ bool FixedPasses<M>::launch(const FxCall &a, int pass, const PassCfg &c)
 #define GSM_FX_LENGTHS_A(X) X(48) X(60) X(72) X(80) X(96) X(100) X(108)
 #define GSM_FX_LENGTHS_B(X) X(120) X(144) X(160) X(180) X(200)
 #define GSM_FX_LENGTHS_C(X) X(216) X(240) X(288) X(300) X(324)
-#define GSM_FX_LENGTHS_D(X) X(360) X(400) X(480) X(500)
+#define GSM_FX_LENGTHS_D(X) X(360) X(400) X(432) X(480) X(500)
 #define GSM_FX_LENGTHS_E(X) X(1024) X(2048)
 #define GSM_FX_LENGTHS(X) \
     GSM_FX_LENGTHS_A(X) GSM_FX_LENGTHS_B(X) GSM_FX_LENGTHS_C(X) GSM_FX_LENGTHS_D(X) GSM_FX_LENGTHS_E(X)

@@ -2,6 +2,8 @@
 the accuracy of single lines against long double, and what one exponent per
 line has to carry (magnitudes far apart, scaling, zeros, subnormals,
 infinities and NaN)."""
+import struct
+
 import numpy as np
 import pytest
 
@@ -166,3 +168,48 @@ def test_conv_of_several_sync_groups_repeats_its_bits(gsm, N):
     u = plan.apply(r)
     for _ in range(200):
         assert torch.equal(plan.apply(r), u)
+
+
+def _fnv1a(data):
+    h = 14695981039346656037
+    for b in data:
+        h = ((h ^ b) * 1099511628211) & 0xFFFFFFFFFFFFFFFF
+    return h
+
+
+def _resaved(data, **fields):
+    """A saved plan's bytes with header fields replaced: version, nl and emax (one value for every
+    pass)."""
+    b = bytearray(data)
+    if "version" in fields:
+        b[8:12] = struct.pack("<I", fields["version"])
+    for at, key in ((52, "nl"), (72, "emax")):
+        if key in fields:
+            b[at:at + 20] = struct.pack("<5i", *[fields[key]] * 5)
+    b[-8:] = struct.pack("<Q", _fnv1a(b[:-8]))
+    return bytes(b)
+
+
+@pytest.mark.parametrize("nl", [1, 2, 3, 4, 8])
+@pytest.mark.parametrize("n", [(216, 20, 18), (18, 216, 20), (20, 18, 216), (100, 60, 48), (40, 250, 54), (512, 30)],
+                         ids=lambda n: "x".join(map(str, n)))
+def test_lines_per_cta_do_not_change_the_bits(gsm, n, nl):
+    """Compiled-in schedules with every number of lines per CTA (a number that does not fit keeps the
+    default) against the kernels of any schedule, and 16 values per thread, which are those."""
+    import torch
+    kernel = "coulomb3d" if len(n) == 3 else "coulomb2d"
+    r = torch.tensor(np.random.default_rng(nl).standard_normal(n[::-1]), device="cuda")
+    data = gsm.Plan(kernel, 4.0, n).save()
+    u = gsm.Plan(kernel, 4.0, n, debug=4).apply(r)
+    for emax in (8, 16):
+        assert torch.equal(gsm.Plan.load(_resaved(data, nl=nl, emax=emax)).apply(r), u)
+
+
+@pytest.mark.parametrize("n", [(216, 60, 96), (64, 216, 36), (60, 36, 216), (150, 90, 120), (96, 128, 160), (32, 64, 128),
+                               (256, 60, 32), (60, 256, 48), (48, 60, 256)], ids=lambda n: "x".join(map(str, n)))
+def test_larger_grids_have_the_general_kernels_bits(gsm, n):
+    """Many CTAs per pass: compiled-in schedules, and the lengths 64 R whose stages are those of the
+    default schedule (all but n = 192), against the kernels of any schedule."""
+    import torch
+    r = torch.tensor(np.random.default_rng(sum(n)).standard_normal(n[::-1]), device="cuda")
+    assert torch.equal(gsm.Plan("coulomb3d", 4.0, n).apply(r), gsm.Plan("coulomb3d", 4.0, n, debug=4).apply(r))
