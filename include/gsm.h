@@ -249,16 +249,22 @@ gsm_status_t gsm_apply_host(gsm_plan_t p, const void *rho_host, void *u_host, vo
  * Apply `count` plans to their densities in one call: u[i] = U_i * rho[i].
  * (No counterpart in the paper, which treats one density at a time.)
  * Plans may differ in size, kernel and precision (each uses its own I/O type)
- * but must be distinct handles.  Plans whose padded lengths are all <= 512 go
- * through ONE kernel launch per precision and dimension (up to 48 instances
- * per launch) with a device work queue: each CTA of the launch takes the next
- * item (pass, instance, tile) from the queue, in pass-major order, when it
- * starts, and runs it once the instance's previous pass is complete, so the
- * passes of different instances overlap and no launch boundary separates
- * them.  Other plans, and FP32 plans with a
- * padded length of exactly 512 (which use register-resident kernels of their
- * own), are applied one by one on the stream.  The results are the same bits
- * as gsm_apply's.
+ * but must be distinct handles.  Each plan is applied in one of three ways, all of
+ * which give the bits of gsm_apply:
+ *   - through the QUEUE: one kernel launch per precision and dimension (up to 48
+ *     instances per launch) with a device work queue: each CTA of the launch
+ *     takes the next item (pass, instance, tile) from the queue, in pass-major
+ *     order, when it starts, and runs it once the instance's previous pass is
+ *     complete, so the passes of different instances overlap and no launch
+ *     boundary separates them.  FP64 and FP32X2 plans with padded lengths <= 512
+ *     whose transformed half spectrum, (n_x + 1) times the other padded lengths,
+ *     has fewer than 2^18 elements and that have no axis of n = 192; FP32 plans
+ *     with padded lengths <= 512 and no axis of n = 32, 64, 96, 128, 160, 192 or
+ *     256 (whose kernels round differently);
+ *   - in a GROUP: one launch per pass for up to 48 plans of one size (the
+ *     instance is a grid dimension), for other plans all of whose axes are 32,
+ *     64, 96, 128, 160, 192 or (not FP32) 256 with their default schedules;
+ *   - alone, one after another on the stream: all others.
  * Each wait of the queue kernel for a previous pass is bounded (10 s by
  * default): if one runs out, the kernel stops taking work, every CTA returns,
  * and the call reports GSM_ERR_TIMEOUT (the outputs are then not valid).  The
@@ -266,7 +272,7 @@ gsm_status_t gsm_apply_host(gsm_plan_t p, const void *rho_host, void *u_host, vo
  * is a safeguard, never reached in normal operation.
  * The call takes its queue state (about 1 KB per instance) from the stream-
  * ordered allocator, and synchronises `cuda_stream` before it returns, to read
- * the kernel's status.  Errors: as gsm_apply, GSM_ERR_OOM, GSM_ERR_TIMEOUT;
+ * the queue's status.  Errors: as gsm_apply, GSM_ERR_OOM, GSM_ERR_TIMEOUT;
  * nothing is launched if any argument is invalid.
  */
 gsm_status_t gsm_apply_batched(int count, const gsm_plan_t *plans, const void *const *rho,
@@ -274,7 +280,7 @@ gsm_status_t gsm_apply_batched(int count, const gsm_plan_t *plans, const void *c
 
 /*
  * The same batched apply recorded once into a CUDA graph (a memset of the
- * queue state and the queue launches), so that every later run is a
+ * queue state and the launches), so that every later run is a
  * single cudaGraphLaunch.  The graph holds the given rho[i] and u[i] pointers
  * and each plan's workspace: refill the same rho arrays between launches; the
  * plans must outlive the batch, and no other apply may be in flight on them

@@ -30,17 +30,11 @@ void launch_f32_stage_twiddles(const Sched &sc, float2 *out, cudaStream_t st)
     k_f32_stage_twiddles<<<(sc.M + 127) / 128, 128, 0, st>>>(sc, out);
 }
 
-template cudaError_t f3f_raise_smem<1>(const Plan *p);
-template void f3f_launch<1>(const Plan *, int, const float *, float *, float2 *, int, cudaStream_t);
-template cudaError_t f3f_raise_smem<2>(const Plan *p);
-template void f3f_launch<2>(const Plan *, int, const float *, float *, float2 *, int, cudaStream_t);
-template cudaError_t f3f_raise_smem<3>(const Plan *p);
-template void f3f_launch<3>(const Plan *, int, const float *, float *, float2 *, int, cudaStream_t);
-template cudaError_t f3f_raise_smem<4>(const Plan *p);
-template void f3f_launch<4>(const Plan *, int, const float *, float *, float2 *, int, cudaStream_t);
-template cudaError_t f3f_raise_smem<5>(const Plan *p);
-template void f3f_launch<5>(const Plan *, int, const float *, float *, float2 *, int, cudaStream_t);
-template cudaError_t f3f_raise_smem<6>(const Plan *p);
-template void f3f_launch<6>(const Plan *, int, const float *, float *, float2 *, int, cudaStream_t);
+template void f3f_launch<1>(const F3Call &c, int pass);
+template void f3f_launch<2>(const F3Call &c, int pass);
+template void f3f_launch<3>(const F3Call &c, int pass);
+template void f3f_launch<4>(const F3Call &c, int pass);
+template void f3f_launch<5>(const F3Call &c, int pass);
+template void f3f_launch<6>(const F3Call &c, int pass);
 
 }  // namespace gsm

@@ -167,10 +167,12 @@ struct F3F {
 };
 
 // ------------------------------------------------------------------ passes
-template <int R>
+template <int R, int COUNT>
 __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
-    k_f3f_xf(const float *__restrict__ rho, float2 *__restrict__ W1, int ny, const float2 *__restrict__ tw)
+    k_f3f_xf(const __grid_constant__ F3Group<COUNT> g, int ny, const float2 *__restrict__ tw)
 {
+    const float *__restrict__ rho = static_cast<const float *>(g.at().rho);
+    float2 *__restrict__ W1 = static_cast<float2 *>(g.at().W1);
     using F = F3<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *s = reinterpret_cast<float2 *>(smem_raw);
@@ -198,10 +200,12 @@ __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
     }
 }
 
-template <int R>
+template <int R, int COUNT>
 __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
-    k_f3f_yf(const float2 *__restrict__ W1, float2 *__restrict__ W2, int nz, int hx, const float2 *__restrict__ tw)
+    k_f3f_yf(const __grid_constant__ F3Group<COUNT> g, int nz, int hx, const float2 *__restrict__ tw)
 {
+    const float2 *__restrict__ W1 = static_cast<const float2 *>(g.at().W1);
+    float2 *__restrict__ W2 = static_cast<float2 *>(g.at().W2);
     using F = F3<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *s = reinterpret_cast<float2 *>(smem_raw);
@@ -223,11 +227,13 @@ __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
 }
 
 // twi: the table of the inverse (R 8 8)
-template <int R, bool IS3D>
+template <int R, bool IS3D, int COUNT>
 __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
-    k_f3f_conv(float2 *__restrict__ Wd, const float *__restrict__ mult, int rows, int ny1,
-               const float2 *__restrict__ tw, const float2 *__restrict__ twi, int full)
+    k_f3f_conv(const __grid_constant__ F3Group<COUNT> g, int rows, int ny1, const float2 *__restrict__ tw,
+               const float2 *__restrict__ twi, int full)
 {
+    float2 *__restrict__ Wd = static_cast<float2 *>(IS3D ? g.at().W2 : g.at().W1);
+    const float *__restrict__ mult = static_cast<const float *>(g.at().mult);
     using F = F3<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *s = reinterpret_cast<float2 *>(smem_raw);
@@ -301,10 +307,12 @@ __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
     }
 }
 
-template <int R>
+template <int R, int COUNT>
 __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
-    k_f3f_yi(const float2 *__restrict__ W2, float2 *__restrict__ W1, int nz, int hx, const float2 *__restrict__ tw)
+    k_f3f_yi(const __grid_constant__ F3Group<COUNT> g, int nz, int hx, const float2 *__restrict__ tw)
 {
+    const float2 *__restrict__ W2 = static_cast<const float2 *>(g.at().W2);
+    float2 *__restrict__ W1 = static_cast<float2 *>(g.at().W1);
     using F = F3<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *s = reinterpret_cast<float2 *>(smem_raw);
@@ -334,10 +342,12 @@ __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
     });
 }
 
-template <int R>
+template <int R, int COUNT>
 __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
-    k_f3f_xi(const float2 *__restrict__ W1, float *__restrict__ u, int ny, const float2 *__restrict__ tw)
+    k_f3f_xi(const __grid_constant__ F3Group<COUNT> g, int ny, const float2 *__restrict__ tw)
 {
+    const float2 *__restrict__ W1 = static_cast<const float2 *>(g.at().W1);
+    float *__restrict__ u = static_cast<float *>(g.at().u);
     using F = F3<R>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float2 *s = reinterpret_cast<float2 *>(smem_raw);
@@ -379,53 +389,44 @@ __global__ void __launch_bounds__(F3<R>::THREADS, F3F<R>::CTAS)
 
 }  // namespace
 
-template <int R>
-cudaError_t f3f_raise_smem(const Plan *p)
-{
-    constexpr size_t smem = F3F<R>::SMEM;
-    cudaError_t e = cudaSuccess;
-    auto chk = [&](cudaError_t x) { if (e == cudaSuccess) e = x; };
-    if (p->M[0] == F3<R>::M) {
-        chk(raise_smem(k_f3f_xf<R>, smem));
-        chk(raise_smem(k_f3f_xi<R>, smem));
-    }
-    if (p->d == 3 && p->M[1] == F3<R>::M) {
-        chk(raise_smem(k_f3f_yf<R>, smem));
-        chk(raise_smem(k_f3f_yi<R>, smem));
-    }
-    if (p->M[p->d - 1] == F3<R>::M)
-        chk(p->d == 3 ? raise_smem(k_f3f_conv<R, true>, smem) : raise_smem(k_f3f_conv<R, false>, smem));
-    return e;
-}
-
 // One pass (see f3_launch); the stage-ordered tables follow the M plain twiddles.
-template <int R>
-void f3f_launch(const Plan *p, int pass, const float *rho, float *u, float2 *W1, int nz, cudaStream_t st)
+template <int R, int COUNT>
+void f3f_launch_group(const F3Call &c, int pass)
 {
     using F = F3<R>;
     constexpr size_t smem = F3F<R>::SMEM;
+    static_assert(smem <= 48 * 1024, "no raised shared-memory limit");
+    F3Group<COUNT> g{};
+    for (int i = 0; i < c.count; ++i) g.inst[i] = c.inst[i];
+    const Plan *p = c.p;
     const int last = p->d == 3 ? 4 : 2, conv = p->d == 3 ? 2 : 1;
-    const int ny = p->n[1], hx = p->n[0] + 1, full = p->mult_full ? 1 : 0;
+    const int ny = p->n[1], hx = p->n[0] + 1, nz = c.nz, full = p->mult_full ? 1 : 0;
     const int axis = pass == 0 || pass == last ? 0 : pass == conv ? p->d - 1 : 1;
     const float2 *tw = static_cast<const float2 *>(p->d_tw[axis]) + F::M;
     const float2 *twi = static_cast<const float2 *>(p->d_twi[axis]) + F::M;
-    const float *mult = static_cast<const float *>(p->d_mult);
-    float2 *W2 = static_cast<float2 *>(p->d_work2);
-    const dim3 gx((ny + 2 * F::NL - 1) / (2 * F::NL), nz), gy((nz + F::NL - 1) / F::NL, hx);
+    const dim3 gx((ny + 2 * F::NL - 1) / (2 * F::NL), nz, c.count), gy((nz + F::NL - 1) / F::NL, hx, c.count);
     if (pass == 0) {
-        k_f3f_xf<R><<<gx, F::THREADS, smem, st>>>(rho, W1, ny, tw);
+        k_f3f_xf<R, COUNT><<<gx, F::THREADS, smem, c.st>>>(g, ny, tw);
     } else if (pass == last) {
-        k_f3f_xi<R><<<gx, F::THREADS, smem, st>>>(W1, u, ny, twi);
+        k_f3f_xi<R, COUNT><<<gx, F::THREADS, smem, c.st>>>(g, ny, twi);
     } else if (pass == conv && p->d == 3) {
         const int My = p->M[1];
-        k_f3f_conv<R, true><<<dim3((My + F::NL - 1) / F::NL, hx), F::THREADS, smem, st>>>(W2, mult, My, ny + 1, tw, twi, full);
+        k_f3f_conv<R, true, COUNT><<<dim3((My + F::NL - 1) / F::NL, hx, c.count), F::THREADS, smem, c.st>>>(
+            g, My, ny + 1, tw, twi, full);
     } else if (pass == conv) {
-        k_f3f_conv<R, false><<<(hx + F::NL - 1) / F::NL, F::THREADS, smem, st>>>(W1, mult, hx, ny + 1, tw, twi, full);
+        k_f3f_conv<R, false, COUNT><<<dim3((hx + F::NL - 1) / F::NL, 1, c.count), F::THREADS, smem, c.st>>>(
+            g, hx, ny + 1, tw, twi, full);
     } else if (pass == 1) {
-        k_f3f_yf<R><<<gy, F::THREADS, smem, st>>>(W1, W2, nz, hx, tw);
+        k_f3f_yf<R, COUNT><<<gy, F::THREADS, smem, c.st>>>(g, nz, hx, tw);
     } else {
-        k_f3f_yi<R><<<gy, F::THREADS, smem, st>>>(W2, W1, nz, hx, twi);
+        k_f3f_yi<R, COUNT><<<gy, F::THREADS, smem, c.st>>>(g, nz, hx, twi);
     }
+}
+template <int R>
+void f3f_launch(const F3Call &c, int pass)
+{
+    if (c.count == 1) f3f_launch_group<R, 1>(c, pass);
+    else f3f_launch_group<R, kF3Group>(c, pass);
 }
 
 }  // namespace gsm

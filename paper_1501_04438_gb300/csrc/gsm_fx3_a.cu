@@ -3,9 +3,7 @@
 
 namespace gsm {
 
-template cudaError_t f3_raise_smem<8>(const Plan *p);
-template void f3_launch<8>(const FxCall &c, int pass);
-template cudaError_t f3_raise_smem<5>(const Plan *p);
-template void f3_launch<5>(const FxCall &c, int pass);
+template void f3_launch<8>(const F3Call &c, int pass);
+template void f3_launch<5>(const F3Call &c, int pass);
 
 }  // namespace gsm

@@ -3,9 +3,7 @@
 
 namespace gsm {
 
-template cudaError_t f3_raise_smem<6>(const Plan *p);
-template void f3_launch<6>(const FxCall &c, int pass);
-template cudaError_t f3_raise_smem<4>(const Plan *p);
-template void f3_launch<4>(const FxCall &c, int pass);
+template void f3_launch<6>(const F3Call &c, int pass);
+template void f3_launch<4>(const F3Call &c, int pass);
 
 }  // namespace gsm

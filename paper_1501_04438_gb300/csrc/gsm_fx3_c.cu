@@ -3,11 +3,8 @@
 
 namespace gsm {
 
-template cudaError_t f3_raise_smem<3>(const Plan *p);
-template void f3_launch<3>(const FxCall &c, int pass);
-template cudaError_t f3_raise_smem<2>(const Plan *p);
-template void f3_launch<2>(const FxCall &c, int pass);
-template cudaError_t f3_raise_smem<1>(const Plan *p);
-template void f3_launch<1>(const FxCall &c, int pass);
+template void f3_launch<3>(const F3Call &c, int pass);
+template void f3_launch<2>(const F3Call &c, int pass);
+template void f3_launch<1>(const F3Call &c, int pass);
 
 }  // namespace gsm

@@ -143,6 +143,24 @@ struct FxCall {
     int nz;
     cudaStream_t st;
 };
+// One pass of plans of one size on the kernels of the lengths 64 R: `count`
+// instances, one grid layer each, that differ in their arrays only.
+constexpr int kF3Group = 48;
+struct F3Inst {
+    const void *rho;
+    void *u;
+    void *W1, *W2;
+    const void *mult;
+    const int *mrow;   // fixed point: exponents of the multiplier's rows
+    FxExps ex;         // fixed point: line exponents
+};
+struct F3Call {
+    const Plan *p;     // sizes and tables of all of them
+    const F3Inst *inst;
+    int count;         // 1 .. kF3Group
+    int nz;
+    cudaStream_t st;
+};
 // Launch of a pass, of the split 2D passes, of the FFT hook; shared-memory
 // limits of their kernels; twiddle tables (gsm_fx.cu, gsm_fx_conv.cu).
 void fx_launch_xy(const FxCall &c, int pass, const PassCfg &cfg);
@@ -155,14 +173,10 @@ cudaError_t fx_raise_conv_smem(const Plan *p, const PassCfg &c);
 cudaError_t fx_raise_split_smem(bool conv, size_t smem);
 // the passes of padded lengths 64 R, R = 1, 2, 3, 4, 5, 6, 8 (gsm_fx3.cuh)
 template <int R>
-cudaError_t f3_raise_smem(const Plan *p);
-template <int R>
-void f3_launch(const FxCall &c, int pass);
+void f3_launch(const F3Call &c, int pass);
 // the same in FP32 (gsm_f3_f32.cuh), R <= 6
 template <int R>
-cudaError_t f3f_raise_smem(const Plan *p);
-template <int R>
-void f3f_launch(const Plan *p, int pass, const float *rho, float *u, float2 *W1, int nz, cudaStream_t st);
+void f3f_launch(const F3Call &c, int pass);
 // w^(j t) of a schedule's stages in stage order (fx_stage_table), FP32 (gsm_f3_f32.cu)
 void launch_f32_stage_twiddles(const Sched &sc, float2 *out, cudaStream_t st);
 size_t fx_table_bytes(int M, int plain);

@@ -696,11 +696,6 @@ gsm_status_t configure_t(Plan *p)
         const PassCfg *c[3] = {&p->cfg_xf, &p->cfg_conv, &p->cfg_xi};
         for (int pass = 0; pass < 3; ++pass) chk(raise_pass_smem<Pol>(p, pass, *c[pass]));
     }
-    for (int a = 0; a < d; ++a)
-        with_f3(p->M[a], [&](auto R) {
-            if constexpr (std::is_same<Pol, FX>::value) chk(f3_raise_smem<R()>(p));
-            else if constexpr (R() != 8) chk(f3f_raise_smem<R()>(p));
-        });
     GSM_CUDA_TRY(e);
     // workspace
     const size_t cb = sizeof(S_t<Pol>);
@@ -739,12 +734,23 @@ void with_f3(int M, F &&f)
     default: break;
     }
 }
-// FP32: R <= 6 (n = 256 has the register-resident kernels)
-void launch_f3f(const Plan *p, int pass, const float *rho, float *u, float2 *W1, int nz, cudaStream_t st)
+// What the kernels of the lengths 64 R take of plan p, and one of its passes on
+// them; FP32: R <= 6 (n = 256 has the register-resident kernels).
+F3Inst f3_inst(const Plan *p, const void *rho, void *u)
 {
-    with_f3(pass_len(p, pass), [&](auto R) {
-        if constexpr (R() != 8) f3f_launch<R()>(p, pass, rho, u, W1, nz, st);
+    return {rho, u, p->d_work1, p->d_work2, p->d_mult, p->d_mrow, p->opt.precision == GSM_FP32 ? FxExps() : fx_exps(p)};
+}
+void launch_f3(const F3Call &c, int pass)
+{
+    with_f3(pass_len(c.p, pass), [&](auto R) {
+        if (c.p->opt.precision != GSM_FP32) f3_launch<R()>(c, pass);
+        else if constexpr (R() != 8) f3f_launch<R()>(c, pass);
     });
+}
+void launch_f3(const Plan *p, int pass, const void *rho, void *u, cudaStream_t st)
+{
+    const F3Inst inst = f3_inst(p, rho, u);
+    launch_f3({p, &inst, 1, p->d == 3 ? p->n[2] : 1, st}, pass);
 }
 
 void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cudaStream_t st)
@@ -765,7 +771,7 @@ void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cuda
     const tw *twyi = static_cast<const tw *>(p->d_twi[1]);
     const int last = p->d == 3 ? 4 : 2;
     if (pass_uses_f3(p, pass)) {
-        launch_f3f(p, pass, rho, u, W1, nz, st);
+        launch_f3(p, pass, rho, u, st);
         return;
     }
     if constexpr (std::is_same<Pol, F32>::value) {
@@ -865,7 +871,7 @@ void launch_pass_fx(const Plan *p, int pass, const void *rho, void *u, cudaStrea
     const FxCall c{p,           fx_exps(p),   static_cast<const double *>(rho), static_cast<double *>(u), p->d_work1,
                    p->d_work2, p->d == 3 ? p->n[2] : 1, st};
     const int conv = p->d == 3 ? 2 : 1;
-    if (pass_uses_f3(p, pass)) with_f3(pass_len(p, pass), [&](auto R) { f3_launch<R()>(c, pass); });
+    if (pass_uses_f3(p, pass)) launch_f3(p, pass, rho, u, st);
     else if (pass_is_split(p, pass)) fx_launch_split(c, pass);
     else if (pass == conv) fx_launch_conv(c, p->cfg_conv);
     else fx_launch_xy(c, pass, *pass_cfg(const_cast<Plan *>(p), pass));
@@ -1619,25 +1625,26 @@ gsm_status_t x_slabs_t(const Plan *p, bool inverse, int z0, int z1, const void *
     const tw *twx = static_cast<const tw *>(p->d_tw[0]);
     const tw *twxi = static_cast<const tw *>(p->d_twi[0]);
     if (z1 <= z0) return GSM_OK;
+    if (pass_uses_f3(p, inverse ? 4 : 0)) {
+        F3Inst inst = f3_inst(p, static_cast<const io *>(rho_v) + in_off, static_cast<io *>(u_v) + in_off);
+        inst.W1 = W1;
+        if constexpr (std::is_same<Pol, FX>::value) {
+            inst.ex.xf += (size_t)z0 * ((ny + 1) / 2);
+            inst.ex.yi += (size_t)z0 * hx;
+        }
+        launch_f3({p, &inst, 1, z1 - z0, st}, inverse ? 4 : 0);
+        GSM_CUDA_TRY(cudaGetLastError());
+        return GSM_OK;
+    }
     if constexpr (std::is_same<Pol, FX>::value) {
         FxCall c{p, fx_exps(p), static_cast<const io *>(rho_v) + in_off, static_cast<io *>(u_v) + in_off, W1, nullptr,
                  z1 - z0, st};
         c.ex.xf += (size_t)z0 * ((ny + 1) / 2);
         c.ex.yi += (size_t)z0 * hx;
-        const int pass = inverse ? 4 : 0;
-        if (pass_uses_f3(p, pass)) with_f3(p->M[0], [&](auto R) { f3_launch<R()>(c, pass); });
-        else fx_launch_xy(c, pass, inverse ? p->cfg_xi : p->cfg_xf);
+        fx_launch_xy(c, inverse ? 4 : 0, inverse ? p->cfg_xi : p->cfg_xf);
         GSM_CUDA_TRY(cudaGetLastError());
         return GSM_OK;
     } else {
-    if constexpr (std::is_same<Pol, F32>::value) {
-        const int pass = inverse ? 4 : 0;
-        if (pass_uses_f3(p, pass)) {
-            launch_f3f(p, pass, static_cast<const io *>(rho_v) + in_off, static_cast<io *>(u_v) + in_off, W1, z1 - z0, st);
-            GSM_CUDA_TRY(cudaGetLastError());
-            return GSM_OK;
-        }
-    }
     if constexpr (std::is_same<Pol, F32>::value) {
         if (p->M[0] == 512 && p->rr_conv) {
             if (!inverse) launch_x_rr512_f32(false, static_cast<const io *>(rho_v) + in_off, W1, ny, z1 - z0, twx, st);
@@ -1848,19 +1855,44 @@ gsm_status_t launch_fft_lines_noalloc(int M, int nlines, int sign, gsm_precision
 // ------------------------------------------------------------------ grouped batch, host side
 namespace {
 
-bool batch_eligible(const Plan *p)
+// How a batch applies a plan.
+enum class BatchWay { queue, group, alone };
+
+// Padded elements of the conv pass below which a fixed-point plan goes to the
+// queue: 48 instances through the queue against one after another, FP64, 24^3 (6e4)
+// 0.83 / 1.43 ms, 32^3 (1.4e5) 1.10 / 1.76, 2D 256^2 (1.3e5) 0.43 / 1.42, but
+// 48^3 (4.5e5) 2.76 / 2.07, 64^3 (1.1e6) 4.7 / 2.8, 100^3 17.7 / 11.9: the queue's
+// kernel runs the transforms of any length, and from there on its one launch
+// saves less than the kernels of fixed lengths do.
+constexpr size_t kQueueMaxElems = 1 << 18;
+
+// Every way gives the bits of gsm_apply.  The queue does for lengths whose kernels
+// of their own run the same operations as those of any length: fixed point but for
+// n = 192 (stages 8 8 6 instead of 8 8 2 3), FP32 only where there are no such
+// kernels.  Plans all of whose passes run on the kernels of the lengths 64 R are
+// grouped by size, one launch per pass and size.
+BatchWay batch_way(const Plan *p)
 {
-    for (int a = 0; a < p->d; ++a) {
-        if (p->M[a] > kBatchMaxM) return false;
-        // FP32 plans that use the register-resident kernels apply alone, so that
-        // a batch gives the same bits as gsm_apply
-        if (p->opt.precision == GSM_FP32 && p->rr_conv && p->M[a] == 512) return false;
-    }
-    // nor do plans with a pass on the fixed-length kernels, for speed
+    const bool fp32 = p->opt.precision == GSM_FP32;
     const int np = p->d == 3 ? 5 : 3;
-    for (int pass = 0; pass < np; ++pass)
-        if (pass_uses_f3(p, pass)) return false;
-    return true;
+    bool queue = true, all_f3 = true, some_f3 = false;
+    for (int a = 0; a < p->d; ++a)
+        if (p->M[a] > kBatchMaxM || (fp32 && p->rr_conv && p->M[a] == 512)) queue = false;
+    for (int pass = 0; pass < np; ++pass) {
+        const bool f3 = pass_uses_f3(p, pass);
+        all_f3 &= f3;
+        some_f3 |= f3;
+        if (f3 && f3_radix(pass_len(p, pass)) == 6) queue = false;
+    }
+    const size_t conv = (size_t)(p->n[0] + 1) * p->M[1] * (p->d == 3 ? p->M[2] : 1);
+    if (fp32 ? some_f3 : conv >= kQueueMaxElems) queue = false;
+    return queue ? BatchWay::queue : all_f3 ? BatchWay::group : BatchWay::alone;
+}
+// whether two plans may be in one group: the same launches but for the arrays
+bool same_f3_group(const Plan *a, const Plan *b)
+{
+    return a->d == b->d && a->n[0] == b->n[0] && a->n[1] == b->n[1] && a->n[2] == b->n[2] &&
+           (a->opt.precision == GSM_FP32) == (b->opt.precision == GSM_FP32) && a->mult_full == b->mult_full;
 }
 
 // Tile grid of pass `pass` of plan p for lines-per-CTA nl: (gx, gy).
@@ -1920,8 +1952,8 @@ gsm_status_t launch_queue_t(QueueArgs &a, const std::vector<const Plan *> &plans
             d.tw[ax] = ax < p->d ? p->d_tw[ax] : nullptr;
             d.twi[ax] = ax < p->d ? p->d_twi[ax] : nullptr;
             if (ax < p->d) {
-                d.sc[ax] = p->sched_f[ax];
-                d.sci[ax] = p->sched_i[ax];
+                d.sc[ax] = run_sched(p, ax, false);   // what the tables are made for
+                d.sci[ax] = run_sched(p, ax, true);
             }
             if (ax < p->d) smem = std::max(smem, pass_smem<Pol>(p->M[ax], a.nl));
         }
@@ -1959,9 +1991,9 @@ void set_batch_wait(unsigned long long wait_ns, int hold)
     g_batch_hold.store(hold < 0 ? -1 : hold);
 }
 
-// u[i] = U_i * rho[i]: plans with all padded lengths <= 512 are grouped by
-// (precision, dimension) into queue launches (k_batch_queue) of up to
-// kBatchMax instances; the others are applied one by one.  Group g keeps its queue
+// u[i] = U_i * rho[i]: each plan the way batch_way says, queue launches
+// (k_batch_queue) by (precision, dimension) of up to kBatchMax instances, launches
+// of up to kF3Group plans of one size, or alone.  Queue launch g keeps its queue
 // state at state + g * kStateWords (batch_state_bytes(count) bytes in all,
 // zeroed here first).  dry: only prepare the kernels (shared-memory limits),
 // launch nothing.
@@ -1973,17 +2005,30 @@ gsm_status_t launch_batched(int count, const Plan *const *plans, const void *con
     int group = 0;
     for (int i = 0; i < count; ++i) {
         if (done[i]) continue;
-        if (!batch_eligible(plans[i])) {
+        const BatchWay way = batch_way(plans[i]);
+        if (way == BatchWay::alone) {
             gsm_status_t s = dry ? GSM_OK : launch_apply(plans[i], rho[i], u[i], st);
             if (s != GSM_OK) return s;
             done[i] = 1;
+            continue;
+        }
+        if (way == BatchWay::group) {
+            std::vector<F3Inst> inst;
+            for (int j = i; j < count && (int)inst.size() < kF3Group; ++j) {
+                if (done[j] || batch_way(plans[j]) != BatchWay::group || !same_f3_group(plans[i], plans[j])) continue;
+                inst.push_back(f3_inst(plans[j], rho[j], u[j]));
+                done[j] = 1;
+            }
+            const F3Call c{plans[i], inst.data(), (int)inst.size(), plans[i]->d == 3 ? plans[i]->n[2] : 1, st};
+            for (int pass = 0; !dry && pass < (c.p->d == 3 ? 5 : 3); ++pass) launch_f3(c, pass);
+            GSM_CUDA_TRY(cudaGetLastError());
             continue;
         }
         std::vector<const Plan *> grp;
         std::vector<const void *> r;
         std::vector<void *> w;
         for (int j = i; j < count && (int)grp.size() < kBatchMax; ++j) {
-            if (done[j] || !batch_eligible(plans[j])) continue;
+            if (done[j] || batch_way(plans[j]) != BatchWay::queue) continue;
             if (plans[j]->opt.precision != plans[i]->opt.precision || plans[j]->d != plans[i]->d) continue;
             grp.push_back(plans[j]);
             r.push_back(rho[j]);
