@@ -1198,6 +1198,20 @@ float time_pass(const Plan *p, int pass, const void *rho, void *u, cudaStream_t 
     return ms / 3.f;
 }
 
+// The density that candidates are timed on: white noise in [-1, 1).  On zeros the
+// fixed-point passes would skip the shifts that bring a line into range.
+template <class T>
+__global__ void k_noise(T *rho, size_t N)
+{
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
+        unsigned h = (unsigned)i * 2654435761u;
+        h ^= h >> 15;
+        h *= 2246822519u;
+        h ^= h >> 13;
+        rho[i] = (T)((double)(int)h * 0x1p-31);
+    }
+}
+
 template <class Pol>
 gsm_status_t autotune_t(Plan *p, cudaStream_t st, std::string *report)
 {
@@ -1208,7 +1222,8 @@ gsm_status_t autotune_t(Plan *p, cudaStream_t st, std::string *report)
     GSM_CUDA_TRY(dev_alloc(&rho_buf.p, N * sizeof(io)));
     GSM_CUDA_TRY(dev_alloc(&u_buf.p, N * sizeof(io)));
     void *rho = rho_buf.p, *u = u_buf.p;
-    GSM_CUDA_TRY(cudaMemsetAsync(rho, 0, N * sizeof(io), st));
+    k_noise<<<1024, 256, 0, st>>>(static_cast<io *>(rho), N);
+    GSM_CUDA_TRY(cudaGetLastError());
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
