@@ -331,8 +331,11 @@ gsm_status_t gsm_plan_info(gsm_plan_t p, gsm_plan_info_t *info);
  * twiddles and workspace are rebuilt on `cuda_stream`.  precision < 0 keeps
  * the saved precision (and its launch shapes and schedules); GSM_FP64 /
  * GSM_FP32 / GSM_FP32X2 reuse the same FP64 tensor for another pass precision
- * with default launch shapes and schedules.  The result equals the saved plan bit for bit.  A
- * wrong magic, version, size or checksum: GSM_ERR_INVALID_ARG, *out = NULL.
+ * with default launch shapes and schedules.  The result equals the saved plan bit
+ * for bit within one version of the format: plans saved in version 3, whose FP64
+ * and FP32X2 arithmetic was another, are read, but in those precisions with default
+ * launch shapes and schedules.  A wrong magic, version, size or checksum:
+ * GSM_ERR_INVALID_ARG, *out = NULL.
  * The format is native little-endian; the caller owns buf.
  */
 gsm_status_t gsm_plan_save(gsm_plan_t p, void *buf, size_t capacity, size_t *bytes);

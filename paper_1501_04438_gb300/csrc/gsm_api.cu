@@ -330,7 +330,11 @@ gsm_status_t gsm_plan(gsm_plan_t *out, gsm_kernel_t kind, int d, double L, const
 // Gaussian sum (w, tau), the FP64 octant kernel tensor, then a 64-bit FNV-1a
 // checksum of everything before it.
 static const uint64_t kSaveMagic = 0x47534d5341564531ull;   // "GSMSAVE1"
-static const uint32_t kSaveVersion = 3;
+// Version 4 has the layout of version 3.  The shapes and schedules of version 3
+// were chosen for FP64 and float-pair arithmetic, and a conv inverse in engine order
+// was their default: with them a fixed-point plan would run the kernels of any
+// length, so it takes its own defaults.
+static const uint32_t kSaveVersion = 4, kSaveVersionFloating = 3;
 
 struct SaveHeader {
     uint64_t magic;
@@ -438,7 +442,8 @@ gsm_status_t gsm_plan_load(gsm_plan_t *out, const void *buf, size_t bytes, int p
         return GSM_ERR_INVALID_ARG;
     }
     memcpy(&hd, b, sizeof(hd));
-    if (hd.magic != kSaveMagic || hd.version != kSaveVersion || hd.header_bytes != sizeof(SaveHeader)) {
+    if (hd.magic != kSaveMagic || (hd.version != kSaveVersion && hd.version != kSaveVersionFloating) ||
+        hd.header_bytes != sizeof(SaveHeader)) {
         set_error("saved plan: not a plan of this format version");
         return GSM_ERR_INVALID_ARG;
     }
@@ -500,7 +505,8 @@ gsm_status_t gsm_plan_load(gsm_plan_t *out, const void *buf, size_t bytes, int p
     if (s != GSM_OK) return s;
     Plan *p = reinterpret_cast<Plan *>(h);
     p->eps = hd.eps;
-    if (o.precision == hd.precision && hd.npasses == (hd.d == 3 ? 5 : 3)) {
+    const bool shaped = hd.version == kSaveVersion || o.precision == GSM_FP32;
+    if (shaped && o.precision == hd.precision && hd.npasses == (hd.d == 3 ? 5 : 3)) {
         // the saved (possibly tuned) launch shapes; a shape this device
         // cannot run keeps the default
         for (int i = 0; i < hd.npasses; ++i)

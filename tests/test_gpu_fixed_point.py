@@ -215,3 +215,16 @@ def test_larger_grids_have_the_general_kernels_bits(gsm, n):
     r = torch.tensor(np.random.default_rng(sum(n)).standard_normal(n[::-1]), device="cuda")
     kernel = "coulomb3d" if len(n) == 3 else "coulomb2d"
     assert torch.equal(gsm.Plan(kernel, 4.0, n).apply(r), gsm.Plan(kernel, 4.0, n, debug=4).apply(r))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32x2", "fp32"])
+def test_plans_saved_before_fixed_point(gsm, precision):
+    """A plan saved in format version 3 with the schedules of that time (on the conv axis forward and
+    inverse alike) is read; in fixed point it takes the default schedules, FP32 keeps the stored ones."""
+    n = (100, 24, 18)
+    plan = gsm.Plan("coulomb3d", 4.0, n, precision=precision)
+    fresh = plan.info()
+    plan.set_schedule(0, [4, 2, 5, 5])
+    loaded = gsm.Plan.load(_resaved(plan.save(), version=3)).info()
+    assert loaded["radix_fwd"][0] == (plan.info() if precision == "fp32" else fresh)["radix_fwd"][0]
+    assert gsm.Plan.load(plan.save()).info()["radix_fwd"][0] == plan.info()["radix_fwd"][0]
