@@ -64,8 +64,11 @@ typedef enum {
 
 /* Arithmetic of the FFT passes and of the multiplier product.
  *   GSM_FP64   : block fixed point, 64-bit integers with one exponent per
- *                transformed line, whose errors are those of IEEE double
- *                arithmetic or less.           I/O: double.
+ *                transformed line.  Its errors, as a maximum over the grid
+ *                relative to the largest |u|, are those of IEEE double
+ *                arithmetic or less: measured against extended precision on
+ *                smooth, random, single-point and oscillating densities.
+ *                                              I/O: double.
  *   GSM_FP32   : IEEE single.                  I/O: float.
  *   GSM_FP32X2 : computed as GSM_FP64 (at least the 48 bits that pairs of
  *                floats would give).           I/O: double.
@@ -103,9 +106,14 @@ typedef struct {
                                    in every pass even where the register-resident kernels
                                    apply (padded length 512); bit 1 set: 2D plans with a
                                    padded y (x) length >= 4096 transform each conv (x
-                                   forward) line on one CTA instead of two half-length
+                                   forward, but for FP32 x inverse) line on one CTA
+                                   instead of two half-length
                                    transforms on a CTA pair (for comparisons; same results
-                                   to rounding) */
+                                   to rounding); bit 2 set: every pass on the kernels of
+                                   any length instead of those with the length compiled
+                                   in (for comparisons; FP64 and FP32X2 equal bits but
+                                   for n = 192, FP32 equal to rounding).  Not saved with
+                                   a plan */
     double box[3];              /* rectangular box (Sec. 2.5, Eq. tensor_ani): if all
                                    d entries are > 0, axis a spans [-box[a], box[a]]
                                    and L is ignored; all 0 (default): [-L, L]^d.  The
@@ -223,7 +231,12 @@ gsm_status_t gsm_plan_autotune(gsm_plan_t p, void *cuda_stream, char *report, si
  * tables for that axis are rebuilt on
  * `cuda_stream` (synchronised when an old table is freed).  FP32 passes with
  * a padded length of 512 use register-resident kernels of fixed shape and
- * ignore the schedule.  Same plan rules as gsm_apply.  Errors:
+ * ignore the schedule.  Passes of the padded lengths 64 R, R = 1 to 6 and (not
+ * FP32) 8, whose schedule is the default one (gsm_plan_info reports it; on the conv
+ * axis the inverse may be in engine order too) run kernels of fixed stages 8 8 R
+ * and fixed shape, whatever launch shape the plan holds; any other schedule runs
+ * as it was set.  FP64 and FP32X2: the results are those of the reported schedule
+ * but for R = 6 (8 8 6 for 8 8 2 3, equal to rounding).  Same plan rules as gsm_apply.  Errors:
  * GSM_ERR_BAD_PLAN, GSM_ERR_INVALID_ARG (bad axis or schedule), GSM_ERR_OOM.
  */
 gsm_status_t gsm_plan_set_schedule(gsm_plan_t p, int axis, int inverse, const int *radices, int count,
