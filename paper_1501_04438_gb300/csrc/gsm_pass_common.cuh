@@ -43,8 +43,8 @@ __device__ __forceinline__ T ldw(const T *p)
 // Copies `count` elements into shared memory with U global loads in flight
 // per thread (all U loads are issued before the first store waits for its
 // data): for i = t, t + T, ... < count, dst(i, src(i)).  The short FP32 passes
-// wait on these loads: U = 4 against 1, with the line fixed per thread instead
-// of a division per element, 2D 1500x648 98.8 -> 96.5 us.
+// wait on these loads: 2D 1500x648 takes 98.8 us with U = 1 and a division per
+// element, 96.5 with U = 4 and the line fixed per thread.
 template <int U, class Val, class Src, class Dst>
 __device__ __forceinline__ void gather_smem(int t, int T, int count, Src src, Dst dst)
 {

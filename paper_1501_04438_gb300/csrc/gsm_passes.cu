@@ -774,17 +774,15 @@ void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cuda
         launch_f3(p, pass, rho, u, st);
         return;
     }
-    if constexpr (std::is_same<Pol, F32>::value) {
-        if ((pass == 0 || pass == last) && p->M[0] == 512 && p->rr_conv) {
-            if (pass == 0) launch_x_rr512_f32(false, rho, W1, ny, nz, twx, st);
-            else launch_x_rr512_f32(true, W1, u, ny, nz, twx, st);
-            return;
-        }
+    if ((pass == 0 || pass == last) && p->M[0] == 512 && p->rr_conv) {
+        if (pass == 0) launch_x_rr512_f32(false, rho, W1, ny, nz, twx, st);
+        else launch_x_rr512_f32(true, W1, u, ny, nz, twx, st);
+        return;
     }
     if (pass == 0 && p->split_x) {
         const PassCfg &c = p->cfg_xsplit;
         const tw *twh = static_cast<const tw *>(p->d_twxh);
-            k_xf_split<Pol, 16><<<2 * ((ny + 1) / 2), c.nthr, c.smem, st>>>(rho, W1, nx, ny, hx, p->sched_xh, twh, twx);
+        k_xf_split<Pol, 16><<<2 * ((ny + 1) / 2), c.nthr, c.smem, st>>>(rho, W1, nx, ny, hx, p->sched_xh, twh, twx);
         return;
     }
     if (pass == 0) {
@@ -801,34 +799,30 @@ void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cuda
         });
     } else if (p->d == 2) {
         const PassCfg &c = p->cfg_conv;
-        if constexpr (std::is_same<Pol, F32>::value) {
-            if (p->M[1] == 512 && p->rr_conv) {
-                launch_conv_rr512_f32(W1, mult, hx, 0, 1, ny + 1, p->mult_full, twy, st);
-                return;
-            }
+        if (p->M[1] == 512 && p->rr_conv) {
+            launch_conv_rr512_f32(W1, mult, hx, 0, 1, ny + 1, p->mult_full, twy, st);
+            return;
         }
         if (p->split_conv) {
             const PassCfg &cs = p->cfg_split;
             const tw *th = static_cast<const tw *>(p->d_twh), *thi = static_cast<const tw *>(p->d_twhi);
             k_conv_split<Pol, 16><<<2 * hx, cs.nthr, cs.smem, st>>>(W1, mult, hx, ny + 1, p->sched_hf, p->sched_hi,
-                                                                        th, thi, twy, p->mult_full ? 1 : 0);
+                                                                    th, thi, twy, p->mult_full ? 1 : 0);
             return;
         }
         with_emax(c, [&](auto E) {
             k_conv<Pol, E()><<<(hx + c.nl - 1) / c.nl, c.nthr, c.smem, st>>>(
-                    W1, mult, hx, ny, 0, 1, ny + 1, p->sched_f[1], p->sched_i[1], c.nl, c.gthr, twy, twyi,
-                    p->mult_full ? 1 : 0);
+                W1, mult, hx, ny, 0, 1, ny + 1, p->sched_f[1], p->sched_i[1], c.nl, c.gthr, twy, twyi,
+                p->mult_full ? 1 : 0);
         });
     } else {
         const tw *twz = static_cast<const tw *>(p->d_tw[2]);
         const tw *twzi = static_cast<const tw *>(p->d_twi[2]);
         const int My = p->M[1];
         if (pass == 1) {
-            if constexpr (std::is_same<Pol, F32>::value) {
-                if (p->M[1] == 512 && p->rr_conv) {
-                    launch_y_rr512_f32(false, W1, W2, nz, hx, twy, st);
-                    return;
-                }
+            if (p->M[1] == 512 && p->rr_conv) {
+                launch_y_rr512_f32(false, W1, W2, nz, hx, twy, st);
+                return;
             }
             const PassCfg &c = p->cfg_yf;
             dim3 g((nz + c.nl - 1) / c.nl, hx);
@@ -838,23 +832,19 @@ void launch_pass_f32(const Plan *p, int pass, const void *rho_v, void *u_v, cuda
         } else if (pass == 2) {
             const PassCfg &c = p->cfg_conv;
             const int nlines = hx * My;
-            if constexpr (std::is_same<Pol, F32>::value) {
-                if (p->M[2] == 512 && p->rr_conv) {
-                    launch_conv_rr512_f32(W2, mult, nlines, 1, My, ny + 1, p->mult_full, twz, st);
-                    return;
-                }
+            if (p->M[2] == 512 && p->rr_conv) {
+                launch_conv_rr512_f32(W2, mult, nlines, 1, My, ny + 1, p->mult_full, twz, st);
+                return;
             }
             with_emax(c, [&](auto E) {
                 k_conv<Pol, E()><<<(nlines + c.nl - 1) / c.nl, c.nthr, c.smem, st>>>(
-                        W2, mult, nlines, nz, 1, My, ny + 1, p->sched_f[2], p->sched_i[2], c.nl, c.gthr, twz, twzi,
-                        p->mult_full ? 1 : 0);
+                    W2, mult, nlines, nz, 1, My, ny + 1, p->sched_f[2], p->sched_i[2], c.nl, c.gthr, twz, twzi,
+                    p->mult_full ? 1 : 0);
             });
         } else {
-            if constexpr (std::is_same<Pol, F32>::value) {
-                if (p->M[1] == 512 && p->rr_conv) {
-                    launch_y_rr512_f32(true, W2, W1, nz, hx, twy, st);
-                    return;
-                }
+            if (p->M[1] == 512 && p->rr_conv) {
+                launch_y_rr512_f32(true, W2, W1, nz, hx, twy, st);
+                return;
             }
             const PassCfg &c = p->cfg_yi;
             dim3 g((nz + c.nl - 1) / c.nl, hx);
@@ -1660,31 +1650,29 @@ gsm_status_t x_slabs_t(const Plan *p, bool inverse, int z0, int z1, const void *
         GSM_CUDA_TRY(cudaGetLastError());
         return GSM_OK;
     } else {
-    if constexpr (std::is_same<Pol, F32>::value) {
         if (p->M[0] == 512 && p->rr_conv) {
             if (!inverse) launch_x_rr512_f32(false, static_cast<const io *>(rho_v) + in_off, W1, ny, z1 - z0, twx, st);
             else launch_x_rr512_f32(true, W1, static_cast<io *>(u_v) + in_off, ny, z1 - z0, twx, st);
             GSM_CUDA_TRY(cudaGetLastError());
             return GSM_OK;
         }
-    }
-    if (!inverse) {
-        const PassCfg &c = p->cfg_xf;
-        dim3 g((ny + 2 * c.nl - 1) / (2 * c.nl), z1 - z0);
-        const io *rho = static_cast<const io *>(rho_v) + in_off;
-        with_emax(c, [&](auto E) {
-            k_xf<Pol, E()><<<g, c.nthr, c.smem, st>>>(rho, W1, nx, ny, hx, p->sched_f[0], c.nl, c.gthr, twx);
-        });
-    } else {
-        const PassCfg &c = p->cfg_xi;
-        dim3 g((ny + 2 * c.nl - 1) / (2 * c.nl), z1 - z0);
-        io *u = static_cast<io *>(u_v) + in_off;
-        with_emax(c, [&](auto E) {
-            k_xi<Pol, E()><<<g, c.nthr, c.smem, st>>>(W1, u, nx, ny, hx, p->sched_i[0], c.nl, c.gthr, twxi);
-        });
-    }
-    GSM_CUDA_TRY(cudaGetLastError());
-    return GSM_OK;
+        if (!inverse) {
+            const PassCfg &c = p->cfg_xf;
+            dim3 g((ny + 2 * c.nl - 1) / (2 * c.nl), z1 - z0);
+            const io *rho = static_cast<const io *>(rho_v) + in_off;
+            with_emax(c, [&](auto E) {
+                k_xf<Pol, E()><<<g, c.nthr, c.smem, st>>>(rho, W1, nx, ny, hx, p->sched_f[0], c.nl, c.gthr, twx);
+            });
+        } else {
+            const PassCfg &c = p->cfg_xi;
+            dim3 g((ny + 2 * c.nl - 1) / (2 * c.nl), z1 - z0);
+            io *u = static_cast<io *>(u_v) + in_off;
+            with_emax(c, [&](auto E) {
+                k_xi<Pol, E()><<<g, c.nthr, c.smem, st>>>(W1, u, nx, ny, hx, p->sched_i[0], c.nl, c.gthr, twxi);
+            });
+        }
+        GSM_CUDA_TRY(cudaGetLastError());
+        return GSM_OK;
     }
 }
 
