@@ -936,7 +936,8 @@ std::string tune_key(const Plan *p, int pass)
     for (char &ch : name)
         if (ch == ' ') ch = '_';
     char buf[256];
-    snprintf(buf, sizeof(buf), "v5 %s p%d d%d n%d,%d,%d pass%d", name.c_str(), (int)p->opt.precision, p->d, p->n[0],
+    // (the version: entries of another were timed on other kernels or another density)
+    snprintf(buf, sizeof(buf), "v6 %s p%d d%d n%d,%d,%d pass%d", name.c_str(), (int)p->opt.precision, p->d, p->n[0],
              p->n[1], p->d == 3 ? p->n[2] : 1, pass);
     return buf;
 }

@@ -228,3 +228,15 @@ def test_plans_saved_before_fixed_point(gsm, precision):
     loaded = gsm.Plan.load(_resaved(plan.save(), version=3)).info()
     assert loaded["radix_fwd"][0] == (plan.info() if precision == "fp32" else fresh)["radix_fwd"][0]
     assert gsm.Plan.load(plan.save()).info()["radix_fwd"][0] == plan.info()["radix_fwd"][0]
+
+
+def test_tuned_choices_of_another_version_are_not_used(gsm, tmp_path, monkeypatch):
+    """Entries of the tuner's cache are used again by the version that wrote them and by no other."""
+    cache = tmp_path / "tune.txt"
+    monkeypatch.setenv("GSM_AUTOTUNE_CACHE", str(cache))
+    n = (54, 40, 36)
+    assert "cached" not in gsm.Plan("coulomb3d", 4.0, n).autotune()
+    entries = cache.read_text()
+    assert entries.startswith("v6 ") and gsm.Plan("coulomb3d", 4.0, n).autotune().count(" cached ") == 5
+    cache.write_text(entries.replace("v6 ", "v5 "))
+    assert "cached" not in gsm.Plan("coulomb3d", 4.0, n).autotune()
