@@ -17,13 +17,14 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libgsm.so")
-SOURCES = ["gsm_api.cu", "gsm_plan.cu", "gsm_passes.cu", "gsm_fx.cu", "gsm_fx_conv.cu", "gsm_fx_len_a.cu", "gsm_fx_len_b.cu",
-           "gsm_fx_len_c.cu", "gsm_fx_len_d.cu", "gsm_fx_len_e.cu", "gsm_fx_queue2d.cu",
-           "gsm_fx_queue3d.cu", "gsm_fx3_a.cu", "gsm_fx3_b.cu", "gsm_fx3_c.cu", "gsm_f3_f32.cu",
-           "gsm_conv_rr.cu", "gsm_tc.cu"]
-HEADERS = ["gsm_arith.cuh", "gsm_fft.cuh", "gsm_fx.cuh", "gsm_fx_passes.cuh", "gsm_fx_kernels.cuh", "gsm_fx3.cuh", "gsm_f3_f32.cuh", "gsm_fx_queue.cuh", "gsm_pass_common.cuh", "gsm_internal.h"]
+# the units that take longest to compile first
+SOURCES = [*(f"gsm_fx_split_{u}.cu" for u in "abcde"), *(f"gsm_fx_len_{u}.cu" for u in "abcdefghijkl"), "gsm_passes.cu",
+           "gsm_fx_queue3d.cu", "gsm_fx_queue2d.cu", "gsm_fx3_c.cu", "gsm_fx3_a.cu", "gsm_fx3_b.cu", "gsm_f3_f32.cu",
+           "gsm_fx.cu", "gsm_fx_conv.cu", "gsm_conv_rr.cu", "gsm_tc.cu", "gsm_plan.cu", "gsm_api.cu"]
+HEADERS = ["gsm_arith.cuh", "gsm_fft.cuh", "gsm_fx.cuh", "gsm_fx_passes.cuh", "gsm_fx_kernels.cuh", "gsm_fx_split.cuh",
+           "gsm_fx3.cuh", "gsm_f3_f32.cuh", "gsm_fx_queue.cuh", "gsm_pass_common.cuh", "gsm_internal.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
+FLAGS = ["-O3", "-lineinfo", "--compress-mode=size", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
 def nvcc() -> str:

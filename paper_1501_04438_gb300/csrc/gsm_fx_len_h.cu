@@ -1,0 +1,7 @@
+// gsm_fx_len_h.cu -- fixed-point passes of padded lengths known at compile time (gsm_fx_kernels.cuh).
+#define GSM_FX_LENGTH_UNIT
+#include "gsm_fx_kernels.cuh"
+
+namespace gsm {
+GSM_FX_LENGTHS_H(GSM_FX_DEFINE)
+}  // namespace gsm

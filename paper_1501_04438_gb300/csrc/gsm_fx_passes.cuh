@@ -44,16 +44,16 @@ __device__ __forceinline__ FxThread fx_thread()
     th.tid = threadIdx.y * blockDim.x + threadIdx.x;
     return th;
 }
-// the same for a schedule known at compile time: 8 values per thread
-template <class SC>
-constexpr int fixed_threads() { return ((SC::M + 7) / 8 + 31) / 32 * 32; }
-template <class SC>
+// the same for a schedule known at compile time
+template <class SC, int EMAX>
+constexpr int fixed_threads() { return ((SC::M + EMAX - 1) / EMAX + 31) / 32 * 32; }
+template <class SC, int EMAX>
 __device__ __forceinline__ FxThread fx_thread_of()
 {
     FxThread th = fx_thread();
     if constexpr (is_fixed_sched<SC>::value) {
-        th.g.T = fixed_threads<SC>();
-        if (fixed_threads<SC>() == 32) th.g.bar = -1;
+        th.g.T = fixed_threads<SC, EMAX>();
+        if (fixed_threads<SC, EMAX>() == 32) th.g.bar = -1;
     }
     return th;
 }

@@ -170,7 +170,7 @@ cudaError_t fx_launch_hook(const PassCfg &c, int nlines, int sign, const Sched &
                            const void *tw, cudaStream_t st);
 cudaError_t fx_raise_smem(const Plan *p, int pass, const PassCfg &c);
 cudaError_t fx_raise_conv_smem(const Plan *p, const PassCfg &c);
-cudaError_t fx_raise_split_smem(bool conv, size_t smem);
+cudaError_t fx_raise_split_smem(bool conv, int half, size_t smem);
 // the passes of padded lengths 64 R, R = 1, 2, 3, 4, 5, 6, 8 (gsm_fx3.cuh)
 template <int R>
 void f3_launch(const F3Call &c, int pass);

@@ -621,9 +621,9 @@ cudaError_t raise_pass_smem(const Plan *p, int pass, const PassCfg &c)
     }
 }
 template <class Pol>
-cudaError_t raise_split_smem(bool conv, size_t smem)
+cudaError_t raise_split_smem(bool conv, int half, size_t smem)
 {
-    if constexpr (std::is_same<Pol, FX>::value) return fx_raise_split_smem(conv, smem);
+    if constexpr (std::is_same<Pol, FX>::value) return fx_raise_split_smem(conv, half, smem);
     else if (conv) return raise_smem(k_conv_split<Pol, 16>, smem);
     else return raise_smem(k_xf_split<Pol, 16>, smem);
 }
@@ -675,7 +675,7 @@ gsm_status_t configure_t(Plan *p)
                 set_error("no launch shape for the split conv pass");
                 return GSM_ERR_UNSUPPORTED_SIZE;
             }
-            GSM_CUDA_TRY(raise_split_smem<Pol>(true, p->cfg_split.smem));
+            GSM_CUDA_TRY(raise_split_smem<Pol>(true, p->M[1] / 2, p->cfg_split.smem));
         }
         // the same for the x forward pass
         p->split_x = p->M[0] >= kSplitMinM && p->M[0] == 2 * p->n[0] && (p->opt.debug & 2) == 0;
@@ -684,7 +684,7 @@ gsm_status_t configure_t(Plan *p)
                 set_error("no launch shape for the split x pass");
                 return GSM_ERR_UNSUPPORTED_SIZE;
             }
-            GSM_CUDA_TRY(raise_split_smem<Pol>(false, p->cfg_xsplit.smem));
+            GSM_CUDA_TRY(raise_split_smem<Pol>(false, p->M[0] / 2, p->cfg_xsplit.smem));
         }
     }
     cudaError_t e = cudaSuccess;

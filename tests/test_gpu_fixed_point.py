@@ -240,3 +240,33 @@ def test_tuned_choices_of_another_version_are_not_used(gsm, tmp_path, monkeypatc
     assert entries.startswith("v6 ") and gsm.Plan("coulomb3d", 4.0, n).autotune().count(" cached ") == 5
     cache.write_text(entries.replace("v6 ", "v5 "))
     assert "cached" not in gsm.Plan("coulomb3d", 4.0, n).autotune()
+
+
+LONG = sorted(n for n in (2 ** a * 3 ** b * 5 ** c for a in range(1, 13) for b in range(8) for c in range(6))
+              if 256 < n <= 4096)
+
+
+@pytest.mark.parametrize("n", LONG)
+def test_long_lengths_have_the_general_kernels_bits(gsm, n):
+    """Compiled-in schedules of the lengths over 256, whole lines and (from 2048 on) half lines, as x and
+    y of 2D grids and, up to 512, as x and z of 3D grids, against the kernels of any schedule."""
+    import torch
+    rng = np.random.default_rng(n)
+    grids = [(n, 18), (20, n)] + ([(n, 8, 10), (8, 10, n)] if n <= 512 else [])
+    for g in grids:
+        kernel = "coulomb3d" if len(g) == 3 else "poisson2d"
+        r = torch.tensor(rng.standard_normal(g[::-1]), device="cuda")
+        assert torch.equal(gsm.Plan(kernel, 4.0, g).apply(r), gsm.Plan(kernel, 4.0, g, debug=4).apply(r)), g
+
+
+@pytest.mark.parametrize("nl", [1, 2, 3, 4])
+@pytest.mark.parametrize("n", [(320, 54), (54, 750), (1080, 40), (40, 2000)], ids=lambda n: "x".join(map(str, n)))
+def test_lines_per_cta_of_long_lengths(gsm, n, nl):
+    """The same with every number of lines per CTA, with 8 and (padded lengths over 2048) 16 values
+    per thread."""
+    import torch
+    r = torch.tensor(np.random.default_rng(nl).standard_normal(n[::-1]), device="cuda")
+    data = gsm.Plan("coulomb2d", 4.0, n).save()
+    u = gsm.Plan("coulomb2d", 4.0, n, debug=4).apply(r)
+    for emax in (8, 16):
+        assert torch.equal(gsm.Plan.load(_resaved(data, nl=nl, emax=emax)).apply(r), u)
