@@ -186,8 +186,12 @@ __device__ __forceinline__ void body_conv(S_t<Pol> *__restrict__ W, const typena
     for (int z = g.t; z < n; z += g.T) w[z] = s[pidx<Pol>(z)];
 }
 
+// Registers: with 56 an SM holds three CTAs of 384 threads (M = 80 with 12 lines, M =
+// 1536, M = 3000), with the 61 that the compiler takes by itself two.  Conv pass in us
+// with 61, 56, 48, 40: 768^2 36.9, 26.6, 26.6, 26.7; 648x1500 67.6, 55.3, 55.3, 57.3; 1536^2
+// 106.5, 88.1, 88.1, 86.0; 1500x648 69.6, 69.6, 69.6, 75.8; 300x48x40 73.0, 61.5, 61.4, 61.4.
 template <class Pol, int EMAX>
-__global__ void __launch_bounds__(kMaxThreads)
+__global__ void __maxnreg__(EMAX == 8 ? 56 : 80)
     k_conv(S_t<Pol> *__restrict__ W, const typename Pol::mult_t *__restrict__ mult,
                                                       int nlines, int n, int is3d, int My, int ny1, Sched sc,
                                                       Sched sci, int nl, int gthr,
