@@ -271,13 +271,17 @@ gsm_status_t gsm_apply_host(gsm_plan_t p, const void *rho_host, void *u_host, vo
  *     complete, so the passes of different instances overlap and no launch
  *     boundary separates them.  FP64 and FP32X2 plans with padded lengths <= 512
  *     whose transformed half spectrum, (n_x + 1) times the other padded lengths,
- *     has fewer than 2^18 elements and that have no axis of n = 192; FP32 plans
- *     with padded lengths <= 512 and no axis of n = 32, 64, 96, 128, 160, 192 or
- *     256 (whose kernels round differently);
+ *     has fewer than 2^16 (3D) or 2^18 (2D) elements and that have no axis of n =
+ *     192; FP32 plans with padded lengths <= 512 and no axis of n = 32, 64, 96, 128,
+ *     160, 192 or 256 (whose kernels round differently);
  *   - in a GROUP: one launch per pass for up to 48 plans of one size (the
- *     instance is a grid dimension), for other plans all of whose axes are 32,
- *     64, 96, 128, 160, 192 or (not FP32) 256 with their default schedules;
- *   - alone, one after another on the stream: all others.
+ *     instance is a grid dimension), for plans all of whose axes are 32, 64, 96, 128,
+ *     160, 192 or (not FP32) 256 with their default schedules: those not fit for the
+ *     queue, and those that are from four of one size on;
+ *   - alone: all others, one after another on the stream, or, with a half spectrum of
+ *     fewer than 2^23 elements, on up to four streams of the call's own, which start
+ *     where `cuda_stream` is and which it waits for.
+ * No u[i] may be another instance's rho or u.
  * Each wait of the queue kernel for a previous pass is bounded (10 s by
  * default): if one runs out, the kernel stops taking work, every CTA returns,
  * and the call reports GSM_ERR_TIMEOUT (the outputs are then not valid).  The

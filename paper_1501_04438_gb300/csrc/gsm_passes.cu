@@ -1867,34 +1867,40 @@ namespace {
 enum class BatchWay { queue, group, alone };
 
 // Padded elements of the conv pass below which a fixed-point plan goes to the
-// queue: 48 instances through the queue against one after another, FP64, 24^3 (6e4)
-// 0.83 / 1.43 ms, 32^3 (1.4e5) 1.10 / 1.76, 2D 256^2 (1.3e5) 0.43 / 1.42, but
-// 48^3 (4.5e5) 2.76 / 2.07, 64^3 (1.1e6) 4.7 / 2.8, 100^3 17.7 / 11.9: the queue's
-// kernel runs the transforms of any length, and from there on its one launch
-// saves less than the kernels of fixed lengths do.
-constexpr size_t kQueueMaxElems = 1 << 18;
+// queue: its kernel runs the transforms of any length, and from there on one launch
+// saves less than the kernels of compiled-in lengths do.  Through the queue against
+// alone on four streams (Fork), FP64, ms: 3D, 48 of 16^3 (1.7e4 elements) 0.45 / 0.91, 24^3
+// (5.8e4) 0.93 / 0.80, 32 of four sizes about 32^3 (1.3e5) 0.96 / 0.61; 2D, with three
+// passes instead of five, 48 of 200^2 (8e4) 0.56 / 0.84, 16 of 100x250 (5e4) 0.30 / 0.37.
+constexpr size_t queue_max_elems(int d) { return d == 3 ? 1 << 16 : 1 << 18; }
+
+size_t conv_elems(const Plan *p) { return (size_t)(p->n[0] + 1) * p->M[1] * (p->d == 3 ? p->M[2] : 1); }
 
 // Every way gives the bits of gsm_apply.  The queue does for lengths whose kernels
 // of their own run the same operations as those of any length: fixed point but for
 // n = 192 (stages 8 8 6 instead of 8 8 2 3), FP32 only where there are no such
 // kernels.  Plans all of whose passes run on the kernels of the lengths 64 R are
-// grouped by size, one launch per pass and size.
+// grouped by size, one launch per pass and size (batch_ways: from kGroupMin plans on
+// before the queue).
+BatchWay group_way(const Plan *p)
+{
+    for (int pass = 0; pass < (p->d == 3 ? 5 : 3); ++pass)
+        if (!pass_uses_f3(p, pass)) return BatchWay::alone;
+    return BatchWay::group;
+}
 BatchWay batch_way(const Plan *p)
 {
     const bool fp32 = p->opt.precision == GSM_FP32;
     const int np = p->d == 3 ? 5 : 3;
-    bool queue = true, all_f3 = true, some_f3 = false;
+    bool some_f3 = false, r6 = false;
     for (int a = 0; a < p->d; ++a)
-        if (p->M[a] > kBatchMaxM || (fp32 && p->rr_conv && p->M[a] == 512)) queue = false;
+        if (p->M[a] > kBatchMaxM || (fp32 && p->rr_conv && p->M[a] == 512)) return group_way(p);
     for (int pass = 0; pass < np; ++pass) {
         const bool f3 = pass_uses_f3(p, pass);
-        all_f3 &= f3;
         some_f3 |= f3;
-        if (f3 && f3_radix(pass_len(p, pass)) == 6) queue = false;
+        r6 |= f3 && f3_radix(pass_len(p, pass)) == 6;
     }
-    const size_t conv = (size_t)(p->n[0] + 1) * p->M[1] * (p->d == 3 ? p->M[2] : 1);
-    if (fp32 ? some_f3 : conv >= kQueueMaxElems) queue = false;
-    return queue ? BatchWay::queue : all_f3 ? BatchWay::group : BatchWay::alone;
+    return r6 || (fp32 ? some_f3 : conv_elems(p) >= queue_max_elems(p->d)) ? group_way(p) : BatchWay::queue;
 }
 // whether two plans may be in one group: the same launches but for the arrays
 bool same_f3_group(const Plan *a, const Plan *b)
@@ -1902,6 +1908,79 @@ bool same_f3_group(const Plan *a, const Plan *b)
     return a->d == b->d && a->n[0] == b->n[0] && a->n[1] == b->n[1] && a->n[2] == b->n[2] &&
            (a->opt.precision == GSM_FP32) == (b->opt.precision == GSM_FP32) && a->mult_full == b->mult_full;
 }
+
+// The ways of a batch's plans: plans that may be grouped are, from kGroupMin of one
+// size on, also where they could go through the queue, whose kernel runs the
+// transforms of any length: 48 plans grouped against queued, FP64, ms: 32^3 0.40 / 1.16,
+// 2D 64^2 0.25 / 0.32, 256^2 0.38 / 0.52.  (Fewer cost a launch per pass and size.)
+constexpr int kGroupMin = 4;
+std::vector<BatchWay> batch_ways(int count, const Plan *const *plans)
+{
+    std::vector<BatchWay> way(count);
+    std::vector<int> can;   // queue or group
+    for (int i = 0; i < count; ++i) {
+        way[i] = batch_way(plans[i]);
+        if (way[i] == BatchWay::queue && group_way(plans[i]) == BatchWay::group) can.push_back(i);
+    }
+    while (!can.empty()) {   // one size after another
+        std::vector<int> same, rest;
+        for (int i : can) (same_f3_group(plans[can[0]], plans[i]) ? same : rest).push_back(i);
+        if ((int)same.size() >= kGroupMin)
+            for (int i : same) way[i] = BatchWay::group;
+        can.swap(rest);
+    }
+    return way;
+}
+
+// Streams beside the caller's, for plans that are applied alone and do not fill the
+// GPU: forked from the caller's stream and joined to it again within the call (or
+// the capture), so that every order the caller sees is that of its own stream.  One
+// after another against on four streams, ms: FP32, 32 of four sizes about 32^3 0.97 ->
+// 0.52, 8 of 64x36x48 0.50 -> 0.35, 6 of 324^2 0.38 -> 0.26; FP64, 48 of 48^3 2.29 -> 1.24, 16
+// of 100^3 3.95 -> 3.43, 4 of 2000^2 (8e6 elements) 3.00 -> 2.65.  Four of 200x128x160
+// (1.6e7) fill the GPU each (2.5).
+constexpr size_t kForkMaxElems = 1 << 23;
+struct Fork {
+    static constexpr int kStreams = 4;
+    cudaStream_t s[kStreams] = {};
+    cudaEvent_t start = nullptr, done[kStreams] = {};
+    int n = 0;   // 0: there are none
+    ~Fork()
+    {
+        for (cudaStream_t t : s)
+            if (t) cudaStreamDestroy(t);   // once what was queued on it has finished
+        for (cudaEvent_t e : done)
+            if (e) cudaEventDestroy(e);
+        if (start) cudaEventDestroy(start);
+    }
+    // up to `want` streams that go on where st is; on failure everything stays on st
+    cudaError_t open(cudaStream_t st, int want)
+    {
+        const int k = std::min(want, kStreams);
+        bool made = k > 1 && cudaEventCreateWithFlags(&start, cudaEventDisableTiming) == cudaSuccess;
+        for (int i = 0; i < k && made; ++i)
+            made = cudaStreamCreateWithFlags(&s[i], cudaStreamNonBlocking) == cudaSuccess &&
+                   cudaEventCreateWithFlags(&done[i], cudaEventDisableTiming) == cudaSuccess;
+        if (!made) {
+            cudaGetLastError();
+            return cudaSuccess;
+        }
+        cudaError_t e = cudaEventRecord(start, st);
+        for (; n < k && e == cudaSuccess; ++n) e = cudaStreamWaitEvent(s[n], start, 0);
+        return e;
+    }
+    cudaError_t join(cudaStream_t st)
+    {
+        cudaError_t e = cudaSuccess;
+        for (int i = 0; i < n; ++i) {
+            cudaError_t x = cudaEventRecord(done[i], s[i]);
+            if (x == cudaSuccess) x = cudaStreamWaitEvent(st, done[i], 0);
+            if (e == cudaSuccess) e = x;
+        }
+        n = 0;
+        return e;
+    }
+};
 
 // Tile grid of pass `pass` of plan p for lines-per-CTA nl: (gx, gy).
 void pass_grid(const Plan *p, int pass, int nl, int *gx, int *gy)
@@ -1999,21 +2078,15 @@ void set_batch_wait(unsigned long long wait_ns, int hold)
     g_batch_hold.store(hold < 0 ? -1 : hold);
 }
 
-// u[i] = U_i * rho[i]: each plan the way batch_way says, queue launches
-// (k_batch_queue) by (precision, dimension) of up to kBatchMax instances, launches
-// of up to kF3Group plans of one size, or alone.  Queue launch g keeps its queue
-// state at state + g * kStateWords (batch_state_bytes(count) bytes in all,
-// zeroed here first).  dry: only prepare the kernels (shared-memory limits),
-// launch nothing.
-gsm_status_t launch_batched(int count, const Plan *const *plans, const void *const *rho, void *const *u,
-                            int nl, cudaStream_t st, bool dry, unsigned *state)
+namespace {
+// The plans that are not done yet.
+gsm_status_t launch_rest(int count, const Plan *const *plans, const void *const *rho, void *const *u, int nl,
+                         cudaStream_t st, bool dry, unsigned *state, const std::vector<BatchWay> &ways, std::vector<int> &done)
 {
-    if (!dry) GSM_CUDA_TRY(cudaMemsetAsync(state, 0, batch_state_bytes(count), st));
-    std::vector<int> done(count, 0);
     int group = 0;
     for (int i = 0; i < count; ++i) {
         if (done[i]) continue;
-        const BatchWay way = batch_way(plans[i]);
+        const BatchWay way = ways[i];
         if (way == BatchWay::alone) {
             gsm_status_t s = dry ? GSM_OK : launch_apply(plans[i], rho[i], u[i], st);
             if (s != GSM_OK) return s;
@@ -2023,7 +2096,7 @@ gsm_status_t launch_batched(int count, const Plan *const *plans, const void *con
         if (way == BatchWay::group) {
             std::vector<F3Inst> inst;
             for (int j = i; j < count && (int)inst.size() < kF3Group; ++j) {
-                if (done[j] || batch_way(plans[j]) != BatchWay::group || !same_f3_group(plans[i], plans[j])) continue;
+                if (done[j] || ways[j] != BatchWay::group || !same_f3_group(plans[i], plans[j])) continue;
                 inst.push_back(f3_inst(plans[j], rho[j], u[j]));
                 done[j] = 1;
             }
@@ -2036,7 +2109,7 @@ gsm_status_t launch_batched(int count, const Plan *const *plans, const void *con
         std::vector<const void *> r;
         std::vector<void *> w;
         for (int j = i; j < count && (int)grp.size() < kBatchMax; ++j) {
-            if (done[j] || batch_way(plans[j]) != BatchWay::queue) continue;
+            if (done[j] || ways[j] != BatchWay::queue) continue;
             if (plans[j]->opt.precision != plans[i]->opt.precision || plans[j]->d != plans[i]->d) continue;
             grp.push_back(plans[j]);
             r.push_back(rho[j]);
@@ -2061,6 +2134,39 @@ gsm_status_t launch_batched(int count, const Plan *const *plans, const void *con
         delete a;
         if (s != GSM_OK) return s;
     }
+    return GSM_OK;
+}
+}  // namespace
+
+// u[i] = U_i * rho[i]: each plan the way batch_way says, queue launches
+// (k_batch_queue) by (precision, dimension) of up to kBatchMax instances, launches
+// of up to kF3Group plans of one size, or alone, small ones on streams beside st
+// (Fork).  Queue launch g keeps its queue
+// state at state + g * kStateWords (batch_state_bytes(count) bytes in all,
+// zeroed here first).  dry: only prepare the kernels (shared-memory limits),
+// launch nothing.
+gsm_status_t launch_batched(int count, const Plan *const *plans, const void *const *rho, void *const *u,
+                            int nl, cudaStream_t st, bool dry, unsigned *state)
+{
+    if (!dry) GSM_CUDA_TRY(cudaMemsetAsync(state, 0, batch_state_bytes(count), st));
+    const std::vector<BatchWay> ways = batch_ways(count, plans);
+    std::vector<int> done(count, 0), small;
+    for (int i = 0; i < count && !dry; ++i)
+        if (ways[i] == BatchWay::alone && conv_elems(plans[i]) < kForkMaxElems) small.push_back(i);
+    Fork fork;
+    cudaError_t forked = fork.open(st, (int)small.size());
+    gsm_status_t alone = GSM_OK;
+    for (int k = 0; k < (int)small.size() && fork.n > 0 && forked == cudaSuccess && alone == GSM_OK; ++k) {
+        const int i = small[k];
+        alone = launch_apply(plans[i], rho[i], u[i], fork.s[k % fork.n]);
+        done[i] = 1;
+    }
+    gsm_status_t s = alone;
+    if (s == GSM_OK && forked == cudaSuccess) s = launch_rest(count, plans, rho, u, nl, st, dry, state, ways, done);
+    const cudaError_t joined = fork.join(st);
+    if (s != GSM_OK) return s;
+    GSM_CUDA_TRY(forked);
+    GSM_CUDA_TRY(joined);
     return GSM_OK;
 }
 
