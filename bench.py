@@ -145,18 +145,37 @@ def apply_model(n: int, cbytes: int):
     return float(flops), float(bytes_)
 
 
-def kernel_source_hash():
-    """Hash of the source that fixes the conv kernel's memory traffic: the FFT
-    engine and arithmetic headers and the conv section of the pass file."""
+# real-arithmetic work of a butterfly of each radix: complex additions (all inputs / half of the
+# inputs or outputs), products by constants
+RADIX_ADDS = {2: (2, 0), 4: (8, 4), 8: (24, 16), 3: (6, 6), 5: (17, 17)}
+RADIX_PRODUCTS = {2: 0, 4: 0, 8: 4, 3: 2, 5: 8}
+
+
+def conv_pass_int_model(n: int):
+    """32-bit integer instructions that the fixed-point conv pass cannot do without: additions of
+    complex 64-bit integers (4), products by a constant or a multiplier entry (3 multiply-adds, 1 to
+    split, 6 to join) and by a twiddle (12, 2 and 12, 4 negations); no addresses, loads, stores or
+    scaling.  One padded transform forward, one inverse."""
+    M, total = 2 * n, 0.0
+    for side in ("forward", "inverse"):
+        m, ns, first = M, 1, True
+        for r in (8, 4, 2, 5, 3):
+            while m % r == 0:
+                m //= r
+                half = (side == "forward" and first) or (side == "inverse" and m == 1)
+                butterfly = 4 * RADIX_ADDS[r][half] + 10 * RADIX_PRODUCTS[r] + (8 if r == 8 else 0)
+                total += M / r * (butterfly + (0 if first else 30 * (r - 1) * (1 - 1 / ns)))
+                ns, first = ns * r, False
+    return (n + 1) * M * (total + 20.0 * M)
+
+
+def kernel_source_hash(precision: str):
+    """Hash of the sources that fix the conv kernel's memory traffic at n = 256."""
     csrc = os.path.join(ROOT, "paper_1501_04438_gb300", "csrc")
     h = hashlib.sha256()
-    for name in ("gsm_fft.cuh", "gsm_arith.cuh"):
+    for name in ("gsm_conv_rr.cu",) if precision == "fp32" else ("gsm_fx.cuh", "gsm_fx3.cuh", "gsm_fx_passes.cuh"):
         with open(os.path.join(csrc, name), "rb") as f:
             h.update(f.read())
-    src = open(os.path.join(csrc, "gsm_passes.cu")).read()
-    a = src.index("// ------------------------------------------------------------------ pass conv")
-    b = src.index("// ------------------------------------------------------------------ pass yi")
-    h.update(src[a:b].encode())
     return h.hexdigest()[:16]
 
 
@@ -167,7 +186,7 @@ def profiled_traffic(kernel: str, precision: str):
         with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
             t = json.load(f)
         e = t["kernels"][f"{kernel}:{precision}"]
-        if e.get("source_hash", t.get("source_hash")) == kernel_source_hash():
+        if e["source_hash"] == kernel_source_hash(precision):
             return e["dram_bytes_per_launch_full_size"]
     except Exception:
         pass
@@ -320,11 +339,20 @@ def main():
     dom_s = avg_pass[dom] / 1e3
     roof = {"bound": "hbm", "achieved": (alg_bytes or b_app) / dom_s / 1e9, "peak": hbm_peak, "unit": "GB/s"}
     roof["frac"] = roof["achieved"] / roof["peak"]
-    # radix-2 model; FP64 and FP32x2 compute in 64-bit integers, so no floating-point peak applies
-    roof["model_tflops"] = (alg_flops or f_app) / dom_s / 1e12
+    if prec != "fp32" and dom_name == "conv":
+        # 64-bit integers: the pass is bound by its integer instructions (profiles/fixed_point_passes.md),
+        # of which an SM issues 128 lanes a clock
+        prop = torch.cuda.get_device_properties(dev)
+        roof.update(hbm_gbs=roof["achieved"], hbm_frac=roof["frac"], bound="int32 issue",
+                    achieved=conv_pass_int_model(n) / dom_s / 1e12,
+                    peak=128 * prop.multi_processor_count * (clocks["sm_mhz"] or 2070.0) * 1e6 / 1e12,
+                    unit="T instructions/s")
+        roof["frac"] = roof["achieved"] / roof["peak"]
+    roof["model_tflops"] = (alg_flops or f_app) / dom_s / 1e12   # radix-2 model
     roof["traffic"] = profiled_traffic(dom_name, prec)
-    roof["kernel"] = f"k_{dom_name} (pass {dom} of {npass})"
-    roof["peak_source"] = ("measured HBM copy, MEASURED_PEAKS.json" if "hbm_gbs" in peaks else
+    roof["kernel"] = f"{dom_name} (pass {dom} of {npass})"
+    roof["peak_source"] = ("128 lanes per SM and clock at the sampled clock" if roof["bound"] != "hbm" else
+                           "measured HBM copy, MEASURED_PEAKS.json" if "hbm_gbs" in peaks else
                            "fallback HBM figure 6.8 TB/s (no MEASURED_PEAKS.json)")
     # the five passes as built move 12 (instead of 8) half-spectrum slabs
     b_5 = b_app + 4 * cbytes * (n + 1) * n * n
@@ -388,31 +416,24 @@ def main():
             result["parity"] = {"rel_err_vs_oracle": relmax(u_gpu, u_oracle), "tolerance": 1e-12,
                                 "oracle": "taylor_mode 0 (literal Algorithm 1)"}
 
-        # reduced / split precision forms of the same apply
+        # the same apply in single precision (FP32X2 runs the FP64 kernels)
         if not a.no_variants and prec == "fp64":
-            variants = {}
-            for vp in ("fp32x2", "fp32"):
-                vdt = torch.float32 if vp == "fp32" else torch.float64
-                vp_plan = gsm.Plan("coulomb3d", L_BOX, n, precision=vp, stream=stream)
-                vp_plan.autotune(stream=stream)
-                vr = rho.to(vdt)
-                vu = torch.empty_like(vr)
-                time_passes(torch, vp_plan, vr, vu, 2, flush, stream)
-                sm_, pm_ = time_passes(torch, vp_plan, vr, vu, max(3, a.steps), flush, stream)
-                ms = float(np.mean(sm_))
-                uv = vu.double().cpu().numpy()
-                ref = u_oracle if u_oracle is not None else u_gpu
-                vcb = 8 if vp == "fp32" else 16
-                _, vb = apply_model(n, vcb)
-                vb5 = vb + 4 * vcb * (n + 1) * n * n
-                variants[vp] = {"value": n ** 3 / (ms / 1e3) / 1e6, "unit": UNIT, "ms_per_step": ms,
-                                "hbm_frac": vb / (ms / 1e3) / 1e9 / hbm_peak,
-                                "hbm_frac_5pass": vb5 / (ms / 1e3) / 1e9 / hbm_peak,
-                                "rel_err": relmax(uv, ref),
-                                "rel_err_vs": "oracle" if u_oracle is not None else "gpu fp64",
-                                "passes_ms": {PASS_NAMES_3D[p]: float(np.mean(pm_[p])) for p in range(npass)}}
-                vp_plan.destroy()
-            result["variants"] = variants
+            vp_plan = gsm.Plan("coulomb3d", L_BOX, n, precision="fp32", stream=stream)
+            vp_plan.autotune(stream=stream)
+            vr = rho.to(torch.float32)
+            vu = torch.empty_like(vr)
+            time_passes(torch, vp_plan, vr, vu, 2, flush, stream)
+            sm_, pm_ = time_passes(torch, vp_plan, vr, vu, max(3, a.steps), flush, stream)
+            ms = float(np.mean(sm_))
+            _, vb = apply_model(n, 8)
+            vb5 = vb + 4 * 8 * (n + 1) * n * n
+            result["variants"] = {"fp32": {
+                "value": n ** 3 / (ms / 1e3) / 1e6, "unit": UNIT, "ms_per_step": ms,
+                "hbm_frac": vb / (ms / 1e3) / 1e9 / hbm_peak, "hbm_frac_5pass": vb5 / (ms / 1e3) / 1e9 / hbm_peak,
+                "rel_err": relmax(vu.double().cpu().numpy(), u_oracle if u_oracle is not None else u_gpu),
+                "rel_err_vs": "oracle" if u_oracle is not None else "gpu fp64",
+                "passes_ms": {PASS_NAMES_3D[p]: float(np.mean(pm_[p])) for p in range(npass)}}}
+            vp_plan.destroy()
             result["tc_dft32_stage"] = tc_stage_measure(torch, gsm, n, stream, flush)
         print(json.dumps(result), flush=True)
     if world > 1:
@@ -424,9 +445,9 @@ def main():
 def tc_stage_measure(torch, gsm, n, stream, flush):
     """The length-32 DFT stage of the conv pass's forward transforms (a
     padded line of 2n = 512 as 16 x 32: (n + 1) 2n lines, 16 vectors of 32
-    each) three ways: on the tensor cores with FP64-class digit planes
-    (gsm_dft32_tc), and through the FFT engine in FP64 and in FP32x2
-    (gsm_fft_lines).  Errors against the FP64 engine's result."""
+    each) two ways: on the tensor cores with FP64-class digit planes
+    (gsm_dft32_tc), and through the FP64 FFT engine (gsm_fft_lines), against
+    whose result the error is."""
     nvec = (n + 1) * 2 * n * (2 * n // 32)
     torch.manual_seed(7)
     x = torch.complex(torch.randn(nvec, 32, dtype=torch.float64, device=stream.device),
@@ -447,9 +468,7 @@ def tc_stage_measure(torch, gsm, n, stream, flush):
 
     ref, ms64 = timed(lambda: gsm.fft_lines(x, -1, "fp64", stream=stream))
     res = {"fft_engine_fp64": {"ms": ms64}}
-    y2, ms2 = timed(lambda: gsm.fft_lines(x, -1, "fp32x2", stream=stream))
     scale = float(ref.abs().max())
-    res["fft_engine_fp32x2"] = {"ms": ms2, "rel_err_vs_fp64": float((y2 - ref).abs().max()) / scale}
     try:
         yt, mst = timed(lambda: gsm.dft32_tc(x, -1, stream=stream))
         res["tensor_core_digit_planes"] = {"ms": mst, "rel_err_vs_fp64": float((yt - ref).abs().max()) / scale,
@@ -457,7 +476,7 @@ def tc_stage_measure(torch, gsm, n, stream, flush):
     except Exception as exc:                 # reported, not hidden
         res["tensor_core_digit_planes"] = {"error": str(exc)}
     out.update(res)
-    del x, ref, y2
+    del x, ref
     torch.cuda.empty_cache()
     return out
 
@@ -492,8 +511,8 @@ def _cpu_leg(run, points: int, sample: str):
 
 def run_suite_sharded(a, rank: int, world: int, local: int):
     """Config 4 over `world` GPUs: the 48 independent applies split by the LPT
-    rule (partition_batch), each rank applying its share with the grouped
-    launch; no collective on the data path.  Time = max over ranks."""
+    rule (partition_batch), each rank applying its share with one batched
+    call; no collective on the data path.  Time = max over ranks."""
     import torch
     import torch.distributed as dist
 
@@ -635,9 +654,9 @@ def run_suite(a):
                   "sizes": [n for n, _ in specs], "points": npts,
                   "loop": {"ms": ms_loop, "Mpts_s": npts / ms_loop / 1e3},
                   "queue": {"ms": ms_grouped, "Mpts_s": npts / ms_grouped / 1e3, "bitwise_equal_loop": same,
-                            "call": "gsm_apply_batched: one launch with a device work queue, status read back"},
+                            "call": "gsm_apply_batched: queue and grouped launches, status read back"},
                   "graph": {"ms": ms_graph, "Mpts_s": npts / ms_graph / 1e3, "bitwise_equal_loop": same_graph,
-                            "call": "gsm_batch_launch: the queue launch recorded in a CUDA graph"},
+                            "call": "gsm_batch_launch: the same launches recorded in a CUDA graph"},
                   "rel_err_vs_oracle_sampled": errs, "cpu_baseline": cpu, "plans_s": plan_s})
             batch.destroy()
             for p in plans:

@@ -2,7 +2,7 @@
 // FP32X2 passes.
 //
 // GB300 executes 2 FP64 operations per SM and clock against 128 32-bit integer
-// additions and 64 32 x 32 -> 64-bit multiply-adds, so an FFT of doubles is
+// additions and 32 32 x 32 -> 64-bit multiply-adds, so an FFT of doubles is
 // bound by its FP64 pipe alone (95 % busy, everything else idle).  Here a line
 // is a block of 64-bit integers with one common exponent:
 //   value = (re + i im) 2^E,   re, im: signed 64-bit, E one per line.

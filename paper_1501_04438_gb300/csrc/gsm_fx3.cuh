@@ -10,12 +10,11 @@
 // The 64 butterflies of radix R per line are dealt over the group's threads
 // anew, so a thread may hold another line there.
 //
-// Measured against the kernels of any length (FP64): 256^3 passes xf 0.184 ->
-// 0.137, yf 0.344 -> 0.270, conv 1.24 -> 0.84, yi 0.41 -> 0.31, xi 0.23 -> 0.15
-// ms (a third of the instructions there were addresses, tests and loops), apply
-// 2.32 -> 1.66 ms; 192^3 (8 8 6 instead of 8 8 2 3) 1.86 -> 0.96 ms with the
-// energy; 160^3 0.92 -> 0.53 ms; 32^3 45 -> 31 us.  The line is drawn at three
-// stages and 8 values per thread: 64 registers, four CTAs per SM.
+// Measured against the kernels of any length (FP64, white noise, L2 cold, us): 256^3
+// passes xf 190 -> 142, yf 375 -> 282, conv 1363 -> 992, yi 420 -> 309, xi 248 -> 166 (a
+// third of the instructions there are addresses, tests and loops), apply 2590 -> 1884;
+// 192^3 (8 8 6 instead of 8 8 2 3) 1940 -> 953; 160^3 1060 -> 582; 32^3 80 -> 35.  The line
+// is drawn at three stages and 8 values per thread: 64 registers, four CTAs per SM.
 #pragma once
 
 #include "gsm_fx_passes.cuh"
